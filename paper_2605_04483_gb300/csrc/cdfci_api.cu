@@ -878,25 +878,57 @@ CDFCI_API int cdfci_energy_with(cdfci_handle c, const double *h, const double *g
 }  // extern "C"
 
 namespace {
-// c^T H c / c^T c of the handle's stored vector with H from P's integrals: every stored i with
-// c_i != 0 gets (Hc)_i from a fresh column (lookups only), partial sums reduced in a fixed order.
-int exact_rq(cdfci_ctx *c, const Problem &P, double *E) {
-    long long n = c->h_st->n_slots;
-    long long *list = nullptr;
-    double *partial = nullptr, *dE = nullptr;
-    const int nblocks = 152 * 4;
-    if (cudaMalloc(&list, (size_t)std::max<long long>(n, 1) * sizeof(long long)) != cudaSuccess ||
-        cudaMalloc(&partial, (size_t)nblocks * 2 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&dE, sizeof(double)) != cudaSuccess) {
-        cudaFree(list); cudaFree(partial); cudaFree(dE);
-        return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+// Room for the list of the determinants with c != 0, its filters, and `extra` doubles beside them
+// (one allocation, freed by the destructor).  The first guess at their number is the snapshot's
+// count, which a restored checkpoint may have stated wrongly: the callers look at the device's
+// count afterwards and, if it is larger, come back with that.
+struct PairBuffers {
+    void *mem = nullptr;
+    PairList Q{};
+    double *extra = nullptr;
+    ~PairBuffers() { cudaFree(mem); }
+    int make(const Problem &P, long long est, size_t n_extra) {
+        cudaFree(mem);
+        mem = nullptr;
+        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, 0xffffffffll - 1)));
+        unsigned nb1 = 0, nb2 = 0;
+        pair_filters(P, est, &nb1, &nb2);
+        size_t at = 0;
+        auto part = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
+        const size_t ok = part((size_t)est * sizeof(ulonglong2)), oc = part((size_t)est * sizeof(double));
+        const size_t o1 = part(nb1 / 8), o2 = part(nb2 / 8), on = part(sizeof(unsigned)), ox = part(n_extra * sizeof(double));
+        if (cudaMalloc(&mem, at) != cudaSuccess) {
+            mem = nullptr;
+            return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+        }
+        unsigned char *m = static_cast<unsigned char *>(mem);
+        Q.key = reinterpret_cast<ulonglong2 *>(m + ok);
+        Q.c = reinterpret_cast<double *>(m + oc);
+        Q.f1 = reinterpret_cast<unsigned *>(m + o1);
+        Q.f2 = reinterpret_cast<unsigned *>(m + o2);
+        Q.n = reinterpret_cast<unsigned *>(m + on);
+        Q.cap = Q.est = (unsigned)est;
+        Q.nb1 = nb1;
+        Q.mask2 = nb2 - 1;
+        extra = reinterpret_cast<double *>(m + ox);
+        return CDFCI_OK;
     }
-    cudaError_t e = cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), c->stream);
-    if (e == cudaSuccess) e = launch_rq(P, c->d_st, list, n, c->d_counter, partial, nblocks, dE, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(E, dE, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(list); cudaFree(partial); cudaFree(dE);
-    if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "energy: %s", cudaGetErrorString(e));
+};
+
+// c^T H c / c^T c of the handle's stored vector with H from P's integrals.
+int exact_rq(cdfci_ctx *c, const Problem &P, double *E) {
+    PairBuffers pb;
+    const size_t np = 2 * rq_partials(P);
+    unsigned n = (unsigned)std::max<long long>(c->h_st->nnz_c, 1);
+    do {
+        const int rc = pb.make(P, n, np + 1);
+        if (rc) return rc;
+        cudaError_t e = launch_rq(P, c->d_st, pb.Q, pb.extra, pb.extra + np, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(E, pb.extra + np, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "energy: %s", cudaGetErrorString(e));
+    } while (n > pb.Q.cap);
     return fill_stats(c, nullptr);
 }
 }  // namespace
@@ -1604,18 +1636,19 @@ namespace {
 // RDMs into device buffers owned by the caller of this helper (N*N and N^4)
 int rdm_device(cdfci_ctx *c, double *g1, double *g2) {
     const size_t n2 = (size_t)c->P.N * c->P.N, n4 = n2 * n2;
-    double *raw1 = nullptr, *raw2 = nullptr, *nrm = nullptr;
-    if (cudaMalloc(&raw1, n2 * sizeof(double)) != cudaSuccess || cudaMalloc(&raw2, n4 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&nrm, sizeof(double)) != cudaSuccess) {
-        cudaFree(raw1); cudaFree(raw2); cudaFree(nrm);
-        return fail(CDFCI_ERR_NOMEM, "device allocation failed");
-    }
-    cudaError_t e = launch_rdm(c->P, c->d_st, raw1, raw2, nrm, g1, g2, c->stream);
+    PairBuffers pb;
+    unsigned n = (unsigned)std::max<long long>(c->h_st->nnz_c, 1);
     double norm = 0.0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&norm, nrm, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(raw1); cudaFree(raw2); cudaFree(nrm);
-    if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "rdm: %s", cudaGetErrorString(e));
+    do {
+        const int rc = pb.make(c->P, n, n2 + n4 + 1);
+        if (rc) return rc;
+        double *raw1 = pb.extra, *raw2 = raw1 + n2, *nrm = raw2 + n4;
+        cudaError_t e = launch_rdm(c->P, c->d_st, pb.Q, raw1, raw2, nrm, g1, g2, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&norm, nrm, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "rdm: %s", cudaGetErrorString(e));
+    } while (n > pb.Q.cap);
     if (!(norm > 0.0)) return fail(CDFCI_ERR_ARG, "rdm: the stored vector is zero");
     return CDFCI_OK;
 }

@@ -1147,76 +1147,6 @@ __global__ void k_ckpt_restore_m1(Problem P, IterState *st, CdRecord *rec, CdPar
 }
 
 // ---------------------------------------------------------------------------
-// Exact Rayleigh quotient: for every stored i with c_i != 0, (Hc)_i from a
-// fresh column (lookups only); per-CTA partial sums, reduced in fixed order.
-// ---------------------------------------------------------------------------
-__global__ void k_list_nonzero(Problem P, long long *list, long long cap, unsigned long long *counter) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P.capacity;
-         i += (long long)gridDim.x * blockDim.x) {
-        Slot sl = P.table[i];
-        if ((sl.a | sl.b) == 0ull || sl.c == 0.0) continue;
-        unsigned long long pos = atomicAdd(counter, 1ull);
-        if ((long long)pos < cap) list[pos] = i;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_rq_partial(Problem P, IterState *st, const long long *list, long long cap,
-                                                    const unsigned long long *count, double *partial) {
-    __shared__ ColLists L;
-    __shared__ double r[2][8];
-    __shared__ unsigned long long s_a, s_b;
-    __shared__ double s_ci, s_diag;
-    const long long n = (long long)*count < cap ? (long long)*count : cap;
-    const long long nh = P.doubles_vanish ? P.seg[2] : P.seg[5];
-    double num_acc = 0.0, den_acc = 0.0;   // meaningful in thread 0
-    for (long long k = blockIdx.x; k < n; k += gridDim.x) {
-        if (threadIdx.x == 0) {
-            Slot sl = P.table[list[k]];
-            s_a = sl.a; s_b = sl.b & kKeyMaskB; s_ci = sl.c;
-        }
-        __syncthreads();
-        build_lists(L, P.N, s_a, s_b);
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            double d = diag_warp(P, L);
-            if (threadIdx.x == 0) s_diag = d;
-        }
-        double acc = 0.0;
-        for (long long e = 1 + threadIdx.x; e < nh; e += blockDim.x) {
-            unsigned long long oa, ob;
-            double H = column_element(P, L, s_a, s_b, e, oa, ob);
-            if (H == 0.0) continue;
-            bool ins = false;
-            long long s = table_find(P, st, oa, ob, false, &ins);
-            if (s < 0) continue;
-            acc = fma(H, P.table[s].c, acc);
-        }
-        acc = warp_sum(acc);
-        if ((threadIdx.x & 31) == 0) r[0][threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += r[0][w];
-            double hc = fma(s_diag, s_ci, t);
-            num_acc = fma(s_ci, hc, num_acc);
-            den_acc = fma(s_ci, s_ci, den_acc);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = num_acc;
-        partial[2 * blockIdx.x + 1] = den_acc;
-    }
-}
-
-__global__ void k_rq_final(const double *partial, int n, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a = 0.0, b = 0.0;
-    for (int i = 0; i < n; ++i) { a += partial[2 * i]; b += partial[2 * i + 1]; }
-    out[0] = a / b;
-}
-
-// ---------------------------------------------------------------------------
 // Set-up kernels
 // ---------------------------------------------------------------------------
 // Validate finiteness and 8-fold symmetry of g (relative tolerance), then make
@@ -1517,16 +1447,6 @@ cudaError_t launch_ckpt_import(const Problem &P, IterState *st, const unsigned l
 cudaError_t launch_ckpt_restore_m1(const Problem &P, IterState *st, CdRecord *rec, CdPartial *gpart, int G,
                                    const CdRecord &r, const CdPartial &folded, cudaStream_t s) {
     k_ckpt_restore_m1<<<1, 256, 0, s>>>(P, st, rec, gpart, G, r, folded);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_rq(const Problem &P, IterState *st, long long *list, long long cap, unsigned long long *counter,
-                      double *partial, int nblocks, double *out, cudaStream_t s) {
-    long long grid = (P.capacity + 255) / 256;
-    if (grid > 152 * 16) grid = 152 * 16;
-    k_list_nonzero<<<(int)grid, 256, 0, s>>>(P, list, cap, counter);
-    k_rq_partial<<<nblocks, 256, 0, s>>>(P, st, list, cap, counter, partial);
-    k_rq_final<<<1, 32, 0, s>>>(partial, nblocks, out);
     return cudaGetLastError();
 }
 

@@ -16,8 +16,6 @@ cudaError_t launch_column(const Problem &P, unsigned long long A, unsigned long 
                           double *vals, long long cap, unsigned long long *counter, cudaStream_t s);
 cudaError_t launch_export(const Problem &P, const IterState *st, unsigned long long *keys, double *c, double *b,
                           long long cap, unsigned long long *counter, cudaStream_t s);
-cudaError_t launch_rq(const Problem &P, IterState *st, long long *list, long long cap, unsigned long long *counter,
-                      double *partial, int nblocks, double *out, cudaStream_t s);
 cudaError_t launch_setup(double *h, double *g, int N, double *J, double *K, double *W3, double *V3, int *status,
                          int *has_doubles, int sym4, cudaStream_t s);
 cudaError_t launch_init_state(IterState *st, CdRecord *rec, unsigned long long A, unsigned long long B, double eta,
@@ -127,8 +125,22 @@ cudaError_t launch_cd_loop_batch(const CdInstance *inst, int n_inst, int cluster
 cudaError_t launch_cd_finalize_batch(const CdInstance *inst, int n_inst, int cluster, cudaStream_t s);
 
 // reduced density matrices and the energy's derivatives (cdfci_rdm.cu)
-cudaError_t launch_rdm(const Problem &P, IterState *st, double *g1_raw, double *g2_raw, double *norm, double *g1,
-                       double *g2, cudaStream_t s);
+// The determinants with c != 0 (key and c, in no particular order) and the bit
+// filters over them; `est` is their expected number, `cap` the list's length
+// (n > cap after the listing: list again with room for n).
+struct PairList {
+    ulonglong2 *key;
+    double *c;
+    unsigned *n, cap, est;
+    unsigned *f1, nb1;                 // filter 1: nb1 bits (0: not used)
+    unsigned *f2, mask2;               // filter 2: mask2 + 1 bits
+};
+void pair_filters(const Problem &P, long long est, unsigned *nb1, unsigned *nb2);
+size_t rq_partials(const Problem &P);   // pairs of doubles that launch_rq needs
+cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, double *g1_raw, double *g2_raw,
+                       double *norm, double *g1, double *g2, cudaStream_t s);
+// c^T H c / c^T c with H from P's integrals
+cudaError_t launch_rq(const Problem &P, IterState *st, const PairList &Q, double *partial, double *out, cudaStream_t s);
 cudaError_t launch_gradient(int N, const double *h, const double *g, const double *G1, const double *G2, double *F,
                             double *dh, double *dg, double *dk, cudaStream_t s);
 
