@@ -890,26 +890,23 @@ struct PairBuffers {
     int make(const Problem &P, long long est, size_t n_extra) {
         cudaFree(mem);
         mem = nullptr;
-        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, 0xffffffffll - 1)));
-        unsigned nb1 = 0, nb2 = 0;
-        pair_filters(P, est, &nb1, &nb2);
+        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, 1ll << 29)));
+        pair_sizes(P, est, &Q);
         size_t at = 0;
         auto part = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
-        const size_t ok = part((size_t)est * sizeof(ulonglong2)), oc = part((size_t)est * sizeof(double));
-        const size_t o1 = part(nb1 / 8), o2 = part(nb2 / 8), on = part(sizeof(unsigned)), ox = part(n_extra * sizeof(double));
+        const size_t orec = part(((size_t)Q.imask + 1) * sizeof(PairRec)), op = part((size_t)est * sizeof(unsigned));
+        const size_t o1 = part(Q.nb1 / 8), o2 = part(((size_t)Q.mask2 + 1) / 8), on = part(sizeof(unsigned));
+        const size_t ox = part(n_extra * sizeof(double));
         if (cudaMalloc(&mem, at) != cudaSuccess) {
             mem = nullptr;
             return fail(CDFCI_ERR_NOMEM, "device allocation failed");
         }
         unsigned char *m = static_cast<unsigned char *>(mem);
-        Q.key = reinterpret_cast<ulonglong2 *>(m + ok);
-        Q.c = reinterpret_cast<double *>(m + oc);
+        Q.rec = reinterpret_cast<PairRec *>(m + orec);
+        Q.pos = reinterpret_cast<unsigned *>(m + op);
         Q.f1 = reinterpret_cast<unsigned *>(m + o1);
         Q.f2 = reinterpret_cast<unsigned *>(m + o2);
         Q.n = reinterpret_cast<unsigned *>(m + on);
-        Q.cap = Q.est = (unsigned)est;
-        Q.nb1 = nb1;
-        Q.mask2 = nb2 - 1;
         extra = reinterpret_cast<double *>(m + ox);
         return CDFCI_OK;
     }

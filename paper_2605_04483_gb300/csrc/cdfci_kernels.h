@@ -125,17 +125,24 @@ cudaError_t launch_cd_loop_batch(const CdInstance *inst, int n_inst, int cluster
 cudaError_t launch_cd_finalize_batch(const CdInstance *inst, int n_inst, int cluster, cudaStream_t s);
 
 // reduced density matrices and the energy's derivatives (cdfci_rdm.cu)
-// The determinants with c != 0 (key and c, in no particular order) and the bit
-// filters over them; `est` is their expected number, `cap` the list's length
-// (n > cap after the listing: list again with room for n).
-struct PairList {
-    ulonglong2 *key;
-    double *c;
-    unsigned *n, cap, est;
-    unsigned *f1, nb1;                 // filter 1: nb1 bits (0: not used)
-    unsigned *f2, mask2;               // filter 2: mask2 + 1 bits
+// The determinants with c != 0: a table of records (at most half full), the
+// positions of the occupied ones (in no particular order) and bit filters;
+// `est` is their expected number, `cap` the most that are taken (n > cap after
+// the listing: list again with room for n).
+struct __align__(32) PairRec {
+    unsigned long long a, b;
+    double c;
+    unsigned long long tag;            // 0: free
 };
-void pair_filters(const Problem &P, long long est, unsigned *nb1, unsigned *nb2);
+struct PairList {
+    PairRec *rec;                      // imask + 1 records
+    unsigned *pos;
+    unsigned *n, cap, est;
+    unsigned imask;
+    unsigned *f1, nb1;                 // filter 1: nb1 bits (0: not used)
+    unsigned *f2, mask2;               // filter 2: mask2 + 1 bits (where filter 1 is not used)
+};
+void pair_sizes(const Problem &P, long long est, PairList *Q);   // everything but the pointers
 size_t rq_partials(const Problem &P);   // pairs of doubles that launch_rq needs
 cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, double *g1_raw, double *g2_raw,
                        double *norm, double *g1, double *g2, cudaStream_t s);

@@ -37,17 +37,19 @@ namespace {
 __device__ __forceinline__ int occ_orbital(const ColLists &L, int na, int t) { return t < na ? L.occA[t] : L.occB[t - na]; }
 
 // ---------------------------------------------------------------------------
-// The list of the determinants with c != 0 and two bit filters over them.
+// The determinants with c != 0 in a hash table of their own, and a bit filter.
 //
-// Almost every excitation of a stored determinant is absent or has c = 0, and
-// a probe that misses reads more than two random slots at a usual load, so what
-// bounds the sums is how fast a miss is seen.  The filters are indexed by an
-// exclusive-or hash, one 64-bit word per spin-orbital: the hash of an excited
-// determinant is that of J with two or four words exchanged, so testing an
-// element costs a handful of integer instructions and one bit.  Its low half
-// indexes filter 1, which each SM keeps in shared memory; its high half filter
-// 2, in L2, larger, asked by the survivors of filter 1 (or by every element
-// when the list is too long for filter 1).
+// Most excitations of a stored determinant are absent or have c = 0, and in the
+// solver's table a probe that misses reads more than two random slots at a usual
+// load, a warp of 32 probes as many as its unluckiest lane.  So the sums copy the
+// nonzeros into a table at most half full (records {A, B, c}, one 32-byte request
+// a probe) and test a bit before asking it.  Both go by an exclusive-or hash z,
+// one 64-bit word per spin-orbital: z of an excited determinant is that of J
+// with two or four words exchanged, so testing an element costs a handful of
+// integer instructions.
+//   filter 1 (low half of z): in each SM's shared memory;
+//   the table (high half): open addressing;
+//   filter 2 (high half): in L2, for more determinants than filter 1 can tell.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long orb_word(int t) {      // t: alpha p, 64 + beta p
     return mix64(0x632be59bd9b4e019ull + (unsigned long long)(t + 1) * 0x9e3779b97f4a7c15ull);
@@ -62,7 +64,15 @@ __device__ __forceinline__ void ld_slot_cg(const Slot *s, unsigned long long &a,
     c = __longlong_as_double((long long)cb);
 }
 
-__global__ void __launch_bounds__(256) k_pair_list(Problem P, PairList L) {
+// a record {A, B, c}, in one 32-byte request
+__device__ __forceinline__ void ld_rec(const PairRec *r, unsigned long long &a, unsigned long long &b, double &c) {
+    unsigned long long cb;
+    [[maybe_unused]] unsigned long long pad;
+    asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(cb), "=l"(pad) : "l"(r));
+    c = __longlong_as_double((long long)cb);
+}
+
+__global__ void __launch_bounds__(256) k_pair_list(Problem P, IterState *st, PairList L) {
     __shared__ unsigned long long s_z[128];
     if (threadIdx.x < 128) s_z[threadIdx.x] = orb_word(threadIdx.x);
     __syncthreads();
@@ -83,8 +93,6 @@ __global__ void __launch_bounds__(256) k_pair_list(Problem P, PairList L) {
         if (!on) continue;
         const unsigned pos = base + __popc(m & ((1u << lane) - 1u));
         if (pos >= L.cap) continue;                     // the caller sees n > cap and lists again
-        L.key[pos] = make_ulonglong2(a, b);
-        L.c[pos] = c;
         unsigned long long z = 0ull;
         for (unsigned long long x = a; x; x &= x - 1) z ^= s_z[__ffsll((long long)x) - 1];
         for (unsigned long long x = b; x; x &= x - 1) z ^= s_z[64 + __ffsll((long long)x) - 1];
@@ -92,8 +100,22 @@ __global__ void __launch_bounds__(256) k_pair_list(Problem P, PairList L) {
             const unsigned k = f1_index(z, L.nb1);
             atomicOr(L.f1 + (k >> 5), 1u << (k & 31));
         }
-        const unsigned k2 = f2_index(z, L.mask2);
-        atomicOr(L.f2 + (k2 >> 5), 1u << (k2 & 31));
+        if (!L.nb1) {
+            const unsigned k2 = f2_index(z, L.mask2);
+            atomicOr(L.f2 + (k2 >> 5), 1u << (k2 & 31));
+        }
+        unsigned at = (unsigned)(z >> 32) & L.imask, probe = 0;
+        for (; probe <= L.imask; ++probe) {
+            if (atomicCAS(&L.rec[at].tag, 0ull, 1ull) == 0ull) break;   // claimed: read by later launches only
+            at = (at + 1) & L.imask;
+        }
+        if (probe <= L.imask) {
+            L.rec[at].a = a;
+            L.rec[at].b = b;
+            L.rec[at].c = c;
+            L.pos[pos] = at;
+        }
+        if (probe > L.imask) set_status(st, kErrInternal);
     }
 }
 
@@ -189,7 +211,7 @@ __host__ __device__ __forceinline__ size_t pair_warp_bytes(int nsA, int nsB) {
 // a time, every lane its own element.  kF1: filter 1 (shared memory) is tested
 // in the loop and filter 2 (L2) in the lookup; else filter 2 in the loop.
 template <class Sink, bool kF1>
-__global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, IterState *st, PairList Q, Sink sink, int singles_only) {
+__global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink sink, int singles_only) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     unsigned *s_f = reinterpret_cast<unsigned *>(s_raw);
     const unsigned nw1 = kF1 ? Q.nb1 / 32 : 0;
@@ -214,9 +236,9 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, IterState *st, Pai
         return ((w >> (k & 31)) & 1u) != 0u;
     };
     for (unsigned at = blockIdx.x * nwarps + warp; at < n; at += gridDim.x * nwarps) {
-        const ulonglong2 key = Q.key[at];
-        const unsigned long long A = key.x, B = key.y;
-        const double cJ = Q.c[at];
+        const PairRec J = Q.rec[Q.pos[at]];
+        const unsigned long long A = J.a, B = J.b;
+        const double cJ = J.c;
         unsigned long long zJ = 0ull;
         for (int t = lane; t < N; t += 32) {
             const int ra = __popcll(A & low_mask(t)), rb = __popcll(B & low_mask(t));
@@ -361,24 +383,15 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, IterState *st, Pai
                             if (x.kind == 1) { x.i = j; x.a = b; } else { x.j = j; x.b = b; }
                         }
                     }
-                    bool look = true;
-                    if (kF1) {
-                        const unsigned k2 = f2_index(z, Q.mask2);
-                        look = (__ldg(Q.f2 + (k2 >> 5)) >> (k2 & 31)) & 1u;
-                    }
+                    unsigned pos = (unsigned)(z >> 32) & Q.imask;
                     double cI = 0.0;
-                    if (look) {
-                        unsigned long long pos = key_hash(oa, ob) & P.mask;
-                        int probe = 0;
-                        for (; probe < P.max_probe; ++probe) {
-                            unsigned long long ka, kb;
-                            double c;
-                            ld_slot_cg(P.table + pos, ka, kb, c);
-                            if (ka == oa && (kb & kKeyMaskB) == ob) { cI = c; break; }
-                            if ((ka | kb) == 0ull) break;
-                            pos = (pos + 1) & P.mask;
-                        }
-                        if (probe == P.max_probe) set_status(st, kErrTableFull);
+                    for (unsigned probe = 0; probe <= Q.imask; ++probe) {
+                        unsigned long long ka, kb;
+                        double c;
+                        ld_rec(Q.rec + pos, ka, kb, c);
+                        if (ka == oa && kb == ob) { cI = c; break; }
+                        if ((ka | kb) == 0ull) break;
+                        pos = (pos + 1) & Q.imask;
                     }
                     if (!is_zero(cI)) sink.hit(P, L, x, cJ, cI);
                 }
@@ -393,58 +406,63 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, IterState *st, Pai
 
 // The number-operator terms: S_PQ = sum_J c_J^2 n_P n_Q over the pairs P <= Q
 // of spin-orbitals (alpha p, then beta p), which give gamma_pp, Gamma_pprr and
-// Gamma_prrp, and c.c.  A warp takes kDiagT pairs per lane (its tile of pairs)
-// over a share of the list, the key and c^2 uniform over the warp; sums stay in
-// registers until the end (a lane's running sums are independent, so the FP64
-// latency of one is hidden behind the others).
-constexpr int kDiagT = 8;
+// Gamma_prrp, and c.c.  A warp adds the occupied pairs of its determinants to an
+// array of its own in shared memory: one lane per pair, so no two lanes of a
+// determinant meet, and the FP64 pipe (two lanes a cycle here) sees only the
+// pairs that are occupied (testing every pair of spin-orbitals in registers took
+// 540 us for 300 k determinants of 10 electrons in 32 spin-orbitals).
+__host__ __device__ __forceinline__ size_t diag_warp_bytes(int N) { return ((size_t)N * (2 * N + 1) + 16) * sizeof(double); }
 __global__ void __launch_bounds__(256) k_rdm_diag(Problem P, PairList Q, double *g1, double *g2, double *norm) {
-    const int N = P.N, NS = 2 * N, lane = threadIdx.x & 31;
-    const int npairs = NS * (NS + 1) / 2;
-    unsigned long long mA[kDiagT], mB[kDiagT];
-    short pp[kDiagT], qq[kDiagT];
-    double s[kDiagT];
-#pragma unroll
-    for (int k = 0; k < kDiagT; ++k) {
-        const int t = (int)blockIdx.y * (32 * kDiagT) + 32 * k + lane;
-        int q = 0, p = 0;
-        if (t < npairs) {                               // t = q (q + 1) / 2 + p, p <= q
-            q = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-            while (q * (q + 1) / 2 > t) --q;
-            while ((q + 1) * (q + 2) / 2 <= t) ++q;
-            p = t - q * (q + 1) / 2;
-        }
-        const unsigned long long bp = 1ull << (p < N ? p : p - N), bq = 1ull << (q < N ? q : q - N);
-        mA[k] = (p < N ? bp : 0ull) | (q < N ? bq : 0ull);
-        mB[k] = (p < N ? 0ull : bp) | (q < N ? 0ull : bq);
-        pp[k] = (short)(t < npairs ? p : -1);
-        qq[k] = (short)q;
-        s[k] = 0.0;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const int N = P.N, NS = 2 * N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int npairs = NS * (NS + 1) / 2, ne = P.na + P.nb, nep = ne * (ne + 1) / 2;
+    double *s = reinterpret_cast<double *>(s_raw + (size_t)warp * diag_warp_bytes(N));
+    unsigned char *occ = reinterpret_cast<unsigned char *>(s + npairs);            // 128 bytes
+    unsigned short *uv = reinterpret_cast<unsigned short *>(s_raw + (size_t)nwarps * diag_warp_bytes(N));
+    for (int t = threadIdx.x; t < nep; t += blockDim.x) {                          // pairs u <= v of occupied positions
+        int v = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while (v * (v + 1) / 2 > t) --v;
+        while ((v + 1) * (v + 2) / 2 <= t) ++v;
+        uv[t] = (unsigned short)((t - v * (v + 1) / 2) | v << 8);
     }
+    for (int t = lane; t < npairs; t += 32) s[t] = 0.0;
+    __syncthreads();
     double nrm = 0.0;
     const unsigned n = min(*Q.n, Q.cap);
-    const unsigned w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = gridDim.x * (blockDim.x >> 5);
-    for (unsigned at = w0; at < n; at += nw) {
-        const ulonglong2 key = Q.key[at];
-        const double c = Q.c[at], c2 = c * c;
-        nrm = fma(c, c, nrm);
-#pragma unroll
-        for (int k = 0; k < kDiagT; ++k)
-            if ((key.x & mA[k]) == mA[k] && (key.y & mB[k]) == mB[k]) s[k] += c2;
+    for (unsigned at = blockIdx.x * nwarps + warp; at < n; at += gridDim.x * nwarps) {
+        const PairRec key = Q.rec[Q.pos[at]];
+        const double c2 = key.c * key.c;
+        nrm += c2;
+        for (int t = lane; t < N; t += 32) {
+            if ((key.a >> t) & 1ull) occ[__popcll(key.a & low_mask(t))] = (unsigned char)t;
+            if ((key.b >> t) & 1ull) occ[P.na + __popcll(key.b & low_mask(t))] = (unsigned char)(N + t);
+        }
+        __syncwarp();
+        for (int t = lane; t < nep; t += 32) {
+            const int p = occ[uv[t] & 0xff], q = occ[uv[t] >> 8];                  // p <= q
+            s[q * (q + 1) / 2 + p] += c2;
+        }
+        __syncwarp();
     }
-    if (blockIdx.y == 0 && lane == 0 && nrm != 0.0) atomicAdd(norm, nrm);
-#pragma unroll
-    for (int k = 0; k < kDiagT; ++k) {
-        const int P0 = pp[k], Q0 = qq[k];
-        if (P0 < 0 || s[k] == 0.0) continue;
+    if (lane == 0 && nrm != 0.0) atomicAdd(norm, nrm);
+    // the block's sums, each pair once
+    __syncthreads();
+    for (int t = threadIdx.x; t < npairs; t += blockDim.x) {
+        double v = 0.0;
+        for (int w = 0; w < nwarps; ++w) v += reinterpret_cast<const double *>(s_raw + (size_t)w * diag_warp_bytes(N))[t];
+        if (v == 0.0) continue;
+        int Q0 = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while (Q0 * (Q0 + 1) / 2 > t) --Q0;
+        while ((Q0 + 1) * (Q0 + 2) / 2 <= t) ++Q0;
+        const int P0 = t - Q0 * (Q0 + 1) / 2;
         const int p = P0 < N ? P0 : P0 - N, r = Q0 < N ? Q0 : Q0 - N;
         if (P0 == Q0) {
-            atomicAdd(&g1[p * N + p], s[k]);
+            atomicAdd(&g1[p * N + p], v);
             continue;
         }
         // both orders of the pair: (pp|rr) and (rr|pp), for one spin also the exchange
-        atomicAdd(&g2[(size_t)(p * N + p) * N * N + r * N + r], 2.0 * s[k]);
-        if ((P0 < N) == (Q0 < N)) atomicAdd(&g2[(size_t)(p * N + r) * N * N + r * N + p], -2.0 * s[k]);
+        atomicAdd(&g2[(size_t)(p * N + p) * N * N + r * N + r], 2.0 * v);
+        if ((P0 < N) == (Q0 < N)) atomicAdd(&g2[(size_t)(p * N + r) * N * N + r * N + p], -2.0 * v);
     }
 }
 
@@ -558,40 +576,45 @@ static PairShape pair_shape(const Problem &P, const PairList &Q) {
     return s;
 }
 
-// Filter sizes for about `est` determinants.  Filter 1 takes 32 bits a
-// determinant up to what shared memory leaves; below one bit a determinant
-// (two of three elements would pass) it is not used.  Filter 2: 32 bits a
-// determinant, 2^15 to 2^28 bits.
-void pair_filters(const Problem &P, long long est, unsigned *nb1, unsigned *nb2) {
+// Sizes for about `est` determinants.  Filter 1 takes 32 bits a determinant up
+// to what shared memory leaves; below one bit a determinant (two of three
+// elements would pass) filter 2 takes its place, with 32 bits a determinant, at
+// most 2^28.  The table has at least 2 records a determinant.
+void pair_sizes(const Problem &P, long long est, PairList *Q) {
     const size_t used = 128 * sizeof(unsigned long long) + (size_t)pair_warps(P) * pair_warp_bytes(P.na * P.va, P.nb * P.vb);
     const long long room = used + 4096 < kPairSmem ? (long long)(kPairSmem - used - 16) / 128 * 1024 : 0;
     const long long want = std::max<long long>(1024, (32 * est + 1023) / 1024 * 1024);
     const long long b1 = std::min(want, room);
-    *nb1 = b1 >= est ? (unsigned)b1 : 0u;
+    Q->nb1 = b1 >= est ? (unsigned)b1 : 0u;
     unsigned long long b2 = 1ull << 15;
     while (b2 < 32ull * (unsigned long long)est && b2 < (1ull << 28)) b2 <<= 1;
-    *nb2 = (unsigned)b2;
+    Q->mask2 = Q->nb1 ? 31u : (unsigned)(b2 - 1);
+    unsigned long long ni = 1024;
+    while (ni < 2ull * (unsigned long long)est) ni <<= 1;
+    Q->imask = (unsigned)(ni - 1);
+    Q->cap = Q->est = (unsigned)est;
 }
 
-cudaError_t launch_pair_list(const Problem &P, const PairList &Q, cudaStream_t s) {
+static cudaError_t launch_pair_list(const Problem &P, IterState *st, const PairList &Q, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(Q.n, 0, sizeof(unsigned), s);
     if (e == cudaSuccess && Q.nb1) e = cudaMemsetAsync(Q.f1, 0, Q.nb1 / 8, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(Q.f2, 0, ((size_t)Q.mask2 + 1) / 8, s);
+    if (e == cudaSuccess && !Q.nb1) e = cudaMemsetAsync(Q.f2, 0, ((size_t)Q.mask2 + 1) / 8, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(Q.rec, 0, ((size_t)Q.imask + 1) * sizeof(PairRec), s);
     if (e != cudaSuccess) return e;
     long long grid = (P.capacity + 255) / 256;
     if (grid > 152 * 8) grid = 152 * 8;
-    k_pair_list<<<(unsigned)grid, 256, 0, s>>>(P, Q);
+    k_pair_list<<<(unsigned)grid, 256, 0, s>>>(P, st, Q);
     return cudaGetLastError();
 }
 
 template <class Sink>
-static cudaError_t launch_pairs(const Problem &P, IterState *st, const PairList &Q, const Sink &sink, int singles_only,
+static cudaError_t launch_pairs(const Problem &P, const PairList &Q, const Sink &sink, int singles_only,
                                 cudaStream_t s) {
     const PairShape g = pair_shape(P, Q);
     auto kernel = Q.nb1 ? k_pairs<Sink, true> : k_pairs<Sink, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
     if (e != cudaSuccess) return e;
-    kernel<<<g.blocks, 32 * g.warps, g.smem, s>>>(P, st, Q, sink, singles_only);
+    kernel<<<g.blocks, 32 * g.warps, g.smem, s>>>(P, Q, sink, singles_only);
     return cudaGetLastError();
 }
 
@@ -602,13 +625,16 @@ cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, doubl
     cudaError_t e = cudaMemsetAsync(g1_raw, 0, n2 * sizeof(double), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(g2_raw, 0, n4 * sizeof(double), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(norm, 0, sizeof(double), s);
-    if (e == cudaSuccess) e = launch_pair_list(P, Q, s);
-    if (e == cudaSuccess) e = launch_pairs(P, st, Q, RdmSink{g1_raw, g2_raw}, 0, s);
+    if (e == cudaSuccess) e = launch_pair_list(P, st, Q, s);
+    if (e == cudaSuccess) e = launch_pairs(P, Q, RdmSink{g1_raw, g2_raw}, 0, s);
     if (e != cudaSuccess) return e;
-    const int tiles = (N * (2 * N + 1) + 32 * kDiagT - 1) / (32 * kDiagT);
-    const long long blocks = std::max<long long>(1, std::min<long long>(std::max(1, 152 * 4 / tiles),
-                                                                        ((long long)Q.est + 63) / 64));
-    k_rdm_diag<<<dim3((unsigned)blocks, (unsigned)tiles), 256, 0, s>>>(P, Q, g1_raw, g2_raw, norm);
+    int dw = 8;                                         // warps a block: their arrays within 100 KB (200 KB for one)
+    while (dw > 1 && dw * diag_warp_bytes(N) > 100 * 1024) --dw;
+    const size_t dsm = dw * diag_warp_bytes(N) + (size_t)(P.na + P.nb) * (P.na + P.nb + 1);
+    e = cudaFuncSetAttribute(k_rdm_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e != cudaSuccess) return e;
+    const long long dblocks = std::max<long long>(1, std::min<long long>(152 * 2, ((long long)Q.est + 8 * dw - 1) / (8 * dw)));
+    k_rdm_diag<<<(unsigned)dblocks, 32 * dw, dsm, s>>>(P, Q, g1_raw, g2_raw, norm);
     k_rdm_finalize<<<152 * 4, 256, 0, s>>>(N, g1_raw, g2_raw, norm, g1, g2);
     return cudaGetLastError();
 }
@@ -616,8 +642,8 @@ cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, doubl
 size_t rq_partials(const Problem &P) { return 152 * (size_t)pair_warps(P); }
 
 cudaError_t launch_rq(const Problem &P, IterState *st, const PairList &Q, double *partial, double *out, cudaStream_t s) {
-    cudaError_t e = launch_pair_list(P, Q, s);
-    if (e == cudaSuccess) e = launch_pairs(P, st, Q, QuotientSink{partial, 0.0, 0.0}, P.doubles_vanish, s);
+    cudaError_t e = launch_pair_list(P, st, Q, s);
+    if (e == cudaSuccess) e = launch_pairs(P, Q, QuotientSink{partial, 0.0, 0.0}, P.doubles_vanish, s);
     if (e != cudaSuccess) return e;
     const PairShape g = pair_shape(P, Q);
     k_rq_final<<<1, 1024, 0, s>>>(partial, g.blocks * g.warps, out);
