@@ -680,11 +680,8 @@ __device__ void mc_ties(const Problem &P, McState *ms, const long long *cand, co
     __syncthreads();
 }
 
-// Bitonic sort, in shared memory, of (choice key, index) pairs into the choice
-// order: |g| descending, then the determinant key ascending (looked up in src
-// for exact ties only).  Padding entries (index -1) sort last.
-// One element of a sort, held in registers: the choice key and the determinant
-// (a strict total order: keys are unique); padding sorts last.
+// One element of a sort: the choice key and the determinant (a strict total
+// order: keys are unique).
 struct SelE {
     unsigned long long g, A, B;
     long long slot;
@@ -693,46 +690,48 @@ __device__ __forceinline__ bool sel_first(const SelE &x, const SelE &y) {   // x
     if (x.g != y.g) return x.g > y.g;
     return key_less(x.A, x.B, y.A, y.B);
 }
-__device__ __forceinline__ SelE sel_pad() { return SelE{0ull, ~0ull, ~0ull, -1}; }
-// Bitonic sort into the choice order of n_pow2 elements, one per thread (thread
-// t holds element t; n_pow2 a power of two).  Only the first max(n_pow2, 32)
-// threads take part (the caller's other threads skip it): a stage whose
-// partners lie in one warp (distance < 32) exchanges by shuffles, the others
-// through buf between two barriers of the taking-part warps (named barrier 1).
-__device__ void bitonic_reg(SelE &e, int n_pow2, SelE *buf) {
-    const int t = threadIdx.x;
-    const int nact = n_pow2 < 32 ? 32 : n_pow2;
-    for (int k = 2; k <= n_pow2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            SelE o;
-            if (j >= 32) {                              // uniform
-                buf[t] = e;
-                asm volatile("bar.sync 1, %0;" ::"r"(nact) : "memory");
-                o = buf[t ^ j];
-                asm volatile("bar.sync 1, %0;" ::"r"(nact) : "memory");
-            } else {
-                o.g = __shfl_xor_sync(0xffffffffu, e.g, j);
-                o.A = __shfl_xor_sync(0xffffffffu, e.A, j);
-                o.B = __shfl_xor_sync(0xffffffffu, e.B, j);
-                o.slot = __shfl_xor_sync(0xffffffffu, e.slot, j);
-            }
-            // the lower position of an ascending pair (and the upper of a descending one) keeps the
-            // first of the two
-            const bool keep_first = ((t & j) == 0) == ((t & k) == 0);
-            const bool o_first = sel_first(o, e), e_first = sel_first(e, o);
-            if (keep_first ? o_first : e_first) e = o;
+
+// Place of each of n <= 1024 elements in the choice order, by counting the
+// elements before it: the 1024 threads form 2^k groups per element (n x 2^k
+// threads at most 1024), each counting over a share of the list in shared
+// memory, 8 bytes per comparison, the determinants only where two choice keys
+// are equal.  Every comparison is independent and one barrier separates the
+// stages, where a bitonic network passes through up to 55 dependent exchanges:
+// the whole kernel at m = 256 on a 4 x 4 lattice 19.5 -> 9.0 us, at m = 64 12.0 -> 3.6 us.
+// buf holds the elements, rank (zeroed here) receives the places; block-wide.
+__device__ void rank_sort(const SelE *buf, int n, unsigned int *rank) {
+    const int tid = threadIdx.x;
+    if (tid < n) rank[tid] = 0u;
+    __syncthreads();
+    int per = 32;                                       // elements per group of threads: a multiple of a warp
+    while (per < n) per <<= 1;
+    const int parts = 1024 / per, part = tid / per, i = tid - part * per;
+    if (i < n) {
+        const int span = (n + parts - 1) / parts, j0 = part * span, j1 = min(n, j0 + span);
+        const unsigned long long g = buf[i].g;
+        unsigned int before = 0;
+        for (int j = j0; j < j1; ++j) {                 // the same j in every lane: broadcast reads
+            const unsigned long long h = buf[j].g;
+            before += h > g ? 1u : 0u;
+            if (h == g && j != i && sel_first(buf[j], buf[i])) ++before;
         }
+        if (before) atomicAdd(&rank[i], before);
     }
+    __syncthreads();
 }
 
-// The in-bin candidates sorted (after the exact-tie pass when more than kInBin
-// share the whole 64-bit choice key), the first sel_need of them join the
+// The in-bin candidates put in order (after the exact-tie pass when more than
+// kInBin share the whole 64-bit choice key), the first sel_need of them join the
 // chosen set; then the chosen set in the choice order (a canonical order for
-// the reduced problem's rows).  1024 threads, one element each.
+// the reduced problem's rows).  The candidates above the threshold digit all
+// precede the in-bin ones, so each of the two sets is ordered by itself.
+// 1024 threads, one element each.
 __global__ void __launch_bounds__(1024) k_mc_sortsel(Problem P, McState *ms, McSel *sel, McSel *inbin, int m,
                                                       IterState *st, const long long *cand,
                                                       const unsigned long long *gkey, McSel *ties) {
     __shared__ SelE buf[kInBin];
+    __shared__ unsigned int rank[kInBin];
+    __shared__ int s_keep, s_digit;
     const int tid = threadIdx.x;
     if (ms->done) return;
     if (ms->sel_level >= kSelLevels && ms->n_inbin > kInBin) mc_ties(P, ms, cand, gkey, ties, inbin);   // uniform
@@ -744,26 +743,55 @@ __global__ void __launch_bounds__(1024) k_mc_sortsel(Problem P, McState *ms, McS
     }
     const int need = ms->sel_level == 0 ? 0 : ms->sel_need;
     const int take = need < n_in ? need : n_in;
+    SelE e{0ull, 0ull, 0ull, -1}, f = e;
+    if (tid < n_above) { const McSel x = sel[tid]; e = SelE{x.gkey, x.A, x.B, x.slot}; }
+    if (take > 0 && tid < n_in) { const McSel x = inbin[tid]; f = SelE{x.gkey, x.A, x.B, x.slot}; }
+    if (tid < n_above) buf[tid] = e;
+    rank_sort(buf, n_above, rank);
+    if (tid < n_above) sel[rank[tid]] = McSel{e.slot, e.g, e.A, e.B};
     if (take > 0) {                                     // uniform
-        int p2 = 1;
-        while (p2 < n_in) p2 <<= 1;
-        SelE e = sel_pad();
-        if (tid < n_in) { const McSel x = inbin[tid]; e = SelE{x.gkey, x.A, x.B, x.slot}; }
-        if (n_in > 1 && tid < (p2 < 32 ? 32 : p2)) bitonic_reg(e, p2, buf);
-        if (tid < take) sel[n_above + tid] = McSel{e.slot, e.g, e.A, e.B};
-        __syncthreads();                                // sel visible to the block
-    }
-    const int msel = n_above + take;
-    if (msel > 1) {
-        int q2 = 1;
-        while (q2 < msel) q2 <<= 1;
-        SelE e = sel_pad();
-        if (tid < msel) { const McSel x = sel[tid]; e = SelE{x.gkey, x.A, x.B, x.slot}; }
-        if (tid < (q2 < 32 ? 32 : q2)) bitonic_reg(e, q2, buf);
-        if (tid < msel) sel[tid] = McSel{e.slot, e.g, e.A, e.B};
+        __syncthreads();                                // rank read
+        // many more than are needed: one 8-bit digit below the selection's prefix first, so that only the
+        // ones at or above the digit of rank `take` are ordered
+        bool keep = tid < n_in;
+        const int low = 64 - sel_cover(ms->sel_level);  // bits the prefix leaves open
+        if (n_in > take + 64 && low >= 8) {             // uniform
+            const unsigned int dg = (unsigned int)(f.g >> (low - 8)) & 0xffu;
+            if (tid < 256) rank[tid] = 0u;
+            if (tid == 0) s_keep = 0;
+            __syncthreads();
+            if (keep) atomicAdd(&rank[dg], 1u);
+            __syncthreads();
+            if (tid < 32) {                             // lane l: digits 255 - 8 l down to 248 - 8 l
+                unsigned int loc = 0;
+                for (int q = 0; q < 8; ++q) loc += rank[255 - 8 * tid - q];
+                unsigned int inc = loc;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const unsigned int v = __shfl_up_sync(0xffffffffu, inc, off);
+                    if (tid >= off) inc += v;
+                }
+                if (inc - loc < (unsigned int)take && (unsigned int)take <= inc) {
+                    unsigned int acc = inc - loc;
+                    int q = 0;
+                    for (; q < 7 && acc + rank[255 - 8 * tid - q] < (unsigned int)take; ++q) acc += rank[255 - 8 * tid - q];
+                    s_digit = 255 - 8 * tid - q;
+                }
+            }
+            __syncthreads();
+            keep = keep && (int)dg >= s_digit;
+            if (keep) buf[atomicAdd(&s_keep, 1)] = f;
+            __syncthreads();
+            n_in = s_keep;
+            if (tid < n_in) f = buf[tid];
+            __syncthreads();
+        } else if (keep) {
+            buf[tid] = f;
+        }
+        rank_sort(buf, n_in, rank);
+        if (tid < n_in && (int)rank[tid] < take) sel[n_above + rank[tid]] = McSel{f.slot, f.g, f.A, f.B};
     }
     if (tid == 0) {
-        ms->m_sel = msel;
+        ms->m_sel = n_above + take;
         ms->n_above = 0;
         ms->n_inbin = 0;
     }

@@ -1037,21 +1037,71 @@ __global__ void __launch_bounds__(256) k_column(Problem P, unsigned long long A,
 // ---------------------------------------------------------------------------
 // Export of the stored entries (true values = stored * scale).
 // ---------------------------------------------------------------------------
-__global__ void k_export(Problem P, const IterState *st, unsigned long long *keys, double *c, double *b,
-                         long long cap, unsigned long long *counter) {
-    const double s = st->scale.hi + st->scale.lo;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P.capacity;
-         i += (long long)gridDim.x * blockDim.x) {
-        Slot sl = P.table[i];
-        if (sl.a == 0ull && sl.b == 0ull) continue;
-        unsigned long long pos = atomicAdd(counter, 1ull);
-        if ((long long)pos < cap) {
-            keys[2 * pos] = sl.a;
-            keys[2 * pos + 1] = sl.b & kKeyMaskB;
-            if (c) c[pos] = sl.c * s;
-            if (b) b[pos] = sl.bv * s;
+// Rows of the occupied slots, appended in block-sized pieces: a block takes
+// kExportTile slots a round, every thread kExportU of them with all loads in
+// flight (32 bytes each, consecutive threads on consecutive slots), counts the
+// occupied ones by ballots and reserves their rows with one atomic.  (One atomic
+// a row on the same counter: 14 M rows of a 2 GiB table took 2.03 ms, now 0.47 ms.)
+constexpr int kExportU = 4, kExportTile = 256 * kExportU;
+__device__ __forceinline__ Slot ld_slot_stream(const Slot *s) {
+    Slot x;
+    unsigned long long c, b;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(x.a), "=l"(x.b), "=l"(c), "=l"(b) : "l"(s));
+    x.c = __longlong_as_double((long long)c);
+    x.bv = __longlong_as_double((long long)b);
+    return x;
+}
+// row(i, slot, pos): write the row of slot i at pos
+template <class Row>
+__device__ __forceinline__ void export_rows(const Problem &P, long long cap, unsigned long long *counter, Row row) {
+    __shared__ unsigned int s_n[kExportU][8];
+    __shared__ unsigned long long s_base;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (long long i0 = (long long)blockIdx.x * kExportTile; i0 < P.capacity; i0 += (long long)gridDim.x * kExportTile) {
+        Slot sl[kExportU];
+        unsigned int m[kExportU];
+#pragma unroll
+        for (int u = 0; u < kExportU; ++u) {
+            const long long i = i0 + u * 256 + tid;
+            if (i < P.capacity) sl[u] = ld_slot_stream(P.table + i);
+            else sl[u].a = sl[u].b = 0ull;
         }
+#pragma unroll
+        for (int u = 0; u < kExportU; ++u) {
+            m[u] = __ballot_sync(0xffffffffu, (sl[u].a | sl[u].b) != 0ull);
+            if (lane == 0) s_n[u][warp] = (unsigned int)__popc(m[u]);
+        }
+        __syncthreads();
+        if (tid < 32) {                                 // exclusive offsets of the 32 (u, warp) pieces
+            const unsigned int x = s_n[tid >> 3][tid & 7];
+            unsigned int inc = x;
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned int v = __shfl_up_sync(0xffffffffu, inc, off);
+                if (tid >= off) inc += v;
+            }
+            s_n[tid >> 3][tid & 7] = inc - x;
+            if (tid == 31) s_base = inc ? atomicAdd(counter, (unsigned long long)inc) : 0ull;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kExportU; ++u) {
+            if ((m[u] >> lane) & 1u) {
+                const unsigned long long pos = s_base + s_n[u][warp] + (unsigned)__popc(m[u] & ((1u << lane) - 1u));
+                if ((long long)pos < cap) row(i0 + u * 256 + tid, sl[u], (long long)pos);
+            }
+        }
+        __syncthreads();                                // s_n, s_base read
     }
+}
+__global__ void __launch_bounds__(256) k_export(Problem P, const IterState *st, unsigned long long *keys, double *c,
+                                                double *b, long long cap, unsigned long long *counter) {
+    const double s = st->scale.hi + st->scale.lo;
+    export_rows(P, cap, counter, [&](long long, const Slot &sl, long long pos) {
+        reinterpret_cast<ulonglong2 *>(keys)[pos] = make_ulonglong2(sl.a, sl.b & kKeyMaskB);
+        if (c) c[pos] = sl.c * s;
+        if (b) b[pos] = sl.bv * s;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -1059,20 +1109,14 @@ __global__ void k_export(Problem P, const IterState *st, unsigned long long *key
 // ---------------------------------------------------------------------------
 // Every stored entry as stored (c, b divided by the scale for m > 1); flags
 // bit 0: the entry is marked as a candidate of the next block selection.
-__global__ void k_ckpt_export(Problem P, unsigned long long *keys, double *c, double *b, unsigned char *flags,
-                              long long cap, unsigned long long *counter) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P.capacity;
-         i += (long long)gridDim.x * blockDim.x) {
-        const Slot sl = P.table[i];
-        if (sl.a == 0ull && sl.b == 0ull) continue;
-        const unsigned long long pos = atomicAdd(counter, 1ull);
-        if ((long long)pos >= cap) continue;
-        keys[2 * pos] = sl.a;
-        keys[2 * pos + 1] = sl.b & kKeyMaskB;
+__global__ void __launch_bounds__(256) k_ckpt_export(Problem P, unsigned long long *keys, double *c, double *b,
+                                                     unsigned char *flags, long long cap, unsigned long long *counter) {
+    export_rows(P, cap, counter, [&](long long i, const Slot &sl, long long pos) {
+        reinterpret_cast<ulonglong2 *>(keys)[pos] = make_ulonglong2(sl.a, sl.b & kKeyMaskB);
         c[pos] = sl.c;
         b[pos] = sl.bv;
         flags[pos] = (P.mark ? mark_test(P, i) : (sl.b & kMarkB) != 0ull) ? 1 : 0;
-    }
+    });
 }
 
 // The pending partials of the last m = 1 column folded by one warp exactly as
@@ -1415,16 +1459,16 @@ cudaError_t launch_column(const Problem &P, unsigned long long A, unsigned long 
 
 cudaError_t launch_export(const Problem &P, const IterState *st, unsigned long long *keys, double *c, double *b,
                           long long cap, unsigned long long *counter, cudaStream_t s) {
-    long long grid = (P.capacity + 255) / 256;
-    if (grid > 152 * 16) grid = 152 * 16;
+    long long grid = (P.capacity + kExportTile - 1) / kExportTile;
+    if (grid > 152 * 6) grid = 152 * 6;
     k_export<<<(int)grid, 256, 0, s>>>(P, st, keys, c, b, cap, counter);
     return cudaGetLastError();
 }
 
 cudaError_t launch_ckpt_export(const Problem &P, unsigned long long *keys, double *c, double *b, unsigned char *flags,
                                long long cap, unsigned long long *counter, cudaStream_t s) {
-    long long grid = (P.capacity + 255) / 256;
-    if (grid > 152 * 16) grid = 152 * 16;
+    long long grid = (P.capacity + kExportTile - 1) / kExportTile;
+    if (grid > 152 * 6) grid = 152 * 6;
     k_ckpt_export<<<(int)grid, 256, 0, s>>>(P, keys, c, b, flags, cap, counter);
     return cudaGetLastError();
 }
