@@ -919,11 +919,15 @@ __global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McSta
 // 4 entries, so that a row of A times a vector reads 16 bytes per load along
 // the row (R is symmetric).
 // ---------------------------------------------------------------------------
-constexpr int kEigSmemN = 160;      // A in shared memory (hi and lo) up to this size
 constexpr int kEigMaxIt = 200;
+// k_mc_eigen_reg: a thread holds kRegRows rows x kRegChunks float4 of R; threads and rows at most
+constexpr int kRegRows = 4, kRegChunks = 3, kRegThreads = 640, kRegMaxN = 320, kRegSlots = 4 * (kRegThreads / 32);
 
 // How the reduced problem of size n1 = m + 1 is laid out:
-//   n1 <= kEigSmemN: one CTA, R in its shared memory, 2 threads per row;
+//   n1 <= kRegMaxN: R's leading parts in registers (reg = 1), one CTA up to 160
+//   rows, else a cluster of 4; tpr >= 4 lanes share kRegRows rows, the smallest
+//   power of two for which a lane's share of a row fits kRegChunks float4 (then
+//   at most kRegThreads threads a CTA);
 //   else a cluster of C = 2, 4 or 8 CTAs, each holding a block of `crows` rows
 //   of R (hi and lo) in its shared memory, tpr threads per row, when such a
 //   split fits (at most 32 warps in the cluster, the rows within
@@ -931,26 +935,34 @@ constexpr int kEigMaxIt = 200;
 //   else one CTA streaming R from global memory (C = 0), 1 thread per row.
 constexpr size_t kEigClusterBytes = 192 * 1024;
 struct EigCfg {
-    int C, tpr, crows;
+    int C, tpr, crows, reg;
 };
 __host__ __device__ __forceinline__ EigCfg eig_cfg(int n1) {
-    if (n1 <= kEigSmemN) return EigCfg{1, 2, n1};
+    if (n1 <= kRegMaxN) {
+        const int C = n1 <= 160 ? 1 : 4, nq = (n1 + 3) / 4;
+        int tpr = 4;
+        while ((nq + tpr - 1) / tpr > kRegChunks) tpr *= 2;
+        return EigCfg{C, tpr, (n1 + C - 1) / C, 1};
+    }
     for (int C = 2; C <= 8; C *= 2) {
         const int crows = (n1 + C - 1) / C;
         for (int tpr = 2; tpr >= 1; --tpr) {
             const int nw = tpr * ((crows + 31) / 32);
             const size_t ldr = 32 * (size_t)((n1 + 31) / 32) + 4 * (size_t)tpr;
-            if (C * nw <= 32 && 8 * (size_t)crows * ldr <= kEigClusterBytes) return EigCfg{C, tpr, crows};
+            if (C * nw <= 32 && 8 * (size_t)crows * ldr <= kEigClusterBytes) return EigCfg{C, tpr, crows, 0};
         }
     }
-    return EigCfg{0, 1, n1};
+    return EigCfg{0, 1, n1, 0};
 }
-// threads per row and R's row stride: a multiple of 32 floats plus 4 tpr, which
+// threads per row and R's row stride: a multiple of 32 floats plus 4 tpr (4 with R in registers), which
 // puts the 16-byte loads of a quarter warp (8 lanes: 8 / tpr rows, tpr chunks
 // each) on distinct banks; the same stride in global and shared memory makes
 // each CTA's block of rows one contiguous bulk copy
 __host__ __device__ __forceinline__ int eig_tpr(int n1) { return eig_cfg(n1).tpr; }
-__host__ __device__ __forceinline__ int eig_ldr(int n1) { return 32 * ((n1 + 31) / 32) + 4 * eig_tpr(n1); }
+__host__ __device__ __forceinline__ int eig_ldr(int n1) {
+    const EigCfg g = eig_cfg(n1);
+    return 32 * ((n1 + 31) / 32) + (g.reg ? 4 : 4 * g.tpr);
+}
 // entries of a vector in absolute indexing, a multiple of 4
 __host__ __device__ __forceinline__ int eig_len(int n1) { return 4 * ((n1 + 3) / 4); }
 
@@ -1205,15 +1217,12 @@ __device__ void eig_stream(const float *Rh, const float *Rl, int ldr, int n1, in
     if (late) set_status(st, kErrTimeout);
 }
 
-// CL = false: one CTA holds the whole problem (R in its shared memory when
-// SM, else streamed from global memory); CL = true (with SM): a cluster of C CTAs,
-// CTA r holding rows [r crows, (r + 1) crows) of R in its shared memory, the
+// The reduced problem above kRegMaxN rows.  CL = false: one CTA, R streamed from
+// global memory; CL = true: a cluster of C CTAs, CTA r holding rows [r crows, (r + 1) crows) of R in its shared memory, the
 // vectors x and w gathered in full in every CTA before each product, the sums
 // taken over the cluster.  Every CTA computes the scalar steps itself, from
 // the same sums in the same order, so they agree bit for bit.
-// (SM is a template parameter so that each instantiation holds only the code it runs: the kernel runs
-// once per iteration on whichever SM is free, its instructions fetched from L2 each time.)
-template <bool CL, bool SM>
+template <bool CL>
 __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, IterState *st, const McSel *sel,
                                                        const double *cI, const double *bI, const double *HIIc,
                                                        const double *Hdiag, const float4 *rowf, float *Rh, float *Rl,
@@ -1238,7 +1247,7 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
     const int m = ms->m_sel, n1 = m + 1;
     // this CTA's rows of R (absolute indices [a0, a1)); one CTA: all
     const int a0 = CL ? (int)rank * crows : 0, a1 = CL ? min(a0 + crows, n1) : n1;
-    constexpr bool in_smem = CL || SM;
+    constexpr bool in_smem = CL;
     // the state scalars, loaded (thread 0) ahead of the sums; read after the barriers below
     __shared__ dd s_mu0, s_al0, s_sc0;
     __shared__ long long s_nnz0;
@@ -1636,6 +1645,622 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
             ms->n_cand = 0;                             // the scatter builds the next candidate list
             if (bad) set_status(st, kErrNonfinite);
         }
+    }
+    __syncthreads();
+    // 6. the scatter weights and the new stored c_I; the change in nonzeros of c
+    const double rsc = s_sc[6];
+    bool to = false, from = false;
+    if (coord) {
+        w[ic] = eta * rsc;
+        if (!bad) {
+            P.table[sel[ic].slot].c = zn * rsc;
+            cnz_set(P, sel[ic].A, sel[ic].B);
+        }
+        from = ct != 0.0 && zn == 0.0;
+        to = ct == 0.0 && zn != 0.0;
+    }
+    const int dn = __popc(__ballot_sync(0xffffffffu, to)) - __popc(__ballot_sync(0xffffffffu, from));
+    if (lane == 0 && dn != 0 && !bad) atomicAdd(reinterpret_cast<unsigned long long *>(&ms->nnz_c),
+                                                (unsigned long long)(long long)dn);
+}
+
+// ---------------------------------------------------------------------------
+// The reduced problem for n1 <= kRegMaxN: the same iteration with the FP32 part
+// of R in registers.  What bounds it is latency: a chain of products, sums and
+// one 3 x 3 problem per iteration on a few warps, in which a load from shared
+// memory returns 64 bytes a cycle to the whole SM whether its lanes share an
+// address or not, and a shuffle is one a cycle or two.  So:
+//   - a group of tpr lanes holds 4 rows of R's leading parts, each lane
+//     kRegChunks float4 chunks q = k, k + tpr, ... of each: every vector entry it
+//     loads serves 4 rows.  The 4 partial sums halve with the lanes, and a lane
+//     ends with the row of its two leading lane bits, which it owns from then on
+//     (tpr / 4 copies; the first one speaks for the row in sums).  R's trailing
+//     parts stay in shared memory for the two float-float products of a solve;
+//   - the sums of an iteration are taken together after the product (13 values,
+//     halved with the lanes as well): the preconditioned residual w enters the
+//     product as it is.  Where x holds a good part (a quarter) of the direction
+//     c~ / nu, whose diagonal R_00 is then close to theta, that direction is left
+//     out of w: its amplified entry would make w parallel to x.  (Left out where
+//     x holds little of it, the iteration does not converge.)  A w that is
+//     parallel to x all the same is orthogonalised and the product taken again;
+//   - theta is predicted from the Ritz value between exact products (x.r enters
+//     the pencil); at the start it is alpha / mu;
+//   - warp 0 alone adds the warps' sums, makes the tests and solves the 3 x 3
+//     problem (ritz_near: Newton's iteration from theta), the coordinates of the
+//     epilogue are packed onto as few warps as hold them (an FP64 instruction
+//     costs its warp's issue, not its lanes').
+// A launch inside the graph: m = 64 40.5 -> 26.1 us, m = 128 55.7 -> 39.6, m = 256 (4 CTAs) 55.9 -> 42.8.
+// Up to 160 rows one CTA; above, a cluster of 4 with the vectors gathered in full
+// in every CTA, the sums taken over the cluster, and the scalar steps computed in
+// every CTA from the same sums in the same order (two cluster barriers an
+// iteration).
+// ---------------------------------------------------------------------------
+// sums of 16 values over the warp: lane l holds the sum of value l >> 1
+__device__ __forceinline__ float wred16(float (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8; h >= 1; h >>= 1) {
+        const bool up = lane & (2 * h);
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float give = up ? v[i] : v[i + h];
+            v[i] = (up ? v[i + h] : v[i]) + __shfl_xor_sync(0xffffffffu, give, 2 * h);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+// The four rows' partial sums over a group of g >= 4 lanes: each lane receives
+// the sum of the row 2 [lane & g/2] + [lane & g/4].
+__device__ __forceinline__ float rows4_sum(const float (&v)[4], int g) {
+    const int lane = threadIdx.x & 31, h2 = g >> 1, h1 = g >> 2;
+    const bool up = lane & h2, up2 = lane & h1;
+    float x0 = up ? v[2] : v[0], x1 = up ? v[3] : v[1];
+    x0 += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], h2);
+    x1 += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], h2);
+    float z = (up2 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, up2 ? x0 : x1, h1);
+    for (int o = h1 >> 1; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    return z;
+}
+__device__ __forceinline__ ff ff_shfl_xor(ff a, int o) {
+    return ff{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ ff rows4_sum_ff(const ff (&v)[4], int g) {
+    const int lane = threadIdx.x & 31, h2 = g >> 1, h1 = g >> 2;
+    const bool up = lane & h2, up2 = lane & h1;
+    const ff x0 = ff_add(up ? v[2] : v[0], ff_shfl_xor(up ? v[0] : v[2], h2));
+    const ff x1 = ff_add(up ? v[3] : v[1], ff_shfl_xor(up ? v[1] : v[3], h2));
+    ff z = ff_add(up2 ? x1 : x0, ff_shfl_xor(up2 ? x0 : x1, h1));
+    for (int o = h1 >> 1; o > 0; o >>= 1) z = ff_add(z, ff_shfl_xor(z, o));
+    return z;
+}
+
+// Sums of one iteration: the pencil P - mu G on span{x, w, p}, P shifted by theta
+// (its x row is (A x - theta x) . [x, w, p]), G the Gram matrix; |r|^2.
+struct RitzSums {
+    float xr, rw, rp, sww, swp, spp, xx, xw, xp, ww, wp, pp, rr;
+};
+// The lowest Ritz pair with y = (1, yw, yp), near mu = 0: eliminating w and p
+// leaves f(mu) = a + b.z = 0 with a = xr - mu xx, b = (rw, rp) - mu (xw, xp),
+// S = P_wp - mu G_wp, z = -S^-1 b, and f'(mu) = -|y|_G^2; so Newton's step is the
+// quotient y^T P y / y^T G y.  Taken from mu = 0 until mu no longer moves S (late
+// iterations: one step; a z off by 0.03 % changes the quotient, which is exact
+// for the y returned, by its square).  With S positive definite it is the lowest
+// pair (the only root to the left of S's).  false: S is not safely positive
+// definite, or four steps have not settled.
+__device__ __forceinline__ bool ritz_near(const RitzSums &s, bool use_p, float &mu, float &yw, float &yp) {
+    mu = 0.0f; yw = 0.0f; yp = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const float b0 = fmaf(-mu, s.xw, s.rw), b1 = use_p ? fmaf(-mu, s.xp, s.rp) : 0.0f;
+        const float s00 = fmaf(-mu, s.ww, s.sww);
+        const float s01 = use_p ? fmaf(-mu, s.wp, s.swp) : 0.0f, s11 = use_p ? fmaf(-mu, s.pp, s.spp) : 1.0f;
+        const float prod = s00 * s11, det = fmaf(-s01, s01, prod);
+        if (!(s00 > 0.0f && det > 1e-4f * prod)) return false;
+        const float id = __fdividef(1.0f, det);
+        yw = (s01 * b1 - s11 * b0) * id;
+        yp = (s01 * b0 - s00 * b1) * id;
+        const float py = (s.xr + 2.0f * fmaf(s.rw, yw, s.rp * yp)) + fmaf(yw, fmaf(s.sww, yw, 2.0f * s.swp * yp), s.spp * yp * yp);
+        const float gy = (s.xx + 2.0f * fmaf(s.xw, yw, s.xp * yp)) + fmaf(yw, fmaf(s.ww, yw, 2.0f * s.wp * yp), s.pp * yp * yp);
+        if (!(gy > 0.0f)) return false;
+        const float nu = __fdividef(py, gy), step = fabsf(nu - mu);
+        mu = nu;
+        if (step * s.ww <= 3e-4f * s00 && (!use_p || step * s.pp <= 3e-4f * s11)) return true;
+    }
+    return false;
+}
+// The lowest Ritz pair in general, by the Cholesky factor of G (|y|_G = 1, yx >= 0);
+// without p when it is not usable, x alone when w is not.
+__device__ __noinline__ void ritz_full(const RitzSums &s, bool use_p, float &mu, float &yx, float &yw, float &yp) {
+    mu = 0.0f; yx = 1.0f; yw = 0.0f; yp = 0.0f;
+    const float i0 = rsqrtf(s.xx), l10 = s.xw * i0, l20 = s.xp * i0, d11 = s.ww - l10 * l10;
+    if (!(d11 > 1e-12f * s.ww) || !(s.ww > 0.0f)) return;
+    const float i1 = rsqrtf(d11);
+    float l21 = 0.0f, i2 = 0.0f;
+    use_p = use_p && s.pp > 0.0f;
+    if (use_p) {
+        l21 = (s.wp - l20 * l10) * i1;
+        const float d22 = s.pp - l20 * l20 - l21 * l21;
+        use_p = d22 > 1e-6f * s.pp;
+        if (use_p) i2 = rsqrtf(d22);
+    }
+    // M = L^-1 P (rows), then C = M L^-T
+    const float m00 = s.xr * i0, m01 = s.rw * i0, m02 = s.rp * i0;
+    const float m10 = (s.rw - l10 * m00) * i1, m11 = (s.sww - l10 * m01) * i1, m12 = (s.swp - l10 * m02) * i1;
+    const float c00 = m00 * i0, c01 = (m01 - l10 * c00) * i1, c10 = m10 * i0, c11 = (m11 - l10 * c10) * i1;
+    float v0, v1, v2 = 0.0f, lam;
+    if (use_p) {
+        const float m20 = (s.rp - l20 * m00 - l21 * m10) * i2, m21 = (s.swp - l20 * m01 - l21 * m11) * i2;
+        const float m22 = (s.spp - l20 * m02 - l21 * m12) * i2;
+        const float c02 = (m02 - l20 * c00 - l21 * c01) * i2, c12 = (m12 - l20 * c10 - l21 * c11) * i2;
+        const float c20 = m20 * i0, c22 = (m22 - l20 * c20 - l21 * ((m21 - l10 * c20) * i1)) * i2;
+        sym3_lowest(c00, c01, c02, c11, c12, c22, lam, v0, v1, v2);
+    } else {
+        sym2_lowest(c00, c01, c11, lam, v0, v1);
+    }
+    yp = v2 * i2;
+    yw = (v1 - l21 * yp) * i1;
+    yx = (v0 - l10 * yw - l20 * yp) * i0;
+    if (yx < 0.0f) { yx = -yx; yw = -yw; yp = -yp; }
+    // mu as the quotient of y: the root of the cubic carries the rounding of the pencil's largest
+    // entries, the quotient only that of its own small terms
+    const float py = yx * (s.xr * yx + 2.0f * (s.rw * yw + s.rp * yp)) + yw * (s.sww * yw + 2.0f * s.swp * yp) +
+                     s.spp * yp * yp;
+    const float gy = yx * (s.xx * yx + 2.0f * (s.xw * yw + s.xp * yp)) + yw * (s.ww * yw + 2.0f * s.wp * yp) +
+                     s.pp * yp * yp;
+    mu = __fdividef(py, gy);
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState *ms, IterState *st, const McSel *sel,
+                                                              const double *cI, const double *bI, const double *HIIc,
+                                                              const double *Hdiag, const float4 *rowf,
+                                                              const float *Rh, const float *Rl, int ldr, int tpr,
+                                                              int crows, double *w, double *thr, double *etaout) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ __align__(16) float s_r2[2][kRegSlots * 16];
+    __shared__ ff s_rff[kRegSlots * 2];
+    __shared__ double s_red[32 * 4];
+    __shared__ ff s_row0[6];                            // nu, R_00, (A x)_0 of the start, 1 / nu; theta and x.x of the start
+    __shared__ ff s_x0;                                 // x_0 at the end (CL: from CTA 0)
+    __shared__ float s_y[7];                            // mu, yx, yw, yp; 1 / |new p|; new x.p / x.x, or x.w / x.x; new |x|^2
+    __shared__ int s_ctl;                               // 1: converged, 2: recompute A x, 4: orthogonalise w and repeat
+    __shared__ double s_sc[8];
+    __shared__ float s_drms;
+    __shared__ int s_nzr[32], s_flag, s_zero, s_late[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (ms->done || st->status) return;
+    unsigned rank = 0, C = 1;
+    if (CL) {
+        rank = cg::this_cluster().block_rank();
+        C = cg::this_cluster().num_blocks();
+    }
+    const int ns = (int)C * nw, slot = (int)rank * nw + warp;
+    auto sync_all = [&]() { if (CL) cg::this_cluster().sync(); else __syncthreads(); };
+    // the same address of `p` in every CTA of the cluster: f(pointer)
+    auto everywhere = [&](auto *p, auto f) {
+        if (CL) {
+            cg::cluster_group cl = cg::this_cluster();
+            for (unsigned r = 0; r < C; ++r) f(cl.map_shared_rank(p, r));
+        } else {
+            f(p);
+        }
+    };
+    const int m = ms->m_sel, n1 = m + 1;
+    const int a0 = CL ? (int)rank * crows : 0, a1 = CL ? min(a0 + crows, n1) : n1;
+    __shared__ dd s_mu0, s_al0, s_sc0;
+    __shared__ long long s_nnz0;
+    if (tid == 0) { s_mu0 = ms->mu; s_al0 = ms->alpha; s_sc0 = ms->scale; s_nnz0 = ms->nnz_c; }
+    const int L = eig_len(n1), nq = L / 4;
+    const int nown = a1 > a0 ? a1 - a0 : 0;             // rows held here
+    // (offsets use crows and the block's m, not this CTA's own number of rows: the other CTAs address them)
+    float *sl = sm;
+    __shared__ unsigned long long s_bar;
+    if (tid == 0 && nown > 0) {                         // R's trailing parts: one bulk copy, needed late
+        const unsigned bytes = (unsigned)nown * (unsigned)ldr * 4u;
+        mbar_init_arm(&s_bar, bytes);
+        bulk_g2s(sl, Rl + (size_t)a0 * ldr, bytes, &s_bar);
+    }
+    // this thread's share of R's leading parts: rows a0 + 4 grp + i (columns past n1 meet zeros of the
+    // vectors); the row it owns
+    const int grp = tid / tpr, kk = tid - grp * tpr;
+    const int ra = a0 + kRegRows * grp + ((kk & (tpr >> 1)) ? 2 : 0) + ((kk & (tpr >> 2)) ? 1 : 0);
+    const bool row = ra < a1;
+    float4 A[kRegRows][kRegChunks];
+#pragma unroll
+    for (int i = 0; i < kRegRows; ++i) {
+        const int rr = a0 + kRegRows * grp + i;
+        const float4 *src = reinterpret_cast<const float4 *>(Rh + (size_t)(rr < a1 ? rr : a0) * ldr);
+#pragma unroll
+        for (int u = 0; u < kRegChunks; ++u) {
+            const int q = kk + tpr * u;
+            A[i][u] = rr < a1 && q < nq ? __ldcg(src + q) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    }
+    float *vec = sm + (size_t)crows * ldr;
+    float *xs = vec;                                    // float-float x (2 L floats)
+    float *ws = vec + 2 * L;                            // FP32 w (L floats)
+    float *az = vec + 3 * L;                            // the start's A x (float-float, 2 L floats)
+    float *hs = vec + 5 * L;                            // the start's H_II c_I (float-float, 2 L floats)
+    float *r0s = vec + 7 * L;                           // row 0 of R (float-float, 2 L floats)
+
+    // 1. sums over I (FP64): c.c, c.b, c.H_II c, |diag H_II|^2, nonzeros; the start values staged
+    const int nsw = (min(m, (int)blockDim.x) + 31) >> 5;
+    double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
+    int nzc = 0;
+    for (int t = tid; t < m; t += blockDim.x) {
+        const double c0 = cI[t], bt = bI[t], ht = HIIc[t], hd = Hdiag[t];
+        const float4 f0 = rowf[2 * t], f1 = rowf[2 * t + 1];
+        p0 = fma(c0, c0, p0); p1 = fma(c0, bt, p1); p2 = fma(c0, ht, p2); p3 = fma(hd, hd, p3);
+        nzc += (__double_as_longlong(c0) << 1) != 0 ? 1 : 0;
+        const int a = t + 1;
+        xs[2 * a] = f0.x; xs[2 * a + 1] = f0.y;         // c_i
+        az[2 * a] = f0.z; az[2 * a + 1] = f0.w;         // b_i
+        hs[2 * a] = f1.x; hs[2 * a + 1] = f1.y;         // (H_II c_I)_i
+        r0s[2 * a] = f1.z; r0s[2 * a + 1] = f1.w;       // b_i - (H_II c_I)_i
+    }
+    if (warp < nsw) {
+        const double t = wsum4(p0, p1, p2, p3);
+        const int nzw = __reduce_add_sync(0xffffffffu, nzc);
+        if ((lane & 7) == 0) s_red[warp * 4 + (lane >> 3)] = t;
+        if (lane == 0) s_nzr[warp] = nzw;
+    }
+    for (int t = n1 + tid; t < L; t += blockDim.x) {
+        xs[2 * t] = 0.0f; xs[2 * t + 1] = 0.0f; ws[t] = 0.0f;
+        r0s[2 * t] = 0.0f; r0s[2 * t + 1] = 0.0f;
+    }
+    if (tid == 0) { xs[0] = 0.0f; xs[1] = 0.0f; ws[0] = 0.0f; }
+    __syncthreads();
+    // 2. warp 0: nu, R_00, (A x)_0, 1 / nu (see k_mc_eigen)
+    if (warp == 0) {
+        double t = 0.0;
+        for (int q = lane & 7; q < nsw; q += 8) t += s_red[q * 4 + (lane >> 3)];
+        t += __shfl_xor_sync(0xffffffffu, t, 4);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        const double cc = __shfl_sync(0xffffffffu, t, 0), cb = __shfl_sync(0xffffffffu, t, 8);
+        const double chc = __shfl_sync(0xffffffffu, t, 16), hh = __shfl_sync(0xffffffffu, t, 24);
+        int nz = 0;
+        for (int q = 0; q < nsw; ++q) nz += s_nzr[q];
+        // (lanes 4..7: alpha, mu, c.H c, c.c as they are, for the quotient of the start)
+        const dd a = lane == 0 || lane == 5 ? s_mu0 : (lane == 6 || lane == 7 ? dd_from(lane == 6 ? chc : cc) : s_al0);
+        const double p = lane == 0 ? -cc : (lane == 1 ? -2.0 * cb : (lane >= 4 ? 0.0 : -cb));
+        const double q = lane == 1 ? chc : 0.0;
+        const dd s1 = dd_two_sum(a.hi, p), s2 = dd_two_sum(s1.hi, q);
+        const double r = s2.hi + ((s1.lo + s2.lo) + a.lo);
+        const double nu2 = __shfl_sync(0xffffffffu, r, 0);
+        const long long nb = __double_as_longlong(nu2);
+        const bool deg = (nz >= s_nnz0) || nb <= 0;     // nu^2 <= 0
+        const int ex = (int)((nb >> 52) & 0x7ff) - 1023;
+        const ff rf = ff_from_double(r), n2f = {__shfl_sync(0xffffffffu, rf.hi, 0), __shfl_sync(0xffffffffu, rf.lo, 0)};
+        ff inu_f = {0.0f, 0.0f};
+        if (!deg) {
+            if (ex > -120 && ex < 120) inu_f = ff_rsqrt(n2f);
+            else inu_f = ff_from_double(rsqrt(nu2));
+        }
+        // lane 0: nu = nu^2 / nu, lane 1: R_00, lane 2: (A x)_0, lane 3: 1 / nu
+        const ff yf = lane == 3 ? inu_f : ff_mul(ff_mul(rf, inu_f), lane == 1 ? inu_f : ff{1.0f, 0.0f});
+        if (lane < 4) s_row0[lane] = yf;
+        // theta of the start (x.x = mu, x.A x = alpha for x = [nu; c_I]): lane 4 takes alpha / mu, or
+        // c.H c / c.c in the degenerate case
+        const int from = deg ? 6 : 4;
+        const ff tn = {__shfl_sync(0xffffffffu, rf.hi, from), __shfl_sync(0xffffffffu, rf.lo, from)};
+        const ff td = {__shfl_sync(0xffffffffu, rf.hi, from + 1), __shfl_sync(0xffffffffu, rf.lo, from + 1)};
+        if (lane == 4) {
+            s_row0[4] = td.hi != 0.0f ? ff_div(tn, td) : ff{0.0f, 0.0f};
+            s_row0[5] = td;
+        }
+        const float r00 = __shfl_sync(0xffffffffu, yf.hi, 1);
+        if (lane == 0) {
+            s_sc[0] = deg ? 1.0 : 0.0;
+            s_zero = (deg && __double_as_longlong(cc) <= 0) ? 1 : 0;   // c = 0: no start vector
+            const float nf = (float)(m + (deg ? 0 : 1));
+            s_drms = sqrtf((__double2float_rn(hh) + (deg ? 0.0f : r00 * r00)) / nf);
+        }
+    }
+    // the copy: a bounded wait, the decision shared over the cluster (see k_mc_eigen)
+    const bool late = nown > 0 && !mbar_wait0(&s_bar, 1 << 22);
+    bool any_late = __syncthreads_or(late);
+    if (CL) {
+        if (tid == 0) everywhere(s_late, [&](int *p) { p[rank] = any_late ? 1 : 0; });
+        cg::this_cluster().sync();
+        any_late = false;
+        for (unsigned r = 0; r < C; ++r) any_late |= s_late[r] != 0;
+    }
+    if (any_late) {
+        if (tid == 0) set_status(st, kErrTimeout);
+        if (late) mbar_wait0(&s_bar, 1 << 22);
+        return;
+    }
+    const bool deg = s_sc[0] != 0.0;
+    const int off = deg ? 1 : 0;
+    const int n = n1 - off;                             // active size
+    // row and column 0 of R: R_0i = (b_i - (H_II c_I)_i) / nu (zero when not active), into r0s, column 0
+    // of the trailing parts here, and below into the registers that hold them
+    {
+        const ff inu = s_row0[3];
+        for (int t = tid; t < n1; t += blockDim.x) {
+            ff v = {0.0f, 0.0f};
+            if (!deg) v = t == 0 ? s_row0[1] : ff_mul(ff{r0s[2 * t], r0s[2 * t + 1]}, inu);
+            r0s[2 * t] = v.hi; r0s[2 * t + 1] = v.lo;
+            if (t >= a0 && t < a1) sl[(size_t)(t - a0) * ldr] = v.lo;
+            if (a0 == 0 && nown > 0) sl[t] = v.lo;
+        }
+    }
+    __syncthreads();
+    if (kk == 0) {
+#pragma unroll
+        for (int i = 0; i < kRegRows; ++i) {
+            const int rr = a0 + kRegRows * grp + i;
+            if (rr < a1) A[i][0].x = r0s[2 * rr];
+        }
+    }
+    if (a0 == 0 && grp == 0) {
+#pragma unroll
+        for (int u = 0; u < kRegChunks; ++u) {
+            const int q = kk + tpr * u;
+            if (q < nq) A[0][u] = make_float4(r0s[8 * q], r0s[8 * q + 2], r0s[8 * q + 4], r0s[8 * q + 6]);
+        }
+    }
+
+    // 3. the start: x = [nu; c_I], A x in closed form (see k_mc_eigen)
+    const bool act = row && ra >= off, lead = act && (kk & ((tpr >> 2) - 1)) == 0;
+    const bool zero_start = s_zero != 0;
+    ff x = {0.0f, 0.0f}, ax = {0.0f, 0.0f};
+    float d = 0.0f;
+    if (act) {
+        if (zero_start) {
+            x = ff{ra == off ? 1.0f : 0.0f, 0.0f};
+        } else if (ra == 0) {
+            x = s_row0[0];
+            ax = s_row0[2];
+        } else {
+            x = ff{xs[2 * ra], xs[2 * ra + 1]};
+            const float *src = deg ? hs : az;
+            ax = ff{src[2 * ra], src[2 * ra + 1]};
+        }
+        d = ra == 0 ? s_row0[1].hi : __ldcg(Rh + (size_t)ra * ldr + ra);
+    }
+    if (CL) cg::this_cluster().sync();                  // xs and ws are rewritten by other CTAs from here on
+    float pv = 0.0f, apv = 0.0f;                        // search direction p and A p
+    bool have_p = false;
+    ff theta = s_row0[4], xx = {1.0f, 0.0f};
+    float xxf = zero_start ? 1.0f : s_row0[5].hi;       // |x|^2 (FP32)
+    float best = 3.0e38f;                               // (the tests' state: warp 0)
+    int stall = 0, it = 0;
+    const float drms = s_drms;                          // RMS of diag A, a scale for the tests below
+    // A x follows x implicitly and is recomputed exactly each time the residual falls below `refresh`
+    // and before convergence is accepted (see k_mc_eigen); theta is exact then
+    bool exact = false, want_exact = zero_start;
+    float refresh = 1e-12f;                             // (relative |r|^2: |r| below 1e-6 of the scale)
+    for (;; ++it) {
+        exact = want_exact;
+        if (want_exact) {
+            if (lead) everywhere(xs, [&](float *p) { p[2 * ra] = x.hi; p[2 * ra + 1] = x.lo; });
+            sync_all();
+            float sh[kRegRows], sv[kRegRows];
+#pragma unroll
+            for (int i = 0; i < kRegRows; ++i) sh[i] = sv[i] = 0.0f;
+            const float4 *x4 = reinterpret_cast<const float4 *>(xs);
+#pragma unroll
+            for (int u = 0; u < kRegChunks; ++u) {
+                const int q = kk + tpr * u;
+                if (q < nq) {
+                    const float4 xa = x4[2 * q], xb = x4[2 * q + 1];
+#pragma unroll
+                    for (int i = 0; i < kRegRows; ++i) {
+                        const int rl = kRegRows * grp + i;
+                        const float4 lv = reinterpret_cast<const float4 *>(sl + (size_t)(rl < nown ? rl : 0) * ldr)[q];
+                        ff_mac(sh[i], sv[i], A[i][u].x, lv.x, ff{xa.x, xa.y});
+                        ff_mac(sh[i], sv[i], A[i][u].y, lv.y, ff{xa.z, xa.w});
+                        ff_mac(sh[i], sv[i], A[i][u].z, lv.z, ff{xb.x, xb.y});
+                        ff_mac(sh[i], sv[i], A[i][u].w, lv.w, ff{xb.z, xb.w});
+                    }
+                }
+            }
+            ff v4[kRegRows];
+#pragma unroll
+            for (int i = 0; i < kRegRows; ++i) v4[i] = ff_norm(sh[i], sv[i]);
+            ax = rows4_sum_ff(v4, tpr);
+            if (!act) ax = ff{0.0f, 0.0f};
+            want_exact = false;
+            // theta = x.Ax / x.x in float-float: lanes 0..15 of a warp end with its part of x.Ax, 16..31 of x.x
+            const ff ta = lead ? ff_mul(x, ax) : ff{0.0f, 0.0f}, tb = lead ? ff_mul(x, x) : ff{0.0f, 0.0f};
+            const bool up = lane & 16;
+            ff t = ff_add(up ? tb : ta, ff_shfl_xor(up ? ta : tb, 16));
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t = ff_add(t, ff_shfl_xor(t, o));
+            if ((lane & 15) == 0) everywhere(s_rff, [&](ff *p) { p[slot * 2 + (lane >> 4)] = t; });
+            sync_all();
+            t = ff{0.0f, 0.0f};
+            for (int q = lane & 15; q < ns; q += 16) t = ff_add(t, s_rff[q * 2 + (lane >> 4)]);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t = ff_add(t, ff_shfl_xor(t, o));
+            const ff o = ff_shfl_xor(t, 16);
+            xx = up ? t : o;
+            theta = ff_div(up ? o : t, xx);
+        }
+        // (a) r = A x - theta x and the preconditioned residual w = r / |A_ii - theta|
+        const float r = act ? ff_to_float(ff_add(ax, ff_neg(ff_mul(theta, x)))) : 0.0f;
+        const float th = ff_to_float(theta);
+        const float scale = fmaxf(fabsf(th), drms);
+        const float den = fmaxf(fabsf(d - th), 1e-4f * fmaxf(scale, 1e-30f));
+        const float xh = x.hi;
+        const bool in_x = ra == 0 && !deg && xh * xh > 0.25f * xxf;
+        float wv = act && !in_x ? __fdividef(r, den) : 0.0f;
+        // (b) A w; (c) the iteration's sums, the tests and the 3 x 3 problem (warp 0).  Where w is nearly
+        // parallel to x, both once more with w orthogonalised (before the product, so that A w
+        // stays consistent with the rounded w)
+        int ctl = 0;
+        float awv = 0.0f;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            if (lead) everywhere(ws, [&](float *p) { p[ra] = wv; });
+            sync_all();
+            float acc[kRegRows];
+#pragma unroll
+            for (int i = 0; i < kRegRows; ++i) acc[i] = 0.0f;
+            const float4 *w4 = reinterpret_cast<const float4 *>(ws);
+#pragma unroll
+            for (int u = 0; u < kRegChunks; ++u) {
+                const int q = kk + tpr * u;
+                const float4 v = w4[q < nq ? q : 0];    // (A's chunks past the row are zero)
+#pragma unroll
+                for (int i = 0; i < kRegRows; ++i) {
+                    acc[i] = fmaf(A[i][u].x, v.x, acc[i]);
+                    acc[i] = fmaf(A[i][u].y, v.y, acc[i]);
+                    acc[i] = fmaf(A[i][u].z, v.z, acc[i]);
+                    acc[i] = fmaf(A[i][u].w, v.w, acc[i]);
+                }
+            }
+            awv = rows4_sum(acc, tpr);
+            if (!act) awv = 0.0f;
+            const float aws = awv - th * wv, aps = apv - th * pv;
+            const float xl = lead ? xh : 0.0f, wl = lead ? wv : 0.0f, pl = lead ? pv : 0.0f, rl = lead ? r : 0.0f;
+            float pr[16] = {xl * r, rl * wv, rl * pv, wl * aws, wl * aps, pl * aps, xl * xh, xl * wv, xl * pv, wl * wv,
+                            wl * pv, pl * pv, rl * r, 0.0f, 0.0f, 0.0f};
+            const float v = wred16(pr);
+            if ((lane & 1) == 0) everywhere(s_r2[pass], [&](float *p) { p[slot * 16 + (lane >> 1)] = v; });
+            sync_all();
+            if (warp == 0) {
+                // value lane & 15 over the slots lane >> 4, + 2, ...
+                const float *src = s_r2[pass] + (lane & 15);
+                float t0 = 0.0f, t1 = 0.0f;
+                int q = lane >> 4;
+                for (; q + 6 < ns; q += 8) {
+                    t0 += src[q * 16] + src[(q + 2) * 16];
+                    t1 += src[(q + 4) * 16] + src[(q + 6) * 16];
+                }
+                for (; q < ns; q += 2) t0 += src[q * 16];
+                t0 += t1;
+                t0 += __shfl_xor_sync(0xffffffffu, t0, 16);
+                auto get = [&](int k) { return __shfl_sync(0xffffffffu, t0, k); };
+                RitzSums s;
+                s.xr = get(0); s.rw = get(1); s.rp = get(2); s.sww = get(3); s.swp = get(4); s.spp = get(5);
+                s.xx = get(6); s.xw = get(7); s.xp = get(8); s.ww = get(9); s.wp = get(10); s.pp = get(11); s.rr = get(12);
+                int c = 0;
+                if (pass == 0) {
+                    // stop at the float-float floor, at the cap, or when progress has ended well below it;
+                    // only a residual of an exact A x ends the iteration (see k_mc_eigen; x is not
+                    // normalised here)
+                    const float sc2 = scale * scale * s.xx;
+                    if (s.rr < best * 0.49f) { best = s.rr; stall = 0; } else ++stall;
+                    const bool stop = !(s.rr > 1e-28f * sc2 * (float)n) || it >= kEigMaxIt ||
+                                      (stall >= 4 && s.rr < 1e-22f * sc2);
+                    if (stop && exact) c = 1;
+                    else if (!exact && (stop || s.rr < refresh * sc2)) {
+                        c = 2;
+                        refresh = fminf(refresh, __fdividef(s.rr, fmaxf(sc2, 1e-30f))) * 1e-10f;   // five decades of |r|
+                        if (stop) { best = 3.0e38f; stall = 0; }
+                    }
+                }
+                const bool parallel = s.xw * s.xw > 0.98f * s.xx * s.ww;
+                if (c != 1 && pass == 0 && parallel && s.ww > 0.0f) {
+                    c |= 4;
+                    if (lane == 0) s_y[5] = __fdividef(s.xw, s.xx);
+                } else if (c != 1) {
+                    float mu, yx = 1.0f, yw, yp;
+                    if (!ritz_near(s, have_p, mu, yw, yp)) ritz_full(s, have_p, mu, yx, yw, yp);
+                    // the next p = yw w + yp p: its length, and its part along the new x = yx x + p
+                    const float pn2 = yw * (yw * s.ww + 2.0f * yp * s.wp) + yp * yp * s.pp;
+                    const float xp0 = yx * (yw * s.xw + yp * s.xp);
+                    if (lane == 0) {
+                        s_y[0] = mu; s_y[1] = yx; s_y[2] = yw; s_y[3] = yp;
+                        s_y[4] = pn2 > 0.0f ? rsqrtf(pn2) : 0.0f;
+                        const float xn = yx * yx * s.xx + 2.0f * xp0 + pn2;   // |new x|^2
+                        s_y[5] = __fdividef(xp0 + pn2, xn);
+                        s_y[6] = xn;
+                    }
+                }
+                if (lane == 0) s_ctl = c;
+            }
+            __syncthreads();
+            ctl |= s_ctl;
+            if (!(s_ctl & 4)) break;                    // uniform
+            const float f = s_y[5];
+            wv -= f * xh;
+            __syncthreads();                            // s_ctl, s_y read
+        }
+        if (ctl & 1) break;                             // uniform over the cluster
+        want_exact = (ctl & 2) != 0;
+        const float mu = s_y[0], yx = s_y[1], yw = s_y[2], yp = s_y[3], ip = s_y[4], fx = s_y[5];
+        xxf = s_y[6];
+        // (d) x <- yx x + yw w + yp p, A x likewise; p <- yw w + yp p (unit length) less its part along
+        // x, A p likewise
+        const float np = yw * wv + yp * pv;
+        const float nap = yw * awv + yp * apv;
+        x = ff_add(ff_mul_f(x, yx), ff{np, 0.0f});
+        ax = ff_add(ff_mul_f(ax, yx), ff{nap, 0.0f});
+        theta = ff_add(theta, ff{mu, 0.0f});
+        have_p = ip > 0.0f;
+        pv = (np - fx * x.hi) * ip;
+        apv = (nap - fx * ff_to_float(ax)) * ip;
+    }
+    // 4. z = zs x, zs = sqrt(-lambda / x.x) (float-float); the reduced problem needs lambda < 0
+    //    (theta is the same in every CTA, so all return together)
+    if (!(theta.hi < 0.0f || (theta.hi == 0.0f && theta.lo < 0.0f))) {
+        if (tid == 0 && rank == 0) set_status(st, kErrNotNegative);
+        return;
+    }
+    const ff zq = ff_div(ff_neg(theta), xx);
+    const ff zs_f = ff_mul(zq, ff_rsqrt(zq));
+    if (lead) { xs[2 * ra] = x.hi; xs[2 * ra + 1] = x.lo; }     // this CTA's rows
+    if (tid == 0 && rank == 0) everywhere(&s_x0, [&](ff *p) { *p = x; });
+    sync_all();
+    // sign (Eq. def-z wants gamma >= 0): z_0 >= 0; degenerate or z_0 = 0: z . c_I >= 0, the FP64 dot
+    // taken only then; gamma = z_0 / nu (every CTA the same).  Meanwhile the other warps form
+    // z in FP64, one coordinate per thread.
+    const int ic = a0 + tid - 1;                        // coordinate of this thread (row a0 + tid)
+    const bool coord = tid < nown && ic >= 0;
+    double zc = 0.0, ct = 0.0;
+    if (coord) {
+        zc = ff_to_double(ff{xs[2 * (ic + 1)], xs[2 * (ic + 1) + 1]});
+        ct = cI[ic];
+    }
+    if (tid == blockDim.x - 1) {
+        const ff z0 = deg ? ff{0.0f, 0.0f} : ff_mul(zs_f, s_x0);
+        s_flag = (deg || z0.hi == 0.0f) ? 1 : 0;
+        s_sc[3] = z0.hi < 0.0f ? -1.0 : 1.0;
+        const ff g = ff_mul(ff{fabsf(z0.hi), z0.hi < 0.0f ? -z0.lo : z0.lo}, s_row0[3]);
+        s_sc[4] = deg ? 1.0 : ff_to_double(g);
+        s_sc[5] = ff_to_double(zs_f);
+    }
+    __syncthreads();
+    if (s_flag) {                                       // uniform over the cluster: s_flag agrees
+        double v = zc * ct;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        double *sd = reinterpret_cast<double *>(s_r2[1]);  // the sums' scratch: every reader has passed a barrier
+        if (lane == 0) everywhere(sd, [&](double *p) { p[slot] = v; });
+        sync_all();
+        double dot = 0.0;
+        if (tid == 0) {
+            for (int k = 0; k < ns; ++k) dot += sd[k];
+            s_sc[3] = dot < 0.0 ? -1.0 : 1.0;
+        }
+        __syncthreads();
+    }
+    const double sgn = s_sc[3], gamma = s_sc[4], zs = s_sc[5];
+    const bool bad = !isfinite(gamma) || !(gamma > 1e-200);
+    // 5. eta (Eq. def-z) and the compression thresholds, while the last warp forms the new scale
+    //    s' = s gamma (double-double) and 1 / s'
+    double eta = 0.0, zn = 0.0;
+    if (tid == blockDim.x - 1) {
+        const dd s_new = dd_mul_d(s_sc0, gamma);
+        s_sc[6] = 1.0 / s_new.hi;
+        if (rank == 0) {
+            ms->pend_scale = s_new;
+            ms->pend_gamma = gamma;
+            ms->pend_it = it;
+            ms->pend_deg = deg ? 1 : 0;
+            ms->n_cand = 0;                             // the scatter builds the next candidate list
+            if (bad) set_status(st, kErrNonfinite);
+        }
+    }
+    if (coord) {
+        zn = sgn * (zc * zs);
+        eta = zn - gamma * ct;
+        etaout[ic] = eta;
+        // (without compression no division: 0 / |eta| = 0)
+        thr[ic] = eta != 0.0 ? (P.tau > 0.0 ? P.tau / fabs(eta) : 0.0) : 1.0e308;
     }
     __syncthreads();
     // 6. the scatter weights and the new stored c_I; the change in nonzeros of c
@@ -2375,14 +3000,14 @@ size_t mc_eigen_smem(int m) {
     const int n1 = m + 1;
     const EigCfg g = eig_cfg(n1);
     size_t r;
-    if (g.C == 1) r = 2 * (size_t)n1 * (size_t)eig_ldr(n1);          // R in one CTA
-    else if (g.C > 1) r = 2 * (size_t)g.crows * (size_t)eig_ldr(n1);  // this CTA's rows of R
+    if (g.reg) return ((size_t)g.crows * (size_t)eig_ldr(n1) + 9 * (size_t)eig_len(n1)) * sizeof(float);
+    if (g.C > 1) r = 2 * (size_t)g.crows * (size_t)eig_ldr(n1);  // this CTA's rows of R
     else r = 2 * (size_t)eig_len(n1) + 4 * (size_t)eig_stage_rows(n1) * eig_ldr(n1);   // streamed
     return (r + eig_vec_floats(n1)) * sizeof(float);
 }
 int mc_eigen_threads(int m) {
     const EigCfg g = eig_cfg(m + 1);
-    return g.tpr * 32 * ((g.crows + 31) / 32);
+    return g.reg ? 32 * ((g.tpr * ((g.crows + kRegRows - 1) / kRegRows) + 31) / 32) : g.tpr * 32 * ((g.crows + 31) / 32);
 }
 int mc_eigen_cluster(int m) { return eig_cfg(m + 1).C; }
 int mc_ldr(int m) { return eig_ldr(m + 1); }
@@ -2417,20 +3042,20 @@ McGeom mc_geometry(const Problem &P) {
 }
 
 cudaError_t mc_configure() {
-    size_t most1 = 0, most0 = 0, most_cl = 0;
+    size_t most1 = 0, most4 = 0, most0 = 0, most_cl = 0;
     for (int m = 1; m < kEigMaxN; ++m) {
-        const int C = eig_cfg(m + 1).C;
-        size_t &t = C > 1 ? most_cl : (C == 1 ? most1 : most0);
+        const EigCfg g = eig_cfg(m + 1);
+        size_t &t = g.reg ? (g.C > 1 ? most4 : most1) : (g.C > 1 ? most_cl : most0);
         t = std::max(t, mc_eigen_smem(m));
     }
-    cudaError_t e = cudaFuncSetAttribute(k_mc_eigen<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)most1);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_mc_eigen<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most0);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_mc_eigen<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_cl);
-    if (e != cudaSuccess) return e;
-    return cudaSuccess;
+    auto set = [](auto kernel, size_t bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    cudaError_t e = set(k_mc_eigen_reg<false>, most1);
+    if (e == cudaSuccess) e = set(k_mc_eigen_reg<true>, most4);
+    if (e == cudaSuccess) e = set(k_mc_eigen<false>, most0);
+    if (e == cudaSuccess) e = set(k_mc_eigen<true>, most_cl);
+    return e;
 }
 
 // One matrix element H_{D'D} (Eq. entry; the get_entry / get_diagonal of Sec. "The Hamiltonian Class"):
@@ -2496,32 +3121,28 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
     mark();
     {
         const EigCfg g = eig_cfg(b.m + 1);
-        if (g.C > 1) {                                  // a cluster holding R's rows
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)g.C);
-            cfg.blockDim = dim3((unsigned)mc_eigen_threads(b.m));
-            cfg.dynamicSmemBytes = mc_eigen_smem(b.m);
-            cfg.stream = s;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = (unsigned)g.C;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            cudaLaunchKernelEx(&cfg, k_mc_eigen<true, true>, P, b.ms, b.st, (const McSel *)b.sel,
-                               (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)std::max(g.C, 1));
+        cfg.blockDim = dim3((unsigned)mc_eigen_threads(b.m));
+        cfg.dynamicSmemBytes = mc_eigen_smem(b.m);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)g.C;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = g.C > 1 ? 1 : 0;
+        if (g.reg)
+            cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen_reg<true> : k_mc_eigen_reg<false>, P, b.ms, b.st,
+                               (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
+                               (const double *)b.Hdiag, (const float4 *)b.rowf, (const float *)b.Rh,
+                               (const float *)b.Rl, b.ldr, g.tpr, g.crows, b.w, b.thr, b.eta);
+        else
+            cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen<true> : k_mc_eigen<false>, P, b.ms, b.st,
+                               (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
                                (const double *)b.Hdiag, (const float4 *)b.rowf, b.Rh, b.Rl, b.ldr, g.tpr, g.crows,
                                b.w, b.thr, b.eta);
-        } else if (g.C == 1) {                          // one CTA, R in its shared memory
-            k_mc_eigen<false, true><<<1, mc_eigen_threads(b.m), mc_eigen_smem(b.m), s>>>(
-                P, b.ms, b.st, b.sel, b.cI, b.bI, b.HIIc, b.Hdiag, b.rowf, b.Rh, b.Rl, b.ldr, g.tpr, b.m + 1, b.w,
-                b.thr, b.eta);
-        } else {                                        // one CTA streaming R from L2
-            k_mc_eigen<false, false><<<1, mc_eigen_threads(b.m), mc_eigen_smem(b.m), s>>>(
-                P, b.ms, b.st, b.sel, b.cI, b.bI, b.HIIc, b.Hdiag, b.rowf, b.Rh, b.Rl, b.ldr, g.tpr, b.m + 1, b.w,
-                b.thr, b.eta);
-        }
     }
     mark();
     // one more block than the scatter's own: block 0 updates mu, alpha and the scale meanwhile
