@@ -235,18 +235,18 @@ int setup_block(cdfci_ctx *c, int m) {
     b.geom = mc_geometry(P);
     // grids sized to the problem's work (a small problem leaves the rest of the GPU to the other
     // problems of a batch): the scatter's warps take about two items each, at most the resident
-    // blocks; the candidate passes give every thread at least eight candidates, at most 4 blocks per SM
+    // blocks; the candidate passes give every thread four candidates, at most 4 blocks per SM
     const int resident = mc_scatter_grid(P);
     if (resident <= 0) return fail(CDFCI_ERR_CUDA, "occupancy query of the scatter failed");
     const long long items = (long long)m * b.geom.per_col;
     b.scatter_grid = (int)std::max<long long>(1, std::min<long long>(resident, (items + 15) / 16));
-    b.cand_grid = (int)std::max<long long>(1, std::min<long long>(152 * 4, (cap_cand + 2047) / 2048));
+    b.cand_grid = (int)std::max<long long>(1, std::min<long long>(152 * 4, (cap_cand + 1023) / 1024));
     const size_t ns = (size_t)b.geom.nsA + (size_t)b.geom.nsB;
     b.st = c->d_st;
     const size_t n1 = (size_t)m + 1;
     b.ldr = mc_ldr(m);
     if (mb_alloc(c, &b.ms, 1) || mb_alloc(c, &b.cand, (size_t)cap_cand) || mb_alloc(c, &b.gkey, (size_t)cap_cand) ||
-        mb_alloc(c, &b.hist, 4096 + 1) || mb_alloc(c, &b.sel, (size_t)m) || mb_alloc(c, &b.inbin, 4096) || mb_alloc(c, &b.ties, (size_t)cap_cand) ||
+        mb_alloc(c, &b.hist, 4096 + 2) || mb_alloc(c, &b.selcb, (size_t)m) || mb_alloc(c, &b.sel, (size_t)m) || mb_alloc(c, &b.inbin, 4096) || mb_alloc(c, &b.ties, (size_t)cap_cand) ||
         mb_alloc(c, &b.cI, (size_t)m) || mb_alloc(c, &b.bI, (size_t)m) || mb_alloc(c, &b.Hdiag, (size_t)m) ||
         mb_alloc(c, &b.HIIc, (size_t)m) || mb_alloc(c, &b.Rh, n1 * (size_t)b.ldr) ||
         mb_alloc(c, &b.Rl, n1 * (size_t)b.ldr) ||
@@ -1519,7 +1519,7 @@ CDFCI_API int cdfci_checkpoint(cdfci_handle c, cdfci_checkpoint_header *hdr, uin
         McState ms;
         CK(cudaMemcpyAsync(&ms, c->mb.ms, sizeof(ms), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
-        h.done = ms.done;
+        h.done = ms.done || ms.done_pending ? 1 : 0;
         h.mu[0] = ms.mu.hi; h.mu[1] = ms.mu.lo; h.alpha[0] = ms.alpha.hi; h.alpha[1] = ms.alpha.lo;
         h.scale[0] = ms.scale.hi; h.scale[1] = ms.scale.lo;
         h.dx = ms.dx; h.energy = ms.energy; h.last_gamma = ms.last_gamma;

@@ -3,10 +3,11 @@
 // One iteration is a fixed sequence of kernels (captured once in a CUDA graph):
 //   k_mc_gkeys     |g_j| ~ |b_j + mu c_j| of every candidate (the union of the
 //                  last columns, deduplicated by a mark bit), clearing the marks;
-//   k_mc_hist/scan radix selection of the m largest |g| on the 64-bit pattern,
-//                  16 bits per pass;
-//   k_mc_collect   the candidates above the threshold digit prefix, and the ones
-//                  on it (sorted by (|g| desc, key asc) in k_mc_sortsel);
+//                  a histogram around the last threshold, which nearly always
+//                  finds the bin of the m-th largest;
+//   k_mc_hist      else: radix selection on the 64-bit pattern, 12 bits per pass;
+//   k_mc_select    the candidates above the threshold bin, and the ones on it,
+//                  put in order by (|g| desc, key asc) by its last block;
 //   k_mc_prepare   c_I, b_I, H_II (Slater-Condon between the selected
 //                  determinants) and H_II c_I;
 //   k_mc_eigen     the reduced (m+1)-dimensional problem R = Q^T H Q with
@@ -321,13 +322,19 @@ __device__ __forceinline__ void sym2_lowest(float a00, float a01, float a11, flo
 // ---------------------------------------------------------------------------
 // Candidates and selection (Alg. 2, choice of I): the m largest choice keys
 // |b_j + mu c_j| (the bit pattern of a non-negative double orders like the
-// value), ties to the smaller key.  Radix selection from the top, 12 bits per
-// level (12 x 5 + 4 = 64 bits): a block counts its keys in a shared-memory
-// histogram and adds it to the global one; the last block to finish (a device
-// counter, after a fence) finds the digit holding the key of rank sel_need,
-// narrows the prefix and clears the histogram.  Most selections resolve after
-// one or two levels; later levels return at once.
+// value), ties to the smaller key.  The key of rank m moves little from one
+// iteration to the next, so k_mc_gkeys counts the keys in bins of 1/256 octave
+// (key >> kWinShift) from two octaves below the last threshold upwards: one pass
+// gives the bin of rank m, with a handful of candidates on it, and the mass of
+// candidates below the window is not counted at all.  Where that fails (a first
+// iteration, a jump of the threshold, more than kInBin candidates on the bin) the
+// radix selection of k_mc_hist takes over: from the top, 12 bits per level (12 x
+// 5 + 4 = 64 bits).  In both a block counts in a shared-memory histogram and adds
+// it to the global one; the last block to finish (a device counter, after a
+// fence) finds the bin and clears the histogram.  The choice does not depend on
+// which way found it.
 // ---------------------------------------------------------------------------
+constexpr int kWinShift = 44, kWinBelow = 512;
 constexpr int kSelBins = 4096;
 
 // Candidates in the list: the count, clamped to the list's capacity (a count
@@ -376,69 +383,86 @@ __device__ bool sel_merge(unsigned int *sh, unsigned int *hist, unsigned int *co
     return s_last;
 }
 
-// In the last block: the digit of the key of rank need (1 = largest) among the
-// counted ones; record it, clear the histogram and the counter.
-__device__ void sel_scan(McState *ms, unsigned int *hist, unsigned int *counter, int level, int need) {
+// In the last block (kSelBins / PER threads): the bin of the key of rank need
+// (1 = largest), its count and the count above it, in every thread; false when
+// fewer than need are counted.  Clears the histogram and the counter.  Thread t
+// owns the PER bins from kSelBins - 1 - PER t downwards, in registers.
+template <int PER>
+__device__ bool sel_scan(unsigned int *hist, unsigned int *counter, int need, int &bin, int &count, int &above) {
     __shared__ unsigned int s_warp[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int per = kSelBins / blockDim.x;             // consecutive bins per thread, from the top
-    const int top = kSelBins - 1 - tid * per;
+    __shared__ int s_bin, s_count, s_above;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint4 *own = reinterpret_cast<uint4 *>(hist + kSelBins - PER * (tid + 1));
+    unsigned int v[PER];
     unsigned int loc = 0;
-    for (int q = 0; q < per; ++q) loc += __ldcg(&hist[top - q]);
+#pragma unroll
+    for (int q = 0; q < PER / 4; ++q) {
+        const uint4 x = __ldcg(own + q);
+        v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+        loc += x.x + x.y + x.z + x.w;
+    }
+#pragma unroll
+    for (int q = 0; q < PER / 4; ++q) own[q] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) { *counter = 0u; s_bin = -1; }
     // exclusive prefix of loc over threads (thread 0 owns the largest digits)
     unsigned int inc = loc;
     for (int off = 1; off < 32; off <<= 1) {
-        const unsigned int v = __shfl_up_sync(0xffffffffu, inc, off);
-        if (lane >= off) inc += v;
+        const unsigned int u = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += u;
     }
     if (lane == 31) s_warp[warp] = inc;
     __syncthreads();
-    unsigned int base = 0;
-    for (int w = 0; w < warp; ++w) base += s_warp[w];
-    const unsigned int before = base + inc - loc;
+    unsigned int before = inc - loc;
+    for (int w = 0; w < warp; ++w) before += s_warp[w];
     if (before < (unsigned int)need && (unsigned int)need <= before + loc) {
         unsigned int acc = before;
-        for (int q = 0; q < per; ++q) {
-            const unsigned int c = __ldcg(&hist[top - q]);
-            if (acc + c >= (unsigned int)need) {
-                ms->sel_prefix = (ms->sel_prefix << sel_bits(level)) | (unsigned long long)(top - q);
-                ms->sel_need = need - (int)acc;
-                ms->sel_level = level + 1;
-                ms->sel_nbin = (int)c;
-                ms->sel_resolved = (c <= (unsigned int)kInBin || level == kSelLevels - 1) ? 1 : 0;
-                break;
+        bool found = false;
+#pragma unroll
+        for (int q = PER - 1; q >= 0; --q) {
+            if (!found && acc + v[q] >= (unsigned int)need) {
+                s_bin = kSelBins - PER * (tid + 1) + q;
+                s_count = (int)v[q];
+                s_above = (int)acc;
+                found = true;
             }
-            acc += c;
+            acc += v[q];
         }
     }
-    (void)nw;
     __syncthreads();
-    for (int q = 0; q < per; ++q) hist[top - q] = 0u;
-    if (tid == 0) *counter = 0u;
+    bin = s_bin; count = s_count; above = s_above;
+    return s_bin >= 0;
 }
 
-// choice keys of the candidates, clearing their marks; level-0 histogram
+// choice keys of the candidates, clearing their marks; the histogram around the last threshold
 __global__ void __launch_bounds__(256) k_mc_gkeys(Problem P, McState *ms, IterState *st, const long long *cand,
                                                   unsigned long long *gkey, unsigned int *hist, int m) {
     __shared__ unsigned int sh[kSelBins];
     if (ms->done) return;
+    if (ms->done_pending) {                            // the stopping rule was met in the last iteration
+        if (blockIdx.x == 0 && threadIdx.x == 0) ms->done = 1;
+        return;
+    }
     const int n = mc_ncand(ms, P.cap_cand);
     const double mu = ms->mu.hi;
-    const bool count = n > m;
-    for (int d = threadIdx.x; d < kSelBins; d += blockDim.x) sh[d] = 0u;
-    __syncthreads();
+    const int hint = ms->sel_hint;
+    const bool count = n > m, win = count && hint > 0;
+    const int base = max(hint - kWinBelow, 0);
+    if (win) {
+        for (int d = threadIdx.x; d < kSelBins / 4; d += blockDim.x) reinterpret_cast<uint4 *>(sh)[d] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    }
     const int stride = gridDim.x * blockDim.x;
     unsigned long long pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     // kGkU candidates per thread and round, all their slot loads in flight together
     constexpr int kGkU = 4;
-    for (int base = blockIdx.x * blockDim.x; base < n; base += kGkU * stride) {
+    for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += kGkU * stride) {
         long long slot[kGkU];
         bool ok[kGkU];
         double2 v[kGkU];
 #pragma unroll
         for (int u = 0; u < kGkU; ++u) {
-            const int t = base + u * stride + threadIdx.x;
+            const int t = b0 + u * stride + threadIdx.x;
             ok[u] = t < n;
             slot[u] = ok[u] ? cand[t] : 0;
         }
@@ -452,7 +476,7 @@ __global__ void __launch_bounds__(256) k_mc_gkeys(Problem P, McState *ms, IterSt
         }
 #pragma unroll
         for (int u = 0; u < kGkU; ++u) {
-            const int t = base + u * stride + threadIdx.x;
+            const int t = b0 + u * stride + threadIdx.x;
             unsigned long long k = 0ull;
             if (ok[u] && (unsigned long long)slot[u] >= (unsigned long long)P.capacity) {
                 set_status(st, kErrInternal);              // a candidate outside the table: skip it
@@ -462,40 +486,48 @@ __global__ void __launch_bounds__(256) k_mc_gkeys(Problem P, McState *ms, IterSt
                 gkey[t] = k;
                 mark_clear(P, slot[u]);                    // clear the candidate mark
             }
-            if (count) sel_bin_add(sh, ok[u], sel_digit(k, 0));
+            if (win) {                                     // bin 0 and below: not counted
+                const int d = (int)(k >> kWinShift) - base;
+                sel_bin_add(sh, ok[u] && d > 0, (unsigned int)min(d, kSelBins - 1));
+            }
         }
     }
-    if (!count) {                                      // every candidate is chosen
+    if (!win) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             ms->sel_prefix = 0ull;
-            ms->sel_need = 0;
-            ms->sel_level = 0;
-            ms->sel_nbin = 0;
-            ms->sel_resolved = 1;
+            ms->sel_need = count ? m : 0;
+            ms->sel_shift = 64;                            // (not counted: every candidate is chosen)
+            ms->sel_resolved = count ? 0 : 1;
+            if (!count) ms->sel_hint = 0;
         }
         return;
     }
     if (sel_merge(sh, hist, hist + kSelBins)) {
-        if (threadIdx.x == 0) ms->sel_prefix = 0ull;
-        __syncthreads();
-        sel_scan(ms, hist, hist + kSelBins, 0, m);
+        int bin, c, above;
+        const bool found = sel_scan<kSelBins / 256>(hist, hist + kSelBins, m, bin, c, above);
+        if (threadIdx.x == 0) {
+            // the top bin also holds everything above the window
+            const bool good = found && c <= kInBin && bin < kSelBins - 1;
+            ms->sel_prefix = good ? (unsigned long long)(base + bin) : 0ull;
+            ms->sel_need = good ? m - above : m;
+            ms->sel_shift = good ? kWinShift : 64;
+            ms->sel_resolved = good ? 1 : 0;
+        }
     }
 }
 
-// Levels 2.. by the block that finished level 1 (1024 threads): it stops at once
-// when the selection is resolved, which is the common case; otherwise it counts
-// the keys on the prefix in a shared-memory histogram and scans it, level by
-// level, exactly as the level-1 pass and sel_scan do.
-__device__ void mc_hist_tail(McState *ms, const unsigned long long *gkey, long long cap, unsigned int *sh) {
+// Levels 1.. by the block that finished level 0 (1024 threads): it counts the
+// keys on the prefix in a shared-memory histogram and scans it, level by level,
+// until the selection is resolved.
+__device__ void mc_hist_tail(McState *ms, const unsigned long long *gkey, int n, unsigned int *sh) {
     __shared__ unsigned int s_warp[32];
     __shared__ int s_stop;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int level = 2; level < kSelLevels; ++level) {
-        if (tid == 0) s_stop = (ms->done || ms->sel_resolved) ? 1 : 0;
+    for (int level = 1; level < kSelLevels; ++level) {
+        if (tid == 0) s_stop = ms->sel_resolved;
         for (int d = tid; d < kSelBins; d += blockDim.x) sh[d] = 0u;
         __syncthreads();
         if (s_stop) return;                               // uniform
-        const int n = mc_ncand(ms, cap);
         const unsigned long long prefix = ms->sel_prefix;
         const int need = ms->sel_need;
         for (int base = 0; base < n; base += blockDim.x) {
@@ -526,8 +558,7 @@ __device__ void mc_hist_tail(McState *ms, const unsigned long long *gkey, long l
                 if (acc + c >= (unsigned int)need) {
                     ms->sel_prefix = (ms->sel_prefix << sel_bits(level)) | (unsigned long long)(top - q);
                     ms->sel_need = need - (int)acc;
-                    ms->sel_level = level + 1;
-                    ms->sel_nbin = (int)c;
+                    ms->sel_shift = 64 - sel_cover(level + 1);
                     ms->sel_resolved = (c <= (unsigned int)kInBin || level == kSelLevels - 1) ? 1 : 0;
                     break;
                 }
@@ -539,62 +570,36 @@ __device__ void mc_hist_tail(McState *ms, const unsigned long long *gkey, long l
     }
 }
 
-// level 1 on the grid: the keys on the level-0 prefix; the last block to merge
-// its histogram scans it and goes on with the levels below (mc_hist_tail)
+// The radix selection where the window did not resolve the choice: level 0 on
+// the grid; the last block to merge its histogram scans it and goes on with the
+// levels below (mc_hist_tail)
 constexpr int kHistThreads = 1024;
 __global__ void __launch_bounds__(kHistThreads) k_mc_hist(McState *ms, const unsigned long long *gkey,
                                                           unsigned int *hist, long long cap) {
     __shared__ unsigned int sh[kSelBins];
-    const int level = 1;
     if (ms->done || ms->sel_resolved) return;
     const int n = mc_ncand(ms, cap);
-    const unsigned long long prefix = ms->sel_prefix;
     const int need = ms->sel_need;
     for (int d = threadIdx.x; d < kSelBins; d += blockDim.x) sh[d] = 0u;
     __syncthreads();
     const int stride = gridDim.x * blockDim.x;
     for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
         const int t = base + threadIdx.x;
-        unsigned long long k = t < n ? gkey[t] : 0ull;
-        const bool ok = t < n && sel_top(k, level) == prefix;
-        sel_bin_add(sh, ok, sel_digit(k, level));
+        const unsigned long long k = t < n ? gkey[t] : 0ull;
+        sel_bin_add(sh, t < n, sel_digit(k, 0));
     }
     if (sel_merge(sh, hist, hist + kSelBins)) {
-        sel_scan(ms, hist, hist + kSelBins, level, need);
+        int bin, c, above;
+        sel_scan<kSelBins / kHistThreads>(hist, hist + kSelBins, need, bin, c, above);
+        if (threadIdx.x == 0) {
+            ms->sel_prefix = (unsigned long long)bin;
+            ms->sel_need = need - above;
+            ms->sel_shift = 64 - sel_cover(1);
+            ms->sel_resolved = c <= kInBin ? 1 : 0;
+        }
         __threadfence_block();
         __syncthreads();                                // the scan's McState fields visible to the block
-        mc_hist_tail(ms, gkey, cap, sh);
-    }
-}
-
-__global__ void k_mc_collect(Problem P, McState *ms, const long long *cand, const unsigned long long *gkey,
-                             McSel *sel, McSel *inbin) {
-    if (ms->done) return;
-    const int n = mc_ncand(ms, P.cap_cand);
-    const bool all = ms->sel_level == 0;                 // n_cand <= m: every candidate is selected
-    const int L = ms->sel_level;
-    const unsigned long long prefix = ms->sel_prefix;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const unsigned long long k = gkey[t];
-        const unsigned long long top = sel_top(k, L);
-        McSel x;
-        x.slot = cand[t];
-        x.gkey = k;
-        if (all || top > prefix) {
-            const int pos = atomicAdd(&ms->n_above, 1);
-            const Slot s = P.table[x.slot];
-            x.A = s.a;
-            x.B = s.b & kKeyMaskB;
-            sel[pos] = x;
-        } else if (top == prefix) {
-            const int pos = atomicAdd(&ms->n_inbin, 1);
-            if (pos < kInBin) {
-                const Slot s = P.table[x.slot];
-                x.A = s.a;
-                x.B = s.b & kKeyMaskB;
-                inbin[pos] = x;
-            }
-        }
+        mc_hist_tail(ms, gkey, n, sh);
     }
 }
 
@@ -676,7 +681,7 @@ __device__ void mc_ties(const Problem &P, McState *ms, const long long *cand, co
         }
     __syncthreads();
     if (tid == 0) ms->n_inbin = s_out;                 // = sel_need
-    __threadfence_block();
+    __threadfence();
     __syncthreads();
 }
 
@@ -720,43 +725,95 @@ __device__ void rank_sort(const SelE *buf, int n, unsigned int *rank) {
     __syncthreads();
 }
 
-// The in-bin candidates put in order (after the exact-tie pass when more than
-// kInBin share the whole 64-bit choice key), the first sel_need of them join the
-// chosen set; then the chosen set in the choice order (a canonical order for
-// the reduced problem's rows).  The candidates above the threshold digit all
-// precede the in-bin ones, so each of the two sets is ordered by itself.
-// 1024 threads, one element each.
-__global__ void __launch_bounds__(1024) k_mc_sortsel(Problem P, McState *ms, McSel *sel, McSel *inbin, int m,
-                                                      IterState *st, const long long *cand,
-                                                      const unsigned long long *gkey, McSel *ties) {
+__device__ __forceinline__ McSel ld_sel(const McSel *p) {    // written by other SMs in this launch: through L2
+    const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(p);
+    const ulonglong2 x = __ldcg(q), y = __ldcg(q + 1);
+    return McSel{(long long)x.x, x.y, y.x, y.y};
+}
+
+// The chosen set in the choice order (a canonical order for the reduced
+// problem's rows).  Every block appends its candidates above the threshold bin
+// to sel and the ones on it to inbin; the last block to finish puts both in
+// order (after the exact-tie pass when more than kInBin share the whole 64-bit
+// choice key): the ones above all precede the in-bin ones, so each set is
+// ordered by itself, and the first sel_need of the in-bin ones join.  It also
+// reads c and b of the chosen slots (as stored) for k_mc_prepare, and leaves the
+// threshold for the next iteration's window.  1024 threads, one element each.
+constexpr int kSelThreads = 1024;
+__global__ void __launch_bounds__(kSelThreads) k_mc_select(Problem P, McState *ms, IterState *st, const long long *cand,
+                                                           const unsigned long long *gkey, McSel *sel, McSel *inbin,
+                                                           McSel *ties, double2 *selcb, unsigned int *counter) {
     __shared__ SelE buf[kInBin];
     __shared__ unsigned int rank[kInBin];
     __shared__ int s_keep, s_digit;
+    __shared__ bool s_last;
     const int tid = threadIdx.x;
     if (ms->done) return;
-    if (ms->sel_level >= kSelLevels && ms->n_inbin > kInBin) mc_ties(P, ms, cand, gkey, ties, inbin);   // uniform
-    const int n_above = ms->n_above;
-    int n_in = ms->n_inbin;
-    if (ms->sel_level > 0 && n_in > kInBin) {
+    const int shift = ms->sel_shift, need = ms->sel_need;
+    const bool all = shift == 64;                        // n_cand <= m: every candidate is selected
+    {
+        const int n = mc_ncand(ms, P.cap_cand);
+        const unsigned long long prefix = ms->sel_prefix;
+        for (int t = blockIdx.x * blockDim.x + tid; t < n; t += gridDim.x * blockDim.x) {
+            const unsigned long long k = gkey[t], top = all ? 0ull : k >> shift;
+            if (!all && top < prefix) continue;
+            McSel x;
+            x.slot = cand[t];
+            x.gkey = k;
+            McSel *to = nullptr;
+            if (all || top > prefix) {
+                to = sel + atomicAdd(&ms->n_above, 1);
+            } else {
+                const int pos = atomicAdd(&ms->n_inbin, 1);
+                if (pos < kInBin) to = inbin + pos;
+            }
+            if (to) {
+                const ulonglong2 key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + x.slot));
+                x.A = key.x;
+                x.B = key.y & kKeyMaskB;
+                *to = x;
+            }
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) *counter = 0u;
+    if (shift == 0 && __ldcg(&ms->n_inbin) > kInBin) mc_ties(P, ms, cand, gkey, ties, inbin);   // uniform
+    const int n_above = __ldcg(&ms->n_above);
+    int n_in = __ldcg(&ms->n_inbin);
+    if (!all && n_in > kInBin) {
         if (tid == 0) set_status(st, kErrArg);            // more than kInBin candidates with one key pattern
         n_in = kInBin;
     }
-    const int need = ms->sel_level == 0 ? 0 : ms->sel_need;
-    const int take = need < n_in ? need : n_in;
+    const int take = all ? 0 : min(need, n_in);
+    const int msel = n_above + take;
     SelE e{0ull, 0ull, 0ull, -1}, f = e;
-    if (tid < n_above) { const McSel x = sel[tid]; e = SelE{x.gkey, x.A, x.B, x.slot}; }
-    if (take > 0 && tid < n_in) { const McSel x = inbin[tid]; f = SelE{x.gkey, x.A, x.B, x.slot}; }
-    if (tid < n_above) buf[tid] = e;
+    double2 ecb = make_double2(0.0, 0.0);
+    if (tid < n_above) {
+        const McSel x = ld_sel(sel + tid);
+        e = SelE{x.gkey, x.A, x.B, x.slot};
+        ecb = __ldcg(reinterpret_cast<const double2 *>(&P.table[x.slot].c));
+        buf[tid] = e;
+    }
+    if (take > 0 && tid < n_in) { const McSel x = ld_sel(inbin + tid); f = SelE{x.gkey, x.A, x.B, x.slot}; }
     rank_sort(buf, n_above, rank);
-    if (tid < n_above) sel[rank[tid]] = McSel{e.slot, e.g, e.A, e.B};
+    if (tid < n_above) {
+        const unsigned int r = rank[tid];
+        sel[r] = McSel{e.slot, e.g, e.A, e.B};
+        selcb[r] = ecb;
+        if (!all && (int)r == msel - 1) ms->sel_hint = (int)(e.g >> kWinShift);
+    }
     if (take > 0) {                                     // uniform
         __syncthreads();                                // rank read
         // many more than are needed: one 8-bit digit below the selection's prefix first, so that only the
         // ones at or above the digit of rank `take` are ordered
         bool keep = tid < n_in;
-        const int low = 64 - sel_cover(ms->sel_level);  // bits the prefix leaves open
-        if (n_in > take + 64 && low >= 8) {             // uniform
-            const unsigned int dg = (unsigned int)(f.g >> (low - 8)) & 0xffu;
+        if (n_in > take + 64 && shift >= 8) {           // uniform
+            const unsigned int dg = (unsigned int)(f.g >> (shift - 8)) & 0xffu;
             if (tid < 256) rank[tid] = 0u;
             if (tid == 0) s_keep = 0;
             __syncthreads();
@@ -788,10 +845,15 @@ __global__ void __launch_bounds__(1024) k_mc_sortsel(Problem P, McState *ms, McS
             buf[tid] = f;
         }
         rank_sort(buf, n_in, rank);
-        if (tid < n_in && (int)rank[tid] < take) sel[n_above + rank[tid]] = McSel{f.slot, f.g, f.A, f.B};
+        if (tid < n_in && (int)rank[tid] < take) {
+            const int r = n_above + (int)rank[tid];
+            sel[r] = McSel{f.slot, f.g, f.A, f.B};
+            selcb[r] = __ldcg(reinterpret_cast<const double2 *>(&P.table[f.slot].c));
+            if (r == msel - 1) ms->sel_hint = (int)(f.g >> kWinShift);
+        }
     }
     if (tid == 0) {
-        ms->m_sel = n_above + take;
+        ms->m_sel = msel;
         ms->n_above = 0;
         ms->n_inbin = 0;
     }
@@ -829,7 +891,8 @@ __device__ __forceinline__ void mc_build_coltab(const Problem &P, const ColLists
 // ---------------------------------------------------------------------------
 constexpr int kPrepWarps = 8;       // rows (warps) per block
 
-__global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McState *ms, const McSel *sel, double *cI,
+__global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McState *ms, const McSel *sel,
+                                                    const double2 *selcb, double *cI,
                                                     double *bI, double *Hdiag, double *HIIc, float4 *rowf, float *Rh,
                                                     float *Rl, int ldr, ColEnt *coltab, ColLists *collists, int ns) {
     __shared__ ColLists Lw[kPrepWarps];
@@ -844,12 +907,12 @@ __global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McSta
         const McSel x = sel[i];
         s_A[i] = x.A;
         s_B[i] = x.B;
-        s_c[i] = P.table[x.slot].c * s;
+        s_c[i] = selcb[i].x * s;
     }
     __syncthreads();
     for (int r = blockIdx.x * kPrepWarps + warp; r < m; r += gridDim.x * kPrepWarps) {
         const unsigned long long rA = s_A[r], rB = s_B[r];
-        const double b_r = lane == 0 ? P.table[sel[r].slot].bv : 0.0;     // issued early: a random slot
+        const double b_r = selcb[r].y;
         ColLists &L = Lw[warp];
         for (int t = lane; t < P.N; t += 32) {
             int ra = __popcll(rA & low_mask(t)), rb = __popcll(rB & low_mask(t));
@@ -882,7 +945,7 @@ __global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McSta
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
         // the row's values, and for the reduced solve c_r, b_r, (H_II c_I)_r, b_r - (H_II c_I)_r as
         // float-float pairs (lanes 0..3, one conversion each)
-        const double hc = __shfl_sync(0xffffffffu, acc, 0), br = __shfl_sync(0xffffffffu, b_r, 0) * s;
+        const double hc = __shfl_sync(0xffffffffu, acc, 0), br = b_r * s;
         if (lane == 0) {
             cI[r] = s_c[r];
             bI[r] = br;
@@ -3111,12 +3174,13 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
     mark();
     k_mc_hist<<<(b.cand_grid + 3) / 4, kHistThreads, 0, s>>>(b.ms, b.gkey, b.hist, b.cap_cand);
     mark();
-    k_mc_collect<<<b.cand_grid, 256, 0, s>>>(P, b.ms, b.cand, b.gkey, b.sel, b.inbin);
+    // (one launch in the places of a collecting and a sorting one: the second reads as zero)
+    k_mc_select<<<(b.cand_grid + 3) / 4, kSelThreads, 0, s>>>(P, b.ms, b.st, b.cand, b.gkey, b.sel, b.inbin, b.ties, b.selcb,
+                                                            b.hist + kSelBins + 1);
     mark();
-    k_mc_sortsel<<<1, 1024, 0, s>>>(P, b.ms, b.sel, b.inbin, b.m, b.st, b.cand, b.gkey, b.ties);
     mark();
     k_mc_prepare<<<(b.m + kPrepWarps - 1) / kPrepWarps, 32 * kPrepWarps, 0, s>>>(
-        P, b.ms, b.sel, b.cI, b.bI, b.Hdiag, b.HIIc, b.rowf, b.Rh, b.Rl, b.ldr, b.coltab, b.collists,
+        P, b.ms, b.sel, b.selcb, b.cI, b.bI, b.Hdiag, b.HIIc, b.rowf, b.Rh, b.Rl, b.ldr, b.coltab, b.collists,
         b.geom.nsA + b.geom.nsB);
     mark();
     {

@@ -145,9 +145,10 @@ struct McState {
     double dx, energy, last_gamma;
     long long iterations, nnz_c, n_slots, elements, applied, dropped, inserted, last_column;
     unsigned long long cnt[4];     // counters of the running scatter
-    unsigned long long sel_prefix; // radix selection: digits fixed so far
+    unsigned long long sel_prefix; // selection: the threshold bin, key >> sel_shift
     int n_cand, m_sel, degenerate, done, done_pending;
-    int sel_need, sel_level, sel_nbin, sel_resolved;
+    int sel_need, sel_shift, sel_resolved;
+    int sel_hint;                  // key >> 44 of the last iteration's threshold (0: none)
     int n_above, n_inbin;
     int eig_iters;                 // LOBPCG iterations of the last reduced problem
     long long eig_iters_total;

@@ -87,7 +87,8 @@ struct McBuffers {
     IterState *st;
     long long *cand;               // candidate slots (deduplicated)
     unsigned long long *gkey;      // their choice keys
-    unsigned int *hist;            // 4096-bin radix histogram, then the last-block counter
+    unsigned int *hist;            // 4096-bin histogram, then two last-block counters
+    double2 *selcb;                // c and b of the chosen slots, as stored
     McSel *sel, *inbin, *ties;     // chosen set, threshold-digit candidates, exact-tie scratch
     double *cI, *bI, *Hdiag, *HIIc, *w, *thr, *eta, *gathp;   // gathp: m x geom.per_col item partials
     float4 *rowf;                  // per chosen row: (c, b), (H_II c_I, b - H_II c_I) as float-float pairs
