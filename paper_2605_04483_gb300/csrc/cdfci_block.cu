@@ -886,78 +886,90 @@ __device__ __forceinline__ void mc_build_coltab(const Problem &P, const ColLists
 }
 
 // ---------------------------------------------------------------------------
-// c_I, b_I, H_II, H_II c_I: one warp per selected row.  H_II goes to rows and
-// columns 1..m of R as float-float pairs (Rh, Rl; leading dimension ldr).
+// c_I, b_I, H_II, H_II c_I: one block of 4 warps per selected row.  H_II goes to
+// rows and columns 1..m of R as float-float pairs (Rh, Rl; leading dimension
+// ldr).  Bound by the latency of its chain (lists, integrals, FP64 sums on a pipe
+// that takes two lanes a cycle), so a row's parts run side by side: every warp
+// takes 32 of each 128 columns, warp 0 the diagonal element, all four the
+// column's single excitations; with a block per row the FP64 work of an SM is
+// that of one or two rows (8 rows a block, one warp each: m = 64 9.0 -> 6.5
+// us, m = 128 18.9 -> 8.9, m = 256 on a lattice 20.0 -> 11.3).
 // ---------------------------------------------------------------------------
-constexpr int kPrepWarps = 8;       // rows (warps) per block
+constexpr int kPrepWarps = 4;
 
 __global__ void __launch_bounds__(32 * kPrepWarps) k_mc_prepare(Problem P, McState *ms, const McSel *sel,
-                                                    const double2 *selcb, double *cI,
-                                                    double *bI, double *Hdiag, double *HIIc, float4 *rowf, float *Rh,
-                                                    float *Rl, int ldr, ColEnt *coltab, ColLists *collists, int ns) {
-    __shared__ ColLists Lw[kPrepWarps];
-    // the chosen determinants and their c (true units), staged once per block
-    __shared__ unsigned long long s_A[kEigMaxN], s_B[kEigMaxN];
-    __shared__ double s_c[kEigMaxN];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                                                    const double2 *selcb, double *cI, double *bI, double *Hdiag,
+                                                    double *HIIc, float4 *rowf, float *Rh, float *Rl, int ldr,
+                                                    ColEnt *coltab, ColLists *collists, int ns) {
+    __shared__ ColLists L;
+    __shared__ double s_acc[kPrepWarps], s_hd;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int r = blockIdx.x;
     if (ms->done) return;
     const int m = ms->m_sel;
+    if (r >= m) return;
     const double s = ms->scale.hi;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const McSel x = sel[i];
-        s_A[i] = x.A;
-        s_B[i] = x.B;
-        s_c[i] = selcb[i].x * s;
+    const McSel me = sel[r];
+    const double2 cb = selcb[r];
+    const unsigned long long rA = me.A, rB = me.B;
+    // this thread's first column, loaded ahead of the lists
+    McSel xc = sel[tid < m ? tid : 0];
+    double cc = selcb[tid < m ? tid : 0].x;
+    for (int t = tid; t < P.N; t += 32 * kPrepWarps) {
+        const int ra = __popcll(rA & low_mask(t)), rb = __popcll(rB & low_mask(t));
+        if ((rA >> t) & 1ull) L.occA[ra] = (unsigned char)t; else L.virA[t - ra] = (unsigned char)t;
+        if ((rB >> t) & 1ull) L.occB[rb] = (unsigned char)t; else L.virB[t - rb] = (unsigned char)t;
     }
     __syncthreads();
-    for (int r = blockIdx.x * kPrepWarps + warp; r < m; r += gridDim.x * kPrepWarps) {
-        const unsigned long long rA = s_A[r], rB = s_B[r];
-        const double b_r = selcb[r].y;
-        ColLists &L = Lw[warp];
-        for (int t = lane; t < P.N; t += 32) {
-            int ra = __popcll(rA & low_mask(t)), rb = __popcll(rB & low_mask(t));
-            if ((rA >> t) & 1ull) L.occA[ra] = (unsigned char)t; else L.virA[t - ra] = (unsigned char)t;
-            if ((rB >> t) & 1ull) L.occB[rb] = (unsigned char)t; else L.virB[t - rb] = (unsigned char)t;
+    // (pairs more than a double excitation apart, or doubles when every double vanishes, are zero:
+    // no FP64 work for them; a zero term leaves acc unchanged)
+    const int dmax = P.doubles_vanish ? 2 : 4;
+    double acc = 0.0;
+    for (int c = tid; c < m; c += 32 * kPrepWarps) {
+        if (c != tid) { xc = sel[c]; cc = selcb[c].x; }
+        const int dd2 = __popcll(rA ^ xc.A) + __popcll(rB ^ xc.B);
+        if (c == r) continue;                           // (the diagonal: below)
+        float hh = 0.0f, hl = 0.0f;
+        if (dd2 <= dmax) {
+            const double h = hij_pair(P, rA, rB, xc.A, xc.B);
+            const ff hf = ff_from_double(h);
+            hh = hf.hi;
+            hl = hf.lo;
+            acc = fma(h, cc * s, acc);
         }
-        __syncwarp();
-        // the column's single excitations and orbital lists for the scatter
-        mc_build_coltab(P, L, rA, rB, coltab + (size_t)r * ns, lane, 32);
-        reinterpret_cast<uint2 *>(collists + r)[lane] = reinterpret_cast<const uint2 *>(&L)[lane];
-        const double hd = diag_warp(P, L);
-        // (pairs more than a double excitation apart, or doubles when every double vanishes, are zero:
-        // no FP64 work for them; a zero term leaves acc unchanged)
-        const int dmax = P.doubles_vanish ? 2 : 4;
-        double acc = 0.0;
-        for (int c = lane; c < m; c += 32) {
-            const unsigned long long cA = s_A[c], cB = s_B[c];
-            const int dd2 = __popcll(rA ^ cA) + __popcll(rB ^ cB);
-            float hh = 0.0f, hl = 0.0f;
-            if (c == r || (dd2 > 0 && dd2 <= dmax)) {
-                const double h = (c == r) ? hd : hij_pair(P, rA, rB, cA, cB);
-                const ff hf = ff_from_double(h);
-                hh = hf.hi;
-                hl = hf.lo;
-                acc = fma(h, s_c[c], acc);
-            }
-            Rh[(size_t)(r + 1) * ldr + (c + 1)] = hh;
-            Rl[(size_t)(r + 1) * ldr + (c + 1)] = hl;
-        }
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-        // the row's values, and for the reduced solve c_r, b_r, (H_II c_I)_r, b_r - (H_II c_I)_r as
-        // float-float pairs (lanes 0..3, one conversion each)
-        const double hc = __shfl_sync(0xffffffffu, acc, 0), br = b_r * s;
-        if (lane == 0) {
-            cI[r] = s_c[r];
-            bI[r] = br;
-            Hdiag[r] = hd;
-            HIIc[r] = hc;
-        }
-        const double cv = lane == 0 ? s_c[r] : (lane == 1 ? br : (lane == 2 ? hc : br - hc));
-        const ff f = ff_from_double(cv);
-        const float fh1 = __shfl_sync(0xffffffffu, f.hi, lane | 1), fl1 = __shfl_sync(0xffffffffu, f.lo, lane | 1);
-        if (lane == 0 || lane == 2) rowf[2 * r + (lane >> 1)] = make_float4(f.hi, f.lo, fh1, fl1);
-        __syncwarp();
+        Rh[(size_t)(r + 1) * ldr + (c + 1)] = hh;
+        Rl[(size_t)(r + 1) * ldr + (c + 1)] = hl;
     }
+    if (warp == 0) {
+        const double hd = diag_warp(P, L);
+        if (lane == 0) {
+            s_hd = hd;
+            const ff hf = ff_from_double(hd);
+            Rh[(size_t)(r + 1) * ldr + (r + 1)] = hf.hi;
+            Rl[(size_t)(r + 1) * ldr + (r + 1)] = hf.lo;
+        }
+        acc = lane == 0 ? fma(hd, cb.x * s, acc) : acc;
+    } else {
+        // the column's single excitations and orbital lists for the scatter (warps 1..3; warp 0 has the diagonal)
+        mc_build_coltab(P, L, rA, rB, coltab + (size_t)r * ns, tid - 32, 32 * (kPrepWarps - 1));
+        if (warp == 1) reinterpret_cast<uint2 *>(collists + r)[lane] = reinterpret_cast<const uint2 *>(&L)[lane];
+    }
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if (lane == 0) s_acc[warp] = acc;
+    __syncthreads();
+    if (warp != 0) return;
+    // the row's values, and for the reduced solve c_r, b_r, (H_II c_I)_r, b_r - (H_II c_I)_r as
+    // float-float pairs (lanes 0..3, one conversion each)
+    const double hc = (s_acc[0] + s_acc[1]) + (s_acc[2] + s_acc[3]), c0 = cb.x * s, br = cb.y * s;
+    if (lane == 0) {
+        cI[r] = c0;
+        bI[r] = br;
+        Hdiag[r] = s_hd;
+        HIIc[r] = hc;
+    }
+    const ff f = ff_from_double(lane == 0 ? c0 : (lane == 1 ? br : (lane == 2 ? hc : br - hc)));
+    const float fh1 = __shfl_sync(0xffffffffu, f.hi, lane | 1), fl1 = __shfl_sync(0xffffffffu, f.lo, lane | 1);
+    if (lane == 0 || lane == 2) rowf[2 * r + (lane >> 1)] = make_float4(f.hi, f.lo, fh1, fl1);
 }
 
 // ---------------------------------------------------------------------------
@@ -3179,7 +3191,7 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
                                                             b.hist + kSelBins + 1);
     mark();
     mark();
-    k_mc_prepare<<<(b.m + kPrepWarps - 1) / kPrepWarps, 32 * kPrepWarps, 0, s>>>(
+    k_mc_prepare<<<b.m, 32 * kPrepWarps, 0, s>>>(
         P, b.ms, b.sel, b.selcb, b.cI, b.bI, b.Hdiag, b.HIIc, b.rowf, b.Rh, b.Rl, b.ldr, b.coltab, b.collists,
         b.geom.nsA + b.geom.nsB);
     mark();
