@@ -234,12 +234,12 @@ int setup_block(cdfci_ctx *c, int m) {
     CK(mc_configure());
     b.geom = mc_geometry(P);
     // grids sized to the problem's work (a small problem leaves the rest of the GPU to the other
-    // problems of a batch): the scatter's warps take about two items each, at most the resident
-    // blocks; the candidate passes give every thread four candidates, at most 4 blocks per SM
+    // problems of a batch): the scatter has a warp per work item, at most the resident blocks (two
+    // items a warp: 3 us more of 30 at m = 64, N = 12); the candidate passes give every thread four candidates, at most 4 blocks per SM
     const int resident = mc_scatter_grid(P);
     if (resident <= 0) return fail(CDFCI_ERR_CUDA, "occupancy query of the scatter failed");
     const long long items = (long long)m * b.geom.per_col;
-    b.scatter_grid = (int)std::max<long long>(1, std::min<long long>(resident, (items + 15) / 16));
+    b.scatter_grid = (int)std::max<long long>(1, std::min<long long>(resident, (items + 7) / 8));
     b.cand_grid = (int)std::max<long long>(1, std::min<long long>(152 * 4, (cap_cand + 1023) / 1024));
     const size_t ns = (size_t)b.geom.nsA + (size_t)b.geom.nsB;
     b.st = c->d_st;

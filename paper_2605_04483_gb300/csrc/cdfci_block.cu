@@ -436,7 +436,7 @@ __device__ bool sel_scan(unsigned int *hist, unsigned int *counter, int need, in
 // choice keys of the candidates, clearing their marks; the histogram around the last threshold
 __global__ void __launch_bounds__(256) k_mc_gkeys(Problem P, McState *ms, IterState *st, const long long *cand,
                                                   unsigned long long *gkey, unsigned int *hist, int m) {
-    __shared__ unsigned int sh[kSelBins];
+    __shared__ __align__(16) unsigned int sh[kSelBins];
     if (ms->done) return;
     if (ms->done_pending) {                            // the stopping rule was met in the last iteration
         if (blockIdx.x == 0 && threadIdx.x == 0) ms->done = 1;
@@ -576,7 +576,7 @@ __device__ void mc_hist_tail(McState *ms, const unsigned long long *gkey, int n,
 constexpr int kHistThreads = 1024;
 __global__ void __launch_bounds__(kHistThreads) k_mc_hist(McState *ms, const unsigned long long *gkey,
                                                           unsigned int *hist, long long cap) {
-    __shared__ unsigned int sh[kSelBins];
+    __shared__ __align__(16) unsigned int sh[kSelBins];
     if (ms->done || ms->sel_resolved) return;
     const int n = mc_ncand(ms, cap);
     const int need = ms->sel_need;
@@ -1302,7 +1302,7 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
                                                        const double *cI, const double *bI, const double *HIIc,
                                                        const double *Hdiag, const float4 *rowf, float *Rh, float *Rl,
                                                        int ldr, int tpr, int crows, double *w,
-                                                       double *thr, double *etaout) {
+                                                       double *thr, double *etaout, long long *cand) {
     extern __shared__ __align__(16) float sm[];
     __shared__ float s_rf[2 * 32 * 16];
     __shared__ ff s_rff[2 * 32 * 2];
@@ -1717,7 +1717,7 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
             ms->pend_gamma = gamma;
             ms->pend_it = it;
             ms->pend_deg = deg ? 1 : 0;
-            ms->n_cand = 0;                             // the scatter builds the next candidate list
+            ms->n_cand = m;                             // the chosen ones come first, the scatter adds its own
             if (bad) set_status(st, kErrNonfinite);
         }
     }
@@ -1727,10 +1727,13 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
     bool to = false, from = false;
     if (coord) {
         w[ic] = eta * rsc;
+        const long long slot = sel[ic].slot;
         if (!bad) {
-            P.table[sel[ic].slot].c = zn * rsc;
+            P.table[slot].c = zn * rsc;
             cnz_set(P, sel[ic].A, sel[ic].B);
         }
+        cand[ic] = slot;                                // (its mark was cleared with the other candidates')
+        mark_set(P, slot);
         from = ct != 0.0 && zn == 0.0;
         to = ct == 0.0 && zn != 0.0;
     }
@@ -1890,7 +1893,8 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
                                                               const double *cI, const double *bI, const double *HIIc,
                                                               const double *Hdiag, const float4 *rowf,
                                                               const float *Rh, const float *Rl, int ldr, int tpr,
-                                                              int crows, double *w, double *thr, double *etaout) {
+                                                              int crows, double *w, double *thr, double *etaout,
+                                                              long long *cand) {
     extern __shared__ __align__(16) float sm[];
     __shared__ __align__(16) float s_r2[2][kRegSlots * 16];
     __shared__ ff s_rff[kRegSlots * 2];
@@ -2326,7 +2330,7 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
             ms->pend_gamma = gamma;
             ms->pend_it = it;
             ms->pend_deg = deg ? 1 : 0;
-            ms->n_cand = 0;                             // the scatter builds the next candidate list
+            ms->n_cand = m;                             // the chosen ones come first, the scatter adds its own
             if (bad) set_status(st, kErrNonfinite);
         }
     }
@@ -2343,10 +2347,13 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
     bool to = false, from = false;
     if (coord) {
         w[ic] = eta * rsc;
+        const long long slot = sel[ic].slot;
         if (!bad) {
-            P.table[sel[ic].slot].c = zn * rsc;
+            P.table[slot].c = zn * rsc;
             cnz_set(P, sel[ic].A, sel[ic].B);
         }
+        cand[ic] = slot;                                // (its mark was cleared with the other candidates')
+        mark_set(P, slot);
         from = ct != 0.0 && zn == 0.0;
         to = ct == 0.0 && zn != 0.0;
     }
@@ -2356,7 +2363,7 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
 }
 
 // ---------------------------------------------------------------------------
-// The scalars of Alg. 2's update of c (one block, inside the scatter's launch,
+// The scalars of Alg. 2's update of c (a few blocks inside the scatter's launch,
 // so that it runs beside the scatter): with gamma and eta from k_mc_eigen,
 //   mu'    = gamma^2 mu + 2 gamma eta.c_I + eta.eta,
 //   alpha' = gamma^2 alpha + 2 gamma eta.b_I + eta^T H_II eta   (double-double),
@@ -2366,11 +2373,17 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
 struct McUpdate {
     const double *cI, *bI, *eta;
     const float *Rh, *Rl;
-    int ldr, on;                    // on = 0: no update block (the scatter of a start vector)
+    int ldr, on;                    // on: blocks of the update (0: none, the scatter of a start vector)
 };
+constexpr int kUpdMax = 8;
+static_assert(sizeof(McState::upd) == kUpdMax * sizeof(ff), "one partial per update block");
+// Blocks of the update: about 64 rows each, so that the product ends before the
+// scatter beside it (m = 256 on one block took 20 of the scatter's 24.7 us).
+__host__ __forceinline__ int mc_update_blocks(int m) { return std::min(kUpdMax, (m + 63) / 64); }
 __device__ void mc_update_block(const Problem &P, McState *ms, IterState *st, const double *cI, const double *bI,
-                                const double *etaout, const float *Rh, const float *Rl, int ldr, int m,
-                                float *s_eta, double *s_red) {
+                                const double *etaout, const float *Rh, const float *Rl, int ldr, int m, int part,
+                                int parts, float *s_eta, double *s_red) {
+    __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int L = eig_len(m + 1), nq = L / 4;
     // eta as float-float in R's absolute indexing (entry 0 and the padding are zero)
@@ -2388,12 +2401,13 @@ __device__ void mc_update_block(const Problem &P, McState *ms, IterState *st, co
         ee = fma(e, e, ee);
     }
     __syncthreads();
-    // eta^T H_II eta over R's rows and columns 1..m: warp w takes the row pairs (a, a + nw),
-    // a = 1 + w, 1 + w + 2 nw, ...; lane l the 4-column chunks l, l + 32, ... of both rows
+    // eta^T H_II eta over R's rows and columns 1..m: warp w of the nwt = parts nw warps takes the row
+    // pairs (a, a + nwt), a = 1 + w, 1 + w + 2 nwt, ...; lane l the 4-column chunks l, l + 32, ...
+    const int nwt = parts * nw;
     const float4 *e4 = reinterpret_cast<const float4 *>(s_eta);
     float ah = 0.0f, al = 0.0f;
-    for (int a = 1 + warp; a <= m; a += 2 * nw) {
-        const int b = a + nw;
+    for (int a = 1 + part * nw + warp; a <= m; a += 2 * nwt) {
+        const int b = a + nwt;
         const bool two = b <= m;
         const float4 *h0 = reinterpret_cast<const float4 *>(Rh + (size_t)a * ldr);
         const float4 *l0 = reinterpret_cast<const float4 *>(Rl + (size_t)a * ldr);
@@ -2431,14 +2445,32 @@ __device__ void mc_update_block(const Problem &P, McState *ms, IterState *st, co
     }
     __syncthreads();
     if (warp != 0) return;
-    // warp 0: the warps' sums in order (every lane), then mu' (lane 0) and alpha' (lane 1) in the same
-    // instructions, double-double
+    // warp 0: the warps' sums in order (every lane)
     double sc = 0.0, sb = 0.0, se = 0.0;
     ff sh = {0.0f, 0.0f};
     for (int q = 0; q < nw; ++q) {
         sc += s_red[4 * q]; sb += s_red[4 * q + 1]; se += s_red[4 * q + 2];
         sh = ff_add(sh, reinterpret_cast<const ff *>(s_red + 4 * q + 3)[0]);
     }
+    if (parts > 1) {
+        // the blocks' parts of eta^T H_II eta, added in block order by the one that comes last (the
+        // other sums are every block's own)
+        if (lane == 0) {
+            reinterpret_cast<ff *>(ms->upd)[part] = sh;
+            __threadfence();
+            s_last = atomicAdd(&ms->upd_cnt, 1u) == (unsigned)parts - 1u;
+            if (s_last) ms->upd_cnt = 0u;
+            __threadfence();
+        }
+        __syncwarp();
+        if (!s_last) return;
+        sh = ff{0.0f, 0.0f};
+        for (int q = 0; q < parts; ++q) {
+            const float2 v = __ldcg(reinterpret_cast<const float2 *>(ms->upd) + q);
+            sh = ff_add(sh, ff{v.x, v.y});
+        }
+    }
+    // mu' (lane 0) and alpha' (lane 1) in the same instructions, double-double
     const dd mu0 = ms->mu, al0 = ms->alpha;
     const double gamma = ms->pend_gamma;
     const bool a1 = lane == 1;
@@ -2817,8 +2849,21 @@ __device__ __forceinline__ void mc_item_s(const Problem &P, McWarp &W, const Col
         const size_t row = (size_t)(i * N + a) * N;
         const double *tA_row = (alpha ? P.W3 : P.V3) + row, *tB_row = (alpha ? P.V3 : P.W3) + row;
         double v = __ldg(P.h + i * N + a);
-        for (unsigned long long m = A; m; m &= m - 1) v += __ldg(tA_row + (__ffsll((long long)m) - 1));
-        for (unsigned long long m = B; m; m &= m - 1) v += __ldg(tB_row + (__ffsll((long long)m) - 1));
+        for (unsigned long long mA = A, mB = B; mA | mB;) {    // eight terms in flight before their adds
+            double t[8];
+            bool in[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool fa = mA != 0ull;
+                const unsigned long long mm = fa ? mA : mB;
+                in[u] = mm != 0ull;
+                t[u] = in[u] ? __ldg((fa ? tA_row : tB_row) + (__ffsll((long long)mm) - 1)) : 0.0;
+                if (fa) mA &= mA - 1; else mB &= mB - 1;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (in[u]) v += t[u];
+        }
         H = apply_parity(v, (unsigned long long)(e.info & 1));
         oa = alpha ? e.key : A;
         ob = alpha ? B : e.key;
@@ -2834,25 +2879,24 @@ __global__ void __launch_bounds__(256, 3) k_mc_scatter(Problem P, McState *ms, I
                                                     const double *w, const double *thr, long long *cand,
                                                     double *gathp, unsigned int *work, McUpdate U) {
     __shared__ unsigned long long q_a[8][kScatterQ], q_b[8][kScatterQ], q_h[8][kScatterQ];
-    __shared__ double q_H[8][kScatterQ];
+    __shared__ __align__(16) double q_H[8][kScatterQ];   // (the update blocks read it in 16-byte words)
     __shared__ long long w_cand[8][kWarpCand];
     __shared__ int s_cnt[4][8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (ms->done || st->status) return;
     const int m = ms->m_sel;
-    if (U.on && blockIdx.x == 0) {                      // the first block: mu, alpha and the scale, beside the scatter
-        mc_update_block(P, ms, st, U.cI, U.bI, U.eta, U.Rh, U.Rl, U.ldr, m, reinterpret_cast<float *>(&q_H[0][0]),
-                        reinterpret_cast<double *>(&q_a[0][0]));
+    if ((int)blockIdx.x < U.on) {                       // the first blocks: mu, alpha and the scale, beside the scatter
+        mc_update_block(P, ms, st, U.cI, U.bI, U.eta, U.Rh, U.Rl, U.ldr, m, (int)blockIdx.x, U.on,
+                        reinterpret_cast<float *>(&q_H[0][0]), reinterpret_cast<double *>(&q_a[0][0]));
         return;
     }
     const int total = m * Gm.per_col;
     const int ns = Gm.nsA + Gm.nsB;
     McWarp W{q_a[warp], q_b[warp], q_h[warp], q_H[warp], w_cand[warp], l2_evict_first(), l2_evict_last(),
              0ull, 0.0, 0.0, 0, 0, 0, 0, 0, 0, false};
-    // the next item's index is fetched while the current one runs
-    int t_next = 0;
-    if (lane == 0) t_next = (int)atomicAdd(work, 1u);
-    t_next = __shfl_sync(0xffffffffu, t_next, 0);
+    // the first item is the warp's own; the next one's index is fetched while the current one runs
+    const int nwarps = ((int)gridDim.x - U.on) * 8;
+    int t_next = ((int)blockIdx.x - U.on) * 8 + warp;
     for (;;) {
         const int t = t_next;
         if (t >= total || W.err) break;
@@ -2886,7 +2930,7 @@ __global__ void __launch_bounds__(256, 3) k_mc_scatter(Problem P, McState *ms, I
         double gsum = W.gather;
         for (int o = 16; o > 0; o >>= 1) gsum += __shfl_down_sync(0xffffffffu, gsum, o);
         if (lane == 0) gathp[(size_t)col * Gm.per_col + k] = gsum;
-        t_next = __shfl_sync(0xffffffffu, (int)fetched, 0);
+        t_next = nwarps + __shfl_sync(0xffffffffu, (int)fetched, 0);
     }
     mc_flush_cand(P, ms, st, w_cand[warp], W.nwc, cand);
     // counters: warp sums, then the warps in order
@@ -2901,65 +2945,51 @@ __global__ void __launch_bounds__(256, 3) k_mc_scatter(Problem P, McState *ms, I
     }
 }
 
-// b_I recalculated (Eq. recalculate-b), the chosen coordinates join the
-// candidates, counters and the host snapshot.  One warp per chosen column (8
-// per block): its gather from the item partials (lane-strided in item order,
-// then a fixed tree), b_i = H_ii c_i + gather, the candidate mark; the block's
-// new candidates in one reservation.  The last block to finish (a counter in
-// McState, reset by that block) writes the counters and the snapshot.
+// b_I recalculated (Eq. recalculate-b): one warp per chosen column (8 per
+// block), its gather from the item partials (lane-strided in item order, then a
+// fixed tree), b_i = H_ii c_i + gather.  The last block instead writes the
+// counters and the host snapshot beside them, from what the scatter left (nothing
+// of it depends on the other blocks).  McState::done is left to the next
+// iteration's first kernel, as blocks of this launch still read it.
 constexpr int kFinWarps = 8;
 __global__ void __launch_bounds__(32 * kFinWarps) k_mc_finalize(Problem P, McState *ms, IterState *st,
                                                                 const McSel *sel, const double *Hdiag,
-                                                                const double *gathp, long long *cand,
-                                                                const double *etaout, int per_col, unsigned int *work) {
-    __shared__ long long s_slot[kFinWarps];
-    __shared__ int s_app[kFinWarps], s_nd[kFinWarps];
-    __shared__ bool s_last;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *work = 0u;   // the next scatter's item counter
-    if (ms->done) return;                               // read-only here: uniform over the blocks
-    const bool skip = st->status != 0;
-    const int m = ms->m_sel;
+                                                                const double *gathp, const double *etaout, int per_col,
+                                                                unsigned int *work) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * kFinWarps + warp;
-    if (lane == 0) { s_app[warp] = 0; s_nd[warp] = 0; }
-    if (!skip && i < m) {                               // warp-uniform
+    const bool books = blockIdx.x == gridDim.x - 1;
+    if (books && threadIdx.x == 0) *work = 0u;         // the next scatter's item counter
+    if (ms->done) return;
+    const int m = ms->m_sel;
+    if (!books) {
+        const int i = blockIdx.x * kFinWarps + warp;
+        const int status = st->status;                  // (a full table may be noticed by the last block just now)
+        if (i >= m || (status != 0 && status != kErrTableFull)) return;
+        Slot *sp = P.table + sel[i].slot;
+        const double hd = Hdiag[i], c = sp->c;
         double t = 0.0;
-        for (int k = lane; k < per_col; k += 32) t += gathp[(size_t)i * per_col + k];
+        const double *g = gathp + (size_t)i * per_col;
+        for (int k = lane; k < per_col; k += 256) {     // eight loads in flight, added in item order
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < per_col ? g[k + 32 * u] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k + 32 * u < per_col) t += v[u];
+        }
         for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) {
-            const long long slot = sel[i].slot;
-            const double hd = Hdiag[i];
-            Slot *sp = P.table + slot;
-            sp->bv = fma(hd, sp->c, t);
-            s_nd[warp] = is_zero(hd) ? 0 : 1;
-            s_slot[warp] = slot;
-            s_app[warp] = mark_set(P, slot) ? 1 : 0;
-        }
+        if (lane == 0) sp->bv = fma(hd, c, t);
+        return;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the block's new candidates (warp order) in one reservation, its nonzero diagonals
-        int na = 0, nd = 0;
-        for (int w = 0; w < kFinWarps; ++w) { na += s_app[w]; nd += s_nd[w]; }
-        if (na) {
-            const int base = atomicAdd(&ms->n_cand, na);
-            for (int w = 0, at = base; w < kFinWarps; ++w)
-                if (s_app[w]) {
-                    if (at < P.cap_cand) cand[at] = s_slot[w];
-                    else set_status(st, kErrInternal);
-                    ++at;
-                }
-        }
-        if (nd) atomicAdd(&ms->fin_nd, nd);
-        __threadfence();
-        s_last = atomicAdd(&ms->fin_blocks, 1u) == gridDim.x - 1;
+    int nd = 0;                                         // nonzero diagonals (none are counted after an error)
+    const bool skip = st->status != 0;
+    for (int i0 = 0; i0 < m; i0 += 32 * kFinWarps) {
+        const int i = i0 + (int)threadIdx.x;
+        nd += __syncthreads_count(!skip && i < m && !is_zero(Hdiag[i]));
     }
-    __syncthreads();
-    if (!s_last || threadIdx.x != 0) return;
-    __threadfence();
+    if (threadIdx.x != 0) return;
     // every field read first (independent loads), then written
-    const long long nd_all = (long long)atomicExch(&ms->fin_nd, 0);
-    ms->fin_blocks = 0u;
+    const long long nd_all = nd;
     const unsigned long long c0 = ms->cnt[0], c1 = ms->cnt[1], c2 = ms->cnt[2], c3 = ms->cnt[3];
     const long long el = ms->elements + (long long)c0 + nd_all, ap = ms->applied + (long long)c1 + nd_all;
     const long long dr = ms->dropped + (long long)c2, in = ms->inserted + (long long)c3;
@@ -2967,7 +2997,7 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_mc_finalize(Problem P, McSta
     const long long its = ms->iterations, nnz = ms->nnz_c, eit = ms->eig_iters_total;
     const dd mu = ms->mu, al = ms->alpha;
     const double dx = ms->dx, en = ms->energy;
-    const int done = ms->done_pending ? 1 : ms->done;
+    const int done = ms->done_pending ? 1 : 0;
     const double eta0 = m > 0 ? etaout[0] : 0.0;
     const unsigned long long la = m > 0 ? sel[0].A : 0ull, lb = m > 0 ? sel[0].B : 0ull;
     ms->elements = el;
@@ -2977,7 +3007,6 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_mc_finalize(Problem P, McSta
     ms->n_slots = ns;
     ms->last_column = (long long)c0 + nd_all;
     for (int k = 0; k < 4; ++k) ms->cnt[k] = 0;
-    ms->done = done;
     if (ns > P.max_entries) set_status(st, kErrTableFull);
     st->iterations = its;
     st->nnz_c = nnz;
@@ -3005,7 +3034,7 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_mc_finalize(Problem P, McSta
 // starts from the reset state: c = e_ref (eta = 1) is the default start of r4.
 __global__ void k_mc_start(Problem P, McState *ms, IterState *st, McSel *sel, double *Hdiag, double *w, double *thr,
                            double *etaout, unsigned long long A, unsigned long long B, double eta, int first,
-                           ColEnt *coltab, ColLists *collists) {
+                           ColEnt *coltab, ColLists *collists, long long *cand) {
     __shared__ ColLists L;
     __shared__ long long s_slot;
     __shared__ double s_bold;
@@ -3049,6 +3078,15 @@ __global__ void k_mc_start(Problem P, McState *ms, IterState *st, McSel *sel, do
                 ms->done_pending = 0;
                 ms->n_above = 0;
                 ms->n_inbin = 0;
+            }
+            if (mark_set(P, s_slot)) {                 // the entry joins the candidates
+                const int at = ms->n_cand;
+                if (at < P.cap_cand) {
+                    cand[at] = s_slot;
+                    ms->n_cand = at + 1;
+                } else {
+                    set_status(st, kErrInternal);
+                }
             }
             McSel x;
             x.slot = s_slot; x.gkey = 0ull; x.A = A; x.B = B;
@@ -3162,15 +3200,15 @@ cudaError_t launch_entry(const Problem &P, unsigned long long A1, unsigned long 
 cudaError_t launch_mc_start(const Problem &P, const McBuffers &b, unsigned long long A, unsigned long long B,
                             double eta, int first, cudaStream_t s) {
     k_mc_start<<<1, 64, 0, s>>>(P, b.ms, b.st, b.sel, b.Hdiag, b.w, b.thr, b.eta, A, B, eta, first, b.coltab,
-                                b.collists);
+                                b.collists, b.cand);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mc_scatter_finalize(const Problem &P, const McBuffers &b, cudaStream_t s) {
     k_mc_scatter<<<b.scatter_grid, 256, 0, s>>>(P, b.ms, b.st, b.sel, b.coltab, b.collists, b.geom, b.w, b.thr,
                                                  b.cand, b.gathp, b.work, McUpdate{});
-    k_mc_finalize<<<(b.m + kFinWarps - 1) / kFinWarps, 32 * kFinWarps, 0, s>>>(P, b.ms, b.st, b.sel, b.Hdiag, b.gathp,
-                                                                              b.cand, b.eta, b.geom.per_col, b.work);
+    k_mc_finalize<<<(b.m + kFinWarps - 1) / kFinWarps + 1, 32 * kFinWarps, 0, s>>>(P, b.ms, b.st, b.sel, b.Hdiag,
+                                                                                  b.gathp, b.eta, b.geom.per_col, b.work);
     return cudaGetLastError();
 }
 
@@ -3213,21 +3251,22 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
             cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen_reg<true> : k_mc_eigen_reg<false>, P, b.ms, b.st,
                                (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
                                (const double *)b.Hdiag, (const float4 *)b.rowf, (const float *)b.Rh,
-                               (const float *)b.Rl, b.ldr, g.tpr, g.crows, b.w, b.thr, b.eta);
+                               (const float *)b.Rl, b.ldr, g.tpr, g.crows, b.w, b.thr, b.eta, b.cand);
         else
             cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen<true> : k_mc_eigen<false>, P, b.ms, b.st,
                                (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
                                (const double *)b.Hdiag, (const float4 *)b.rowf, b.Rh, b.Rl, b.ldr, g.tpr, g.crows,
-                               b.w, b.thr, b.eta);
+                               b.w, b.thr, b.eta, b.cand);
     }
     mark();
-    // one more block than the scatter's own: block 0 updates mu, alpha and the scale meanwhile
-    k_mc_scatter<<<b.scatter_grid + 1, 256, 0, s>>>(P, b.ms, b.st, b.sel, b.coltab, b.collists, b.geom, b.w, b.thr,
-                                                     b.cand, b.gathp, b.work,
-                                                     McUpdate{b.cI, b.bI, b.eta, b.Rh, b.Rl, b.ldr, 1});
+    // beside the scatter's own blocks, the first ones update mu, alpha and the scale
+    const int nu = mc_update_blocks(b.m);
+    k_mc_scatter<<<b.scatter_grid + nu, 256, 0, s>>>(P, b.ms, b.st, b.sel, b.coltab, b.collists, b.geom, b.w, b.thr,
+                                                      b.cand, b.gathp, b.work,
+                                                      McUpdate{b.cI, b.bI, b.eta, b.Rh, b.Rl, b.ldr, nu});
     mark();
-    k_mc_finalize<<<(b.m + kFinWarps - 1) / kFinWarps, 32 * kFinWarps, 0, s>>>(P, b.ms, b.st, b.sel, b.Hdiag, b.gathp,
-                                                                              b.cand, b.eta, b.geom.per_col, b.work);
+    k_mc_finalize<<<(b.m + kFinWarps - 1) / kFinWarps + 1, 32 * kFinWarps, 0, s>>>(P, b.ms, b.st, b.sel, b.Hdiag,
+                                                                                  b.gathp, b.eta, b.geom.per_col, b.work);
     mark();
     return cudaGetLastError();
 }

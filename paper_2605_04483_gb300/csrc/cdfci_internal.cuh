@@ -156,9 +156,8 @@ struct McState {
     dd pend_scale;                 // s gamma
     double pend_gamma;
     int pend_it, pend_deg;
-    // the finalisation's last-block counter and nonzero diagonals (zero between iterations)
-    unsigned int fin_blocks;
-    int fin_nd;
+    float upd[16];                 // the update blocks' parts of eta^T H_II eta (float-float) ...
+    unsigned int upd_cnt;          // ... and how many have written theirs (zero between iterations)
 };
 
 // xCDFCI (Algorithm 3, k1 = K + 1 states) iteration state, one per handle.
@@ -370,7 +369,7 @@ struct CdInstance {
 // Column decoding.  Per column the CTA holds the occupied / virtual orbital
 // lists of both spins in shared memory.
 // ---------------------------------------------------------------------------
-struct ColLists {
+struct __align__(16) ColLists {          // (copied in 8-byte words)
     unsigned char occA[64], virA[64], occB[64], virB[64];
 };
 
