@@ -275,13 +275,13 @@ int setup_xcd(cdfci_ctx *c, int k1, unsigned long long refA, unsigned long long 
     cudaStream_t s = c->stream;
     const long long nh_eff = P.doubles_vanish ? P.seg[2] : P.seg[5];
     c->k1 = k1;
-    b.nscatter = x_scatter_blocks();
-    b.nselect = 152;
+    b.nscatter = x_scatter_blocks(P);
+    b.nselect = x_select_blocks(P);
     b.cap_cand = (long long)k1 * (nh_eff + 1) + 64;
     if (mb_alloc(c, &b.xs, 1) || mb_alloc(c, &b.rows, (size_t)P.capacity * 2 * k1) ||
         mb_alloc(c, &b.cand, (size_t)b.cap_cand) || mb_alloc(c, &b.gathp, (size_t)b.nscatter * k1) ||
         mb_alloc(c, reinterpret_cast<unsigned char **>(&b.bbest), (size_t)b.nselect * x_block_bytes()) ||
-        mb_alloc(c, &b.counter, 1))
+        mb_alloc(c, &b.counter, 2))
         return fail(CDFCI_ERR_NOMEM, "device allocation of the xCDFCI buffers failed");
     b.st = c->d_st;
     XState x;
@@ -289,7 +289,7 @@ int setup_xcd(cdfci_ctx *c, int k1, unsigned long long refA, unsigned long long 
     x.k1 = k1;
     CK(cudaMemcpyAsync(b.xs, &x, sizeof(x), cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(b.rows, 0, (size_t)P.capacity * 2 * k1 * sizeof(double), s));
-    CK(cudaMemsetAsync(b.counter, 0, sizeof(unsigned int), s));
+    CK(cudaMemsetAsync(b.counter, 0, 2 * sizeof(unsigned int), s));
     // the reference column and its diagonals
     CK(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned long long), s));
     CK(launch_column(P, refA, refB, c->d_colkeys, c->d_colvals, P.nh, c->d_counter, s));

@@ -168,6 +168,7 @@ struct XState {
     dd S[kXMax * kXMax], M[kXMax * kXMax];   // C^T C, C^T H C (double-double)
     double g[kXMax];               // G_i of the chosen row (4 B_i + 4 C_i S)
     double wv[kXMax];              // scatter weights eta g
+    double c_old[kXMax], b_old[kXMax];   // the chosen row's C and B before the step
     double thr;                    // |H_ji| >= thr passes the compression rule: tau / max_a |eta g_a|
     double eta, dx, Hii;
     double E[kXMax];               // energies of the pencil (M, S), ascending (on request)
@@ -176,6 +177,7 @@ struct XState {
     long long iterations, nnz_c, n_slots, elements, applied, dropped, inserted, last_column;
     unsigned long long cnt[4];     // counters of the running column
     int n_cand, k1, done;
+    int go;                        // 1: this iteration takes a step
 };
 
 // Everything a kernel needs about the problem and the table.

@@ -1258,11 +1258,14 @@ __global__ void k_jk(const double *g, int N, double *J, double *K, int *has_doub
         J[t] = g[(((size_t)p * N + p) * N + q) * N + q];
         K[t] = g[(((size_t)p * N + q) * N + q) * N + p];
     }
+    // (a flag per thread, one store a block: an atomic for every nonzero element took 190 us at N = 24)
+    bool any = false;
     const long long n4 = (long long)N * N * N * N;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += (long long)gridDim.x * blockDim.x) {
         int s = (int)(t % N), r = (int)((t / N) % N), q = (int)((t / N / N) % N), p = (int)(t / N / N / N);
-        if (p != q && r != s && g[t] != 0.0) atomicExch(has_doubles, 1);
+        any = any || (p != q && r != s && g[t] != 0.0);
     }
+    if (__syncthreads_or(any) && threadIdx.x == 0) *has_doubles = 1;
 }
 
 // Single-excitation term tables (Eq. entry, singles): for the excitation i -> a

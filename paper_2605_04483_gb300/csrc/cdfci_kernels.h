@@ -31,10 +31,11 @@ struct XBuffers {
     long long cap_cand;
     double *gathp;                 // per scatter block: k1 gather sums
     void *bbest;                   // per select block: its best candidate
-    unsigned int *counter;         // last-block counter of the selection
+    unsigned int *counter;         // last-block counters of the choice and the column
     int nscatter, nselect;
 };
-int x_scatter_blocks();
+int x_scatter_blocks(const Problem &P);
+int x_select_blocks(const Problem &P);
 size_t x_block_bytes();
 cudaError_t launch_x_start(const Problem &P, const XBuffers &b, unsigned long long A, unsigned long long B, int k,
                            cudaStream_t s);

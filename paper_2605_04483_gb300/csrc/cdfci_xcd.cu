@@ -1,31 +1,33 @@
 // xCDFCI (Algorithm 3): K + 1 states, one row of C per iteration.
 //
-// Per iteration four launches (captured in a CUDA graph):
-//   k_x_select    argmax over the candidates of ||G_j||_inf, G_j = 4 B_j + 4 C_j S
+// Per iteration two launches (captured in a CUDA graph), each with its serial
+// part in the block that finishes last:
+//   k_x_choose    argmax over the candidates of ||G_j||_inf, G_j = 4 B_j + 4 C_j S
 //                 (ties: the smaller key), by a block argmax and a last-block
-//                 reduction in block order; clears the candidates' marks;
-//   k_x_prepare   H_ii, the quartic of problem choose-eta (appendix "Determining
-//                 Step Size") and its minimiser eta, C_i += eta G_i, the S and M
-//                 updates (double-double, one entry per lane);
-//   k_x_scatter   B_j += eta H_ji G_i for the column of i with the row compression
+//                 reduction in block order, clearing the candidates' marks; then
+//                 H_ii, the quartic of problem choose-eta (appendix "Determining
+//                 Step Size") and its minimiser eta, C_i += eta G_i;
+//   k_x_column    B_j += eta H_ji G_i for the column of i with the row compression
 //                 rule, insertion of absent rows, the gather sum_j H_ji C_j per
-//                 block, the rows it updated become the next candidates;
-//   k_x_finalize  B_i = H_ii C_i + the gather (Eq. recalculate-b, per state),
-//                 counters.
+//                 block, the rows it updated become the next candidates; then
+//                 B_i = H_ii C_i + the gather (Eq. recalculate-b, per state) and
+//                 the counters.  A block of its own updates S and M
+//                 (double-double, one entry per lane) beside it: they are first
+//                 read by the next choice.
+// What bounds an iteration is the latency of its dependent memory requests and
+// FP64 chains (a column of the N = 24 problem is one element a thread).  As four
+// launches (selection, preparation with S and M, column, recalculation) it took
+// 55.4 us with K + 1 = 4 (N = 24, 6 + 5 electrons), now 34.1 us.
 // The energies (the pencil (M, S)) are computed on request by k_x_energies.
 // Each row j occurs once in a column, so B_j is updated by plain loads and
 // stores, and every reduction has a fixed order: the iteration is
 // deterministic.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 
 #include "cdfci_internal.cuh"
 #include "cdfci_kernels.h"
 
 namespace cdfci {
-
-namespace cg = cooperative_groups;
 
 namespace {
 
@@ -46,9 +48,8 @@ __device__ __forceinline__ bool x_better(const XBest &x, const XBest &y) {
 }
 
 
-// ||G_j||_inf and G_j = 4 B_j + 4 C_j S from the row's C and B halves (G may be null)
-__device__ __forceinline__ double x_gnorm(const double (&c)[kXMax], const double (&bb)[kXMax], const double *S, int k1,
-                                           double *G) {
+// ||G_j||_inf, G_j = 4 B_j + 4 C_j S, from the row's C and B halves
+__device__ __forceinline__ double x_gnorm(const double (&c)[kXMax], const double (&bb)[kXMax], const double *S, int k1) {
     double m = 0.0;
 #pragma unroll
     for (int a = 0; a < kXMax; ++a) {
@@ -59,9 +60,7 @@ __device__ __forceinline__ double x_gnorm(const double (&c)[kXMax], const double
             if (b >= k1) break;
             s = fma(c[b], S[b * k1 + a], s);
         }
-        const double ga = 4.0 * bb[a] + 4.0 * s;
-        if (G) G[a] = ga;
-        m = fmax(m, fabs(ga));
+        m = fmax(m, fabs(4.0 * bb[a] + 4.0 * s));
     }
     return m;
 }
@@ -114,72 +113,6 @@ __device__ __forceinline__ void x_load_row(const double *rows, long long j, int 
     }
 }
 
-__global__ void __launch_bounds__(kXThreads) k_x_select(Problem P, XState *xs, IterState *st, const long long *cand,
-                                                        const double *rows, XBest *bbest, unsigned int *counter) {
-    __shared__ double sS[kXMax * kXMax];
-    __shared__ XBest wb[kXThreads / 32];
-    __shared__ bool s_last;
-    if (xs->done || st->status) return;
-    const int k1 = xs->k1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int t = tid; t < k1 * k1; t += blockDim.x) sS[t] = xs->S[t].hi + xs->S[t].lo;
-    __syncthreads();
-    const int n = xs->n_cand;
-    XBest best{0ull, ~0ull, ~0ull, -1};
-    for (int t = blockIdx.x * blockDim.x + tid; t < n; t += gridDim.x * blockDim.x) {
-        const long long s = cand[t];
-        double rc[kXMax], rb[kXMax];
-        x_load_row(rows, s, k1, rc, rb);
-        const ulonglong2 key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + s));
-        P.table[s].b = key.y & kKeyMaskB;                          // no longer a candidate
-        const XBest x{x_abs_bits(x_gnorm(rc, rb, sS, k1, nullptr)), key.x, key.y & kKeyMaskB, s};
-        if (x_better(x, best)) best = x;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        XBest y;
-        y.gbits = __shfl_down_sync(0xffffffffu, best.gbits, off);
-        y.a = __shfl_down_sync(0xffffffffu, best.a, off);
-        y.b = __shfl_down_sync(0xffffffffu, best.b, off);
-        y.slot = __shfl_down_sync(0xffffffffu, best.slot, off);
-        if (x_better(y, best)) best = y;
-    }
-    if (lane == 0) wb[warp] = best;
-    __syncthreads();
-    if (tid == 0) {
-        XBest b = wb[0];
-        for (int w = 1; w < kXThreads / 32; ++w)
-            if (x_better(wb[w], b)) b = wb[w];
-        bbest[blockIdx.x] = b;
-        __threadfence();
-        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last || warp != 0) return;
-    __threadfence();
-    // the last block's warp 0 reduces the blocks' winners: lane l takes blocks l, l + 32, ...
-    XBest b{0ull, ~0ull, ~0ull, -1};
-    for (int k = lane; k < (int)gridDim.x; k += 32) {
-        const XBest y = bbest[k];
-        if (x_better(y, b)) b = y;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        XBest y;
-        y.gbits = __shfl_down_sync(0xffffffffu, b.gbits, off);
-        y.a = __shfl_down_sync(0xffffffffu, b.a, off);
-        y.b = __shfl_down_sync(0xffffffffu, b.b, off);
-        y.slot = __shfl_down_sync(0xffffffffu, b.slot, off);
-        if (x_better(y, b)) b = y;
-    }
-    if (lane != 0) return;
-    *counter = 0u;
-    xs->n_cand = 0;
-    if (b.slot < 0) { xs->done = 1; xs->eta = 0.0; return; }     // nothing left to choose
-    double rc[kXMax], rb[kXMax], G[kXMax];
-    x_load_row(rows, b.slot, k1, rc, rb);
-    x_gnorm(rc, rb, sS, k1, G);
-    for (int a = 0; a < k1; ++a) xs->g[a] = G[a];
-    xs->slot = b.slot; xs->A = b.a; xs->B = b.b;
-}
-
 // H_ii exactly as diag_warp(P, L) computes it (the same terms, per-lane sums
 // in the same order, the same tree), with every lane's loads issued before the
 // first addition: one round trip for the integrals of up to 16 electrons.
@@ -221,45 +154,41 @@ __device__ __forceinline__ double x_diag(const Problem &P, const ColLists &L) {
     return __shfl_sync(0xffffffffu, x, 0);
 }
 
-// forced >= 0: the start step of row {fA, fB} with g = e_forced and eta = 1.
-__global__ void k_x_prepare(Problem P, XState *xs, IterState *st, double *rows, int forced, unsigned long long fA,
-                            unsigned long long fB) {
-    __shared__ ColLists L;
-    __shared__ long long s_slot;
-    __shared__ double s_c[kXMax], s_g[kXMax], s_b[kXMax], s_t[kXMax];
-    __shared__ double s_eta, s_gn, s_w[kXMax];
-    __shared__ int s_stop;
-    if (xs->done || st->status) return;
-    const int k1 = xs->k1, lane = threadIdx.x;
-    if (lane == 0) {
-        s_stop = 0;
-        xs->eta = 0.0;                                               // 0: no step this iteration
-        if (forced >= 0) {
-            bool ins = false;
-            const long long s = table_find(P, st, fA, fB, true, &ins);
-            if (s < 0) { s_stop = 1; } else {
-                if (ins) { xs->n_slots += 1; xs->inserted += 1; }
-                xs->slot = s; xs->A = fA; xs->B = fB;
-                for (int a = 0; a < k1; ++a) xs->g[a] = a == forced ? 1.0 : 0.0;
-            }
-        }
-        s_slot = xs->slot;
+// The step of the chosen row (warp 0 of a block): H_ii, the quartic and eta, the
+// scatter weights, C_i += eta g; c and b of the row as they were are left for the
+// update of S and M.  forced >= 0: the start step of row {fA, fB} with g =
+// e_forced and eta = 1.
+struct XStepShared {
+    ColLists L;
+    double c[kXMax], g[kXMax], b[kXMax], t[kXMax];
+    double eta, gn;
+    int stop;
+};
+__device__ void x_step(const Problem &P, XState *xs, IterState *st, double *rows, const double *sS, XStepShared &W,
+                       long long s, unsigned long long A, unsigned long long B, int forced) {
+    const int k1 = xs->k1, lane = threadIdx.x & 31;
+    if (lane < k1) {                                                  // loads in flight beside the lists
+        W.c[lane] = __ldcg(rows + s * 2 * k1 + lane);
+        W.b[lane] = __ldcg(rows + s * 2 * k1 + k1 + lane);
+    }
+    for (int t = lane; t < P.N; t += 32) {
+        const int ra = __popcll(A & low_mask(t)), rb = __popcll(B & low_mask(t));
+        if ((A >> t) & 1ull) W.L.occA[ra] = (unsigned char)t; else W.L.virA[t - ra] = (unsigned char)t;
+        if ((B >> t) & 1ull) W.L.occB[rb] = (unsigned char)t; else W.L.virB[t - rb] = (unsigned char)t;
+    }
+    if (lane == 0) W.stop = 0;
+    __syncwarp();
+    if (lane < k1) {                                                  // G_a, lane a
+        double m = 0.0;
+        for (int b = 0; b < k1; ++b) m = fma(W.c[b], sS[b * k1 + lane], m);
+        W.g[lane] = forced >= 0 ? (lane == forced ? 1.0 : 0.0) : 4.0 * W.b[lane] + 4.0 * m;
     }
     __syncwarp();
-    if (s_stop) return;
-    build_lists(L, P.N, xs->A, xs->B);
-    const long long s = s_slot;
-    if (lane < k1) {                                                  // loads in flight beside H_ii's
-        s_c[lane] = rows[s * 2 * k1 + lane];
-        s_b[lane] = rows[s * 2 * k1 + k1 + lane];
-        s_g[lane] = xs->g[lane];
-    }
-    __syncwarp();
-    const double Hii = x_diag(P, L);
+    const double Hii = x_diag(P, W.L);
     if (lane < k1 && forced < 0) {                                    // (S g)_a, lane a: the term of g S g^T
         double t = 0.0;
-        for (int b = 0; b < k1; ++b) t = fma(xs->S[lane * k1 + b].hi + xs->S[lane * k1 + b].lo, s_g[b], t);
-        s_t[lane] = t;
+        for (int b = 0; b < k1; ++b) t = fma(sS[lane * k1 + b], W.g[b], t);
+        W.t[lane] = t;
     }
     __syncwarp();
     if (lane == 0) {
@@ -270,100 +199,240 @@ __global__ void k_x_prepare(Problem P, XState *xs, IterState *st, double *rows, 
             // w1 = ||g||^2 (the directional derivative)
             double gg = 0.0, cg = 0.0, cc = 0.0, gSg = 0.0;
             for (int a = 0; a < k1; ++a) {
-                gg = fma(s_g[a], s_g[a], gg);
-                cg = fma(s_c[a], s_g[a], cg);
-                cc = fma(s_c[a], s_c[a], cc);
-                gSg = fma(s_g[a], s_t[a], gSg);
+                gg = fma(W.g[a], W.g[a], gg);
+                cg = fma(W.c[a], W.g[a], cg);
+                cc = fma(W.c[a], W.c[a], cc);
+                gSg = fma(W.g[a], W.t[a], gSg);
             }
             // In t = eta ||g|| the quartic is monic with O(1) coefficients (w / w4 would grow like
             // 1 / ||g||^2 near convergence and overflow the single-precision root stage):
             // t^4 + 4 (c.u) t^3 + (2 H_ii + 2 (c.u)^2 + 2 ||c||^2 + 2 u S u^T) t^2 + ||g|| t, u = g / ||g||.
-            const double gn = sqrt(gg);
-            s_gn = gn;
-            if (!(gn > 0.0)) { xs->done = 1; s_stop = 1; }
+            const double ign = rsqrt(gg), gn = gg * ign;
+            W.gn = gn;
+            if (!(gn > 0.0)) { xs->done = 1; W.stop = 1; }
             else {
-                const double cu = cg / gn;
+                const double cu = cg * ign;
                 const double v3 = 4.0 * cu;
-                const double v2 = 2.0 * Hii + 2.0 * cu * cu + 2.0 * cc + 2.0 * (gSg / gg);
-                eta = line_search(gn, v2, v3) / gn;
-                if (!isfinite(eta)) { set_status(st, kErrNonfinite); s_stop = 1; }
+                const double v2 = 2.0 * Hii + 2.0 * cu * cu + 2.0 * cc + 2.0 * (gSg * ign) * ign;
+                eta = line_search(gn, v2, v3) * ign;
+                if (!isfinite(eta)) { set_status(st, kErrNonfinite); W.stop = 1; }
             }
         }
-        s_eta = eta;
+        W.eta = eta;
     }
     __syncwarp();
-    if (s_stop) return;
-    const double eta = s_eta;
-    // S += eta (c^T g + g^T c) + eta^2 g^T g,  M += eta (b^T g + g^T b) + eta^2 H_ii g^T g (one entry per lane)
-    for (int t = lane; t < k1 * k1; t += 32) {
-        const int a = t / k1, b = t - a * k1;
-        const dd e2 = dd_two_prod(eta, eta);
-        const dd gab = dd_two_prod(s_g[a], s_g[b]);
-        const dd ds = dd_add(dd_mul_d(dd_add(dd_two_prod(s_c[a], s_g[b]), dd_two_prod(s_g[a], s_c[b])), eta),
-                             dd_mul(e2, gab));
-        const dd dm = dd_add(dd_mul_d(dd_add(dd_two_prod(s_b[a], s_g[b]), dd_two_prod(s_g[a], s_b[b])), eta),
-                             dd_mul_d(dd_mul(e2, gab), Hii));
-        xs->S[t] = dd_add(xs->S[t], ds);
-        xs->M[t] = dd_add(xs->M[t], dm);
-    }
+    if (W.stop) return;
+    const double eta = W.eta;
     // C_i += eta g (lane a), the scatter weights eta g and their largest magnitude
     const bool on = lane < k1;
-    double cn = 0.0;
+    double cn = 0.0, wa = 0.0;
     if (on) {
-        cn = fma(eta, s_g[lane], s_c[lane]);
+        const double c0 = W.c[lane], g0 = W.g[lane];
+        cn = fma(eta, g0, c0);
         rows[s * 2 * k1 + lane] = cn;
-        const double wa = eta * s_g[lane];
+        wa = eta * g0;
         xs->wv[lane] = wa;
-        s_w[lane] = fabs(wa);
+        xs->g[lane] = g0;
+        xs->c_old[lane] = c0;
+        xs->b_old[lane] = W.b[lane];
     }
-    const unsigned was = __ballot_sync(0xffffffffu, on && s_c[lane] != 0.0);
+    const unsigned was = __ballot_sync(0xffffffffu, on && W.c[lane & (kXMax - 1)] != 0.0);
     const unsigned now = __ballot_sync(0xffffffffu, on && cn != 0.0);
-    __syncwarp();
+    double wmax = fabs(wa);
+#pragma unroll
+    for (int off = kXMax / 2; off > 0; off >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, off));
     if (lane == 0) {
-        double wmax = 0.0;
-        for (int a = 0; a < k1; ++a) wmax = fmax(wmax, s_w[a]);
+        xs->slot = s; xs->A = A; xs->B = B;
         xs->nnz_c += (now ? 1 : 0) - (was ? 1 : 0);
-        xs->thr = wmax > 0.0 ? P.tau / wmax : 1.0e308;
+        xs->thr = wmax > 0.0 ? (P.tau > 0.0 ? P.tau / wmax : 0.0) : 1.0e308;
         xs->eta = eta;
         xs->Hii = Hii;
+        xs->go = 1;
         if (forced < 0) {
-            xs->dx = P.theta * xs->dx + (1.0 - P.theta) * fabs(eta) * s_gn;   // s_gn = ||g||
+            xs->dx = P.theta * xs->dx + (1.0 - P.theta) * fabs(eta) * W.gn;   // W.gn = ||g||
             xs->iterations += 1;
             if (P.dx_threshold > 0.0 && xs->dx < P.dx_threshold) xs->done = 1;
         }
     }
 }
 
+__global__ void __launch_bounds__(kXThreads) k_x_choose(Problem P, XState *xs, IterState *st, const long long *cand,
+                                                        double *rows, XBest *bbest, unsigned int *counter, int forced,
+                                                        unsigned long long fA, unsigned long long fB) {
+    __shared__ double sS[kXMax * kXMax];
+    __shared__ XBest wb[kXThreads / 32];
+    __shared__ XStepShared W;
+    __shared__ bool s_last;
+    __shared__ long long s_slot;
+    const int k1 = xs->k1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (xs->done || st->status) {
+        if (blockIdx.x == 0 && tid == 0) xs->go = 0;                 // no step this iteration
+        return;
+    }
+    for (int t = tid; t < k1 * k1; t += blockDim.x) sS[t] = xs->S[t].hi + xs->S[t].lo;
+    __syncthreads();
+    if (forced >= 0) {                                               // one block
+        if (warp != 0) return;
+        if (lane == 0) {
+            xs->go = 0;
+            xs->eta = 0.0;
+            bool ins = false;
+            const long long s = table_find(P, st, fA, fB, true, &ins);
+            if (s >= 0 && ins) { xs->n_slots += 1; xs->inserted += 1; }
+            s_slot = s;
+        }
+        __syncwarp();
+        if (s_slot >= 0) x_step(P, xs, st, rows, sS, W, s_slot, fA, fB, forced);
+        return;
+    }
+    const int n = xs->n_cand;
+    XBest best{0ull, ~0ull, ~0ull, -1};
+    for (int t = blockIdx.x * blockDim.x + tid; t < n; t += gridDim.x * blockDim.x) {
+        const long long s = cand[t];
+        double rc[kXMax], rb[kXMax];
+        x_load_row(rows, s, k1, rc, rb);
+        const ulonglong2 key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + s));
+        P.table[s].b = key.y & kKeyMaskB;                          // no longer a candidate
+        const XBest x{x_abs_bits(x_gnorm(rc, rb, sS, k1)), key.x, key.y & kKeyMaskB, s};
+        if (x_better(x, best)) best = x;
+    }
+    auto warp_best = [&](XBest b) {
+        for (int off = 16; off > 0; off >>= 1) {
+            XBest y;
+            y.gbits = __shfl_xor_sync(0xffffffffu, b.gbits, off);
+            y.a = __shfl_xor_sync(0xffffffffu, b.a, off);
+            y.b = __shfl_xor_sync(0xffffffffu, b.b, off);
+            y.slot = __shfl_xor_sync(0xffffffffu, b.slot, off);
+            if (x_better(y, b)) b = y;
+        }
+        return b;
+    };
+    best = warp_best(best);
+    if (lane == 0) wb[warp] = best;
+    __syncthreads();
+    if (tid == 0) {
+        XBest b = wb[0];
+        for (int w = 1; w < kXThreads / 32; ++w)
+            if (x_better(wb[w], b)) b = wb[w];
+        bbest[blockIdx.x] = b;
+        __threadfence();
+        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last || warp != 0) return;
+    __threadfence();
+    // the last block's warp 0 reduces the blocks' winners (lane l takes blocks l, l + 32, ...) and takes the step
+    XBest b{0ull, ~0ull, ~0ull, -1};
+    for (int k = lane; k < (int)gridDim.x; k += 32) {
+        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(bbest + k);
+        const ulonglong2 x = __ldcg(q), y = __ldcg(q + 1);
+        const XBest z{x.x, x.y, y.x, (long long)y.y};
+        if (x_better(z, b)) b = z;
+    }
+    b = warp_best(b);
+    if (lane == 0) {
+        *counter = 0u;
+        xs->n_cand = 0;
+        xs->go = 0;
+        xs->eta = 0.0;
+        if (b.slot < 0) xs->done = 1;                                // nothing left to choose
+    }
+    __syncwarp();
+    if (b.slot >= 0) x_step(P, xs, st, rows, sS, W, b.slot, b.a, b.b, -1);
+}
 
-// The slot of key {a, b} by linear probing from pos (no insert): -1 absent, -2
-// error (status set); kbo receives the slot's b word, candidate mark included.
-__device__ __forceinline__ long long x_find(const Problem &P, IterState *st, unsigned long long a,
-                                            unsigned long long b, unsigned long long pos, unsigned long long &kbo) {
+// The slot of key {a, b} by linear probing from pos (no insert), whose first key
+// the caller has loaded: -1 absent (pos: the empty slot), -2 error (status set);
+// kbo receives the slot's b word, candidate mark included.
+__device__ __forceinline__ long long x_find(const Problem &P, IterState *st, unsigned long long a, unsigned long long b,
+                                            ulonglong2 k, unsigned long long &pos, unsigned long long &kbo) {
     const bool both_nonzero = (P.na > 0) && (P.nb > 0);
     for (int probe = 0; probe < P.max_probe; ++probe) {
         const Slot *s = P.table + pos;
-        ulonglong2 k = __ldcg(reinterpret_cast<const ulonglong2 *>(s));         // the key in one request
+        if (probe > 0) k = __ldcg(reinterpret_cast<const ulonglong2 *>(s));      // the key in one request
         int spins = 0;
         while (both_nonzero && ((k.x == 0ull) != (k.y == 0ull))) {   // an insert in flight
             if (++spins > (1 << 20)) { set_status(st, kErrTimeout); return -2; }
             k = __ldcg(reinterpret_cast<const ulonglong2 *>(s));
         }
-        const unsigned long long ka = k.x, kb = k.y;
-        if (ka == a && (kb & kKeyMaskB) == b) { kbo = kb; return (long long)pos; }
-        if (ka == 0ull && kb == 0ull) return -1;
+        if (k.x == a && (k.y & kKeyMaskB) == b) { kbo = k.y; return (long long)pos; }
+        if (k.x == 0ull && k.y == 0ull) return -1;
         pos = (pos + 1) & P.mask;
     }
     set_status(st, kErrTableFull);
     return -2;
 }
+// Claims an empty slot for a key that no other thread inserts (each row occurs
+// once in a column), from pos on; -1 (status set) when there is none.
+__device__ __forceinline__ long long x_claim(const Problem &P, IterState *st, unsigned long long a, unsigned long long b,
+                                             unsigned long long pos) {
+    for (int probe = 0; probe < P.max_probe; ++probe) {
+        unsigned long long oa, ob;
+        cas128(&P.table[pos].a, 0ull, 0ull, a, b, oa, ob);
+        if (oa == 0ull && ob == 0ull) return (long long)pos;
+        pos = (pos + 1) & P.mask;
+    }
+    set_status(st, kErrTableFull);
+    return -1;
+}
 
-__global__ void __launch_bounds__(kXThreads) k_x_scatter(Problem P, XState *xs, IterState *st, double *rows,
-                                                         long long *cand, long long cap_cand, double *gathp) {
+// S += eta (c^T g + g^T c) + eta^2 g^T g,  M += eta (b^T g + g^T b) + eta^2 H_ii g^T g (one entry per thread)
+__device__ void x_update_sm(XState *xs) {
+    const int k1 = xs->k1;
+    const double eta = xs->eta, Hii = xs->Hii;
+    for (int t = threadIdx.x; t < 2 * k1 * k1; t += blockDim.x) {
+        const bool isM = t >= k1 * k1;
+        const int e = isM ? t - k1 * k1 : t, a = e / k1, b = e - a * k1;
+        const double *v = isM ? xs->b_old : xs->c_old;
+        const dd e2 = dd_two_prod(eta, eta);
+        const dd gab = dd_two_prod(xs->g[a], xs->g[b]);
+        const dd q = dd_mul(e2, gab);
+        const dd d = dd_add(dd_mul_d(dd_add(dd_two_prod(v[a], xs->g[b]), dd_two_prod(xs->g[a], v[b])), eta),
+                            isM ? dd_mul_d(q, Hii) : q);
+        dd *to = isM ? xs->M : xs->S;
+        to[e] = dd_add(to[e], d);
+    }
+}
+
+// A single excitation's element as element_value gives it (the same terms in the
+// same order) from the tables W3 and V3, eight loads in flight before their adds.
+__device__ __forceinline__ double x_single(const Problem &P, unsigned long long A, unsigned long long B, const ElemIdx &x) {
+    const size_t row = (size_t)(x.i * P.N + x.a) * P.N;
+    const double *tA = (x.kind == 0 ? P.W3 : P.V3) + row, *tB = (x.kind == 0 ? P.V3 : P.W3) + row;
+    double v = __ldg(P.h + x.i * P.N + x.a);
+    for (unsigned long long mA = A, mB = B; mA | mB;) {
+        double t[8];
+        bool in[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool fa = mA != 0ull;
+            const unsigned long long mm = fa ? mA : mB;
+            in[u] = mm != 0ull;
+            t[u] = in[u] ? __ldg((fa ? tA : tB) + (__ffsll((long long)mm) - 1)) : 0.0;
+            if (fa) mA &= mA - 1; else mB &= mB - 1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (in[u]) v += t[u];
+    }
+    return apply_parity(v, x.sgn);
+}
+
+__global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, IterState *st, double *rows,
+                                                        long long *cand, long long cap_cand, double *gathp,
+                                                        unsigned int *counter) {
     __shared__ ColLists L;
     __shared__ double sw[kXMax];
     __shared__ double sg[kXThreads / 32][kXMax];
     __shared__ unsigned int s_cnt[4][kXThreads / 32];
-    if (xs->eta == 0.0 || st->status) return;                        // no step this iteration
+    __shared__ double red[kXMax][kXThreads];
+    __shared__ bool s_last;
+    if (!xs->go) return;                                             // no step this iteration
+    const int nb = (int)gridDim.x - 1;                               // blocks of the column; one more for S and M
+    if ((int)blockIdx.x == nb) {
+        x_update_sm(xs);
+        return;
+    }
     const int k1 = xs->k1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned long long A = xs->A, B = xs->B;
     build_lists(L, P.N, A, B);
@@ -375,69 +444,90 @@ __global__ void __launch_bounds__(kXThreads) k_x_scatter(Problem P, XState *xs, 
 #pragma unroll
     for (int a = 0; a < kXMax; ++a) gat[a] = 0.0;
     unsigned int c0 = 0, c1 = 0, c2 = 0, c3 = 0;                     // elements, applied, dropped, inserted
-    for (long long e = 1 + (long long)blockIdx.x * blockDim.x + tid; e < nh; e += (long long)gridDim.x * blockDim.x) {
-        unsigned long long oa, ob;
-        const double H = column_element(P, L, A, B, e, oa, ob);
-        if (is_zero(H)) continue;
-        ++c0;
-        // the row at the key's first probe position loads beside the key (it is usually found
-        // there); no other thread of this launch writes row j or the mark of j (each row occurs
-        // once in a column), so the values loaded here are current
-        const unsigned long long pos0 = key_hash(oa, ob) & P.mask;
-        double rc[kXMax], rb[kXMax];
-        x_load_row(rows, (long long)pos0, k1, rc, rb);
-        unsigned long long kb = 0ull;
-        long long s = x_find(P, st, oa, ob, pos0, kb);
-        if (s >= 0 && s != (long long)pos0) x_load_row(rows, s, k1, rc, rb);
-        double cj[kXMax];
-        bool cnz = false;
+    // (whole warps take every round, and the append below is the whole warp's: lanes that inserted and
+    // lanes that found their row come here at different times, and each such group used to wait for
+    // an atomic of its own, a microsecond after the other)
+    for (long long e0 = 1 + (long long)blockIdx.x * blockDim.x + 32 * warp; e0 < nh; e0 += (long long)nb * blockDim.x) {
+        const long long e = e0 + lane;
+        long long s = -1;                                            // the row, where its mark is new
+        if (e < nh) {
+            unsigned long long oa, ob;
+            ElemIdx ix;
+            decode_element(P, L, A, B, e, oa, ob, ix);
+            // the key at its first probe position and the row there (it is usually found there) load
+            // beside the integrals; no other thread of this launch writes row j or the mark of j (each
+            // row occurs once in a column), so the values loaded here are current
+            const unsigned long long pos = key_hash(oa, ob) & P.mask;
+            double rc[kXMax], rb[kXMax];
+            x_load_row(rows, (long long)pos, k1, rc, rb);
+            const ulonglong2 k0 = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + pos));
+            const double H = ix.kind <= 1 ? x_single(P, A, B, ix) : element_value(P, L, ix);
+            long long at = -2;                                       // -2: nothing to do
+            unsigned long long kb = 0ull;
+            if (!is_zero(H)) {
+                ++c0;
+                unsigned long long empty = pos;
+                at = x_find(P, st, oa, ob, k0, empty, kb);           // -1: absent, the empty slot known
+                if (at >= 0 && at != (long long)pos) x_load_row(rows, at, k1, rc, rb);
+                bool cnz = false;
 #pragma unroll
-        for (int a = 0; a < kXMax; ++a) {
-            cj[a] = s >= 0 && a < k1 ? rc[a] : 0.0;
-            cnz = cnz || cj[a] != 0.0;
+                for (int a = 0; a < kXMax; ++a) {
+                    if (at < 0) rc[a] = rb[a] = 0.0;                 // a row that is not there yet is zero
+                    cnz = cnz || (a < k1 && rc[a] != 0.0);
+                }
+                if (at != -2 && !cnz && !(fabs(H) >= thr)) {
+                    ++c2;
+                    at = -2;
+                } else if (at == -1) {
+                    at = x_claim(P, st, oa, ob, empty);              // -1: table full, status set
+                    if (at < 0) at = -2; else { ++c3; kb = ob; }
+                }
+            }
+            if (at >= 0) {
+                ++c1;
+                double *br = rows + at * 2 * k1 + k1;
+                double bn[kXMax];
+#pragma unroll
+                for (int a = 0; a < kXMax; ++a) {
+                    bn[a] = 0.0;
+                    if (a < k1) {                                    // uniform
+                        bn[a] = fma(H, sw[a], rb[a]);
+                        gat[a] = fma(H, rc[a], gat[a]);
+                    }
+                }
+                if ((k1 & 3) == 0) {                                 // 32-byte stores (see x_load_row)
+#pragma unroll
+                    for (int q = 0; q < kXMax / 4; ++q)
+                        if (4 * q < k1)
+                            asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(br + 4 * q), "d"(bn[4 * q]),
+                                         "d"(bn[4 * q + 1]), "d"(bn[4 * q + 2]), "d"(bn[4 * q + 3])
+                                         : "memory");
+                } else if ((k1 & 1) == 0) {                          // 16-byte stores (see x_load_row)
+#pragma unroll
+                    for (int q = 0; q < kXMax / 2; ++q)
+                        if (2 * q < k1) reinterpret_cast<double2 *>(br)[q] = make_double2(bn[2 * q], bn[2 * q + 1]);
+                } else {
+#pragma unroll
+                    for (int a = 0; a < kXMax; ++a)
+                        if (a < k1) br[a] = bn[a];
+                }
+                if (!(kb & kMarkB)) {
+                    P.table[at].b = kb | kMarkB;
+                    s = at;
+                }
+            }
         }
-        if (!cnz && !(fabs(H) >= thr)) { ++c2; continue; }
-        if (s < 0) {
-            bool ins = false;
-            s = table_find(P, st, oa, ob, true, &ins);
-            if (s < 0) continue;                                      // table full: status set
-            if (ins) ++c3;
-            x_load_row(rows, s, k1, rc, rb);
-            kb = __ldcg(&P.table[s].b);
-        }
-        ++c1;
-        double *br = rows + s * 2 * k1 + k1;
-        double bn[kXMax];
-#pragma unroll
-        for (int a = 0; a < kXMax; ++a) {
-            bn[a] = fma(H, sw[a], rb[a]);
-            if (a < k1) gat[a] = fma(H, cj[a], gat[a]);
-        }
-        if ((k1 & 3) == 0) {                                          // 32-byte stores (see x_load_row)
-#pragma unroll
-            for (int q = 0; q < kXMax / 4; ++q)
-                if (4 * q < k1)
-                    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(br + 4 * q), "d"(bn[4 * q]),
-                                 "d"(bn[4 * q + 1]), "d"(bn[4 * q + 2]), "d"(bn[4 * q + 3])
-                                 : "memory");
-        } else if ((k1 & 1) == 0) {                                   // 16-byte stores (see x_load_row)
-#pragma unroll
-            for (int q = 0; q < kXMax / 2; ++q)
-                if (2 * q < k1) reinterpret_cast<double2 *>(br)[q] = make_double2(bn[2 * q], bn[2 * q + 1]);
-        } else {
-#pragma unroll
-            for (int a = 0; a < kXMax; ++a)
-                if (a < k1) br[a] = bn[a];
-        }
-        if (!(kb & kMarkB)) {
-            P.table[s].b = kb | kMarkB;
-            // one reservation for the lanes that get here together (a warp-aggregated append)
-            const cg::coalesced_group grp = cg::coalesced_threads();
+        __syncwarp();
+        const unsigned m = __ballot_sync(0xffffffffu, s >= 0);
+        if (m) {
             int base = 0;
-            if (grp.thread_rank() == 0) base = atomicAdd(&xs->n_cand, (int)grp.size());
-            const int pos = grp.shfl(base, 0) + (int)grp.thread_rank();
-            if (pos < cap_cand) cand[pos] = s;
-            else set_status(st, kErrInternal);
+            if (lane == 0) base = atomicAdd(&xs->n_cand, __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (s >= 0) {
+                const int to = base + __popc(m & ((1u << lane) - 1u));
+                if (to < cap_cand) cand[to] = s;
+                else set_status(st, kErrInternal);
+            }
         }
     }
     // gather: warp tree, then warps in order (fixed order)
@@ -463,38 +553,38 @@ __global__ void __launch_bounds__(kXThreads) k_x_scatter(Problem P, XState *xs, 
         for (int w = 0; w < kXThreads / 32; ++w) t += s_cnt[tid][w];
         if (t) atomicAdd(&xs->cnt[tid], t);
     }
-}
-
-__global__ void __launch_bounds__(kXThreads) k_x_finalize(Problem P, XState *xs, IterState *st, double *rows,
-                                                          const double *gathp, int nblocks, long long *cand,
-                                                          long long cap_cand) {
-    __shared__ double red[kXMax][kXThreads];
-    if (xs->eta == 0.0 || st->status) return;                        // no step this iteration
-    const int k1 = xs->k1, tid = threadIdx.x;
+    // the last block: B_i recalculated, the row's mark, the counters
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(counter, 1u) == (unsigned)nb - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) *counter = 0u;
+    if (st->status) return;
     const long long s = xs->slot;
     const double Hii = xs->Hii;
     // every state at once: per state, the thread's blocks in order, then the same pairwise tree
     double v[kXMax];
 #pragma unroll
     for (int a = 0; a < kXMax; ++a) v[a] = 0.0;
-    for (int k = tid; k < nblocks; k += blockDim.x) {
+    for (int k = tid; k < nb; k += blockDim.x) {
 #pragma unroll
         for (int a = 0; a < kXMax; ++a)
-            if (a < k1) v[a] += gathp[(size_t)k * k1 + a];
+            if (a < k1) v[a] += __ldcg(gathp + (size_t)k * k1 + a);
     }
 #pragma unroll
     for (int a = 0; a < kXMax; ++a)
         if (a < k1) red[a][tid] = v[a];
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (tid < w) {
+    // (256 partial sums per state: warp a adds state a's, 8 per lane in order, then a tree)
+    if (warp < k1) {
+        double t = 0.0;
 #pragma unroll
-            for (int a = 0; a < kXMax; ++a)
-                if (a < k1) red[a][tid] += red[a][tid + w];
-        }
-        __syncthreads();
+        for (int q = 0; q < kXThreads / 32; ++q) t += red[warp][32 * q + lane];
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+        if (lane == 0) rows[s * 2 * k1 + k1 + warp] = fma(Hii, __ldcg(rows + s * 2 * k1 + warp), t);
     }
-    if (tid < k1) rows[s * 2 * k1 + k1 + tid] = fma(Hii, rows[s * 2 * k1 + tid], red[tid][0]);
     if (tid == 0) {
         const unsigned long long kb = P.table[s].b;
         if (!(kb & kMarkB)) {
@@ -504,12 +594,14 @@ __global__ void __launch_bounds__(kXThreads) k_x_finalize(Problem P, XState *xs,
             else set_status(st, kErrInternal);
         }
         const long long nd = Hii != 0.0 ? 1 : 0;
-        xs->elements += (long long)xs->cnt[0] + nd;
-        xs->applied += (long long)xs->cnt[1] + nd;
-        xs->dropped += (long long)xs->cnt[2];
-        xs->inserted += (long long)xs->cnt[3];
-        xs->n_slots += (long long)xs->cnt[3];
-        xs->last_column = (long long)xs->cnt[0] + nd;
+        const long long n0 = (long long)__ldcg(&xs->cnt[0]), n1 = (long long)__ldcg(&xs->cnt[1]);
+        const long long n2 = (long long)__ldcg(&xs->cnt[2]), n3 = (long long)__ldcg(&xs->cnt[3]);
+        xs->elements += n0 + nd;
+        xs->applied += n1 + nd;
+        xs->dropped += n2;
+        xs->inserted += n3;
+        xs->n_slots += n3;
+        xs->last_column = n0 + nd;
         for (int k = 0; k < 4; ++k) xs->cnt[k] = 0ull;
         if (xs->n_slots > P.max_entries) set_status(st, kErrTableFull);
     }
@@ -654,22 +746,31 @@ cudaError_t launch_x_diag_list(const Problem &P, const unsigned long long *keys,
     return cudaGetLastError();
 }
 
-int x_scatter_blocks() { return 152 * 2; }
+// blocks of a column: an element per thread, at most two blocks per SM; of the choice: a candidate
+// per thread, at most one block per SM
+int x_scatter_blocks(const Problem &P) {
+    const long long nh = P.doubles_vanish ? P.seg[2] : P.seg[5];
+    return (int)std::max<long long>(1, std::min<long long>(152 * 2, (nh - 1 + kXThreads - 1) / kXThreads));
+}
+int x_select_blocks(const Problem &P) { return std::min(152, x_scatter_blocks(P)); }
 
 size_t x_block_bytes() { return sizeof(XBest); }
 
-cudaError_t launch_x_start(const Problem &P, const XBuffers &b, unsigned long long A, unsigned long long B, int k,
-                           cudaStream_t s) {
-    k_x_prepare<<<1, 32, 0, s>>>(P, b.xs, b.st, b.rows, k, A, B);
-    k_x_scatter<<<b.nscatter, kXThreads, 0, s>>>(P, b.xs, b.st, b.rows, b.cand, b.cap_cand, b.gathp);
-    k_x_finalize<<<1, kXThreads, 0, s>>>(P, b.xs, b.st, b.rows, b.gathp, b.nscatter, b.cand, b.cap_cand);
+static cudaError_t launch_x_column(const Problem &P, const XBuffers &b, cudaStream_t s) {
+    k_x_column<<<b.nscatter + 1, kXThreads, 0, s>>>(P, b.xs, b.st, b.rows, b.cand, b.cap_cand, b.gathp, b.counter + 1);
     return cudaGetLastError();
 }
 
+cudaError_t launch_x_start(const Problem &P, const XBuffers &b, unsigned long long A, unsigned long long B, int k,
+                           cudaStream_t s) {
+    k_x_choose<<<1, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.rows, static_cast<XBest *>(b.bbest), b.counter, k, A, B);
+    return launch_x_column(P, b, s);
+}
+
 cudaError_t launch_x_iteration(const Problem &P, const XBuffers &b, cudaStream_t s) {
-    k_x_select<<<b.nselect, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.rows, static_cast<XBest *>(b.bbest),
-                                              b.counter);
-    return launch_x_start(P, b, 0ull, 0ull, -1, s);
+    k_x_choose<<<b.nselect, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.rows, static_cast<XBest *>(b.bbest), b.counter,
+                                               -1, 0ull, 0ull);
+    return launch_x_column(P, b, s);
 }
 
 cudaError_t launch_x_energies(const XBuffers &b, cudaStream_t s) {
