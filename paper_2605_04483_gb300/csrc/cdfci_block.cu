@@ -1292,17 +1292,20 @@ __device__ void eig_stream(const float *Rh, const float *Rl, int ldr, int n1, in
     if (late) set_status(st, kErrTimeout);
 }
 
-// The reduced problem above kRegMaxN rows.  CL = false: one CTA, R streamed from
-// global memory; CL = true: a cluster of C CTAs, CTA r holding rows [r crows, (r + 1) crows) of R in its shared memory, the
+// The reduced problem above kRegMaxN rows, and of the first, short blocks of a
+// run (see eigen_short).  CL = false: one CTA, R in its shared memory when SM
+// (row stride ldr there, ldg in global memory; otherwise the two are the same),
+// else streamed from global memory; CL = true: a cluster of C CTAs, CTA r holding
+// rows [r crows, (r + 1) crows) of R in its shared memory, the
 // vectors x and w gathered in full in every CTA before each product, the sums
 // taken over the cluster.  Every CTA computes the scalar steps itself, from
 // the same sums in the same order, so they agree bit for bit.
-template <bool CL>
-__global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, IterState *st, const McSel *sel,
-                                                       const double *cI, const double *bI, const double *HIIc,
-                                                       const double *Hdiag, const float4 *rowf, float *Rh, float *Rl,
-                                                       int ldr, int tpr, int crows, double *w,
-                                                       double *thr, double *etaout, long long *cand) {
+template <bool CL, bool SM>
+__device__ __forceinline__ void eigen_rows(const Problem &P, McState *ms, IterState *st, const McSel *sel,
+                                           const double *cI, const double *bI, const double *HIIc,
+                                           const double *Hdiag, const float4 *rowf, float *Rh, float *Rl, int ldg,
+                                           int ldr, int tpr, int crows, double *w, double *thr, double *etaout,
+                                           long long *cand) {
     extern __shared__ __align__(16) float sm[];
     __shared__ float s_rf[2 * 32 * 16];
     __shared__ ff s_rff[2 * 32 * 2];
@@ -1322,7 +1325,7 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
     const int m = ms->m_sel, n1 = m + 1;
     // this CTA's rows of R (absolute indices [a0, a1)); one CTA: all
     const int a0 = CL ? (int)rank * crows : 0, a1 = CL ? min(a0 + crows, n1) : n1;
-    constexpr bool in_smem = CL;
+    constexpr bool in_smem = CL || SM;
     // the state scalars, loaded (thread 0) ahead of the sums; read after the barriers below
     __shared__ dd s_mu0, s_al0, s_sc0;
     __shared__ long long s_nnz0;
@@ -1340,8 +1343,15 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
     if (in_smem && tid == 0 && nown > 0) {
         const unsigned bytes = (unsigned)nown * (unsigned)ldr * 4u;
         mbar_init_arm(&s_bar, 2u * bytes);
-        bulk_g2s(sh, Rh + (size_t)a0 * ldr, bytes, &s_bar);
-        bulk_g2s(sl, Rl + (size_t)a0 * ldr, bytes, &s_bar);
+        if (CL) {
+            bulk_g2s(sh, Rh + (size_t)a0 * ldr, bytes, &s_bar);
+            bulk_g2s(sl, Rl + (size_t)a0 * ldr, bytes, &s_bar);
+        } else {                                        // a row at a time (ldr <= ldg)
+            for (int a = 0; a < nown; ++a) {
+                bulk_g2s(sh + (size_t)a * ldr, Rh + (size_t)a * ldg, (unsigned)ldr * 4u, &s_bar);
+                bulk_g2s(sl + (size_t)a * ldr, Rl + (size_t)a * ldg, (unsigned)ldr * 4u, &s_bar);
+            }
+        }
     }
     // R in global memory: two stage buffers for the streamed products, their barriers armed later
     __shared__ unsigned long long s_sbar[2];
@@ -1742,6 +1752,38 @@ __global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, I
                                                 (unsigned long long)(long long)dn);
 }
 
+template <bool CL>
+__global__ void __launch_bounds__(kEigMaxN) k_mc_eigen(Problem P, McState *ms, IterState *st, const McSel *sel,
+                                                       const double *cI, const double *bI, const double *HIIc,
+                                                       const double *Hdiag, const float4 *rowf, float *Rh, float *Rl,
+                                                       int ldr, int tpr, int crows, double *w,
+                                                       double *thr, double *etaout, long long *cand) {
+    eigen_rows<CL, false>(P, ms, st, sel, cI, bI, HIIc, Hdiag, rowf, Rh, Rl, ldr, ldr, tpr, crows, w, thr, etaout,
+                          cand);
+}
+// The short blocks that start a run: fewer candidates than the block's m, so all
+// are taken, and what follows can be a choice among coordinates whose gradient
+// this solve has just made zero up to rounding.  For these the solver that keeps
+// both parts of R in shared memory stays in use (two threads a row): runs from
+// one determinant keep the trajectory that its rounding gives them, down to a
+// 6-site ring whose third block takes 12 of 128 coordinates that way.  It takes
+// blocks that fit the shared memory of the registers' solver, whose launch it
+// shares (m = 128: up to 101 rows; twice that memory would cost it 2.5 us an
+// iteration in L1 space).
+__host__ __device__ __forceinline__ int eig_short_ldr(int n1) { return eig_len(n1) + 4; }
+__device__ __forceinline__ bool eig_short_fits(int n1, int crows, int ldr) {
+    return 2 * n1 * eig_short_ldr(n1) + (int)eig_vec_floats(n1) <= crows * ldr + 9 * eig_len(crows) &&
+           eig_short_ldr(n1) <= ldr && 2 * n1 <= (int)blockDim.x;
+}
+__device__ __noinline__ void eigen_short(const Problem &P, McState *ms, IterState *st, const McSel *sel,
+                                         const double *cI, const double *bI, const double *HIIc, const double *Hdiag,
+                                         const float4 *rowf, float *Rh, float *Rl, int ldr, double *w, double *thr,
+                                         double *etaout, long long *cand) {
+    const int n1 = ms->m_sel + 1;
+    eigen_rows<false, true>(P, ms, st, sel, cI, bI, HIIc, Hdiag, rowf, Rh, Rl, ldr, eig_short_ldr(n1), 2, n1, w, thr,
+                            etaout, cand);
+}
+
 // ---------------------------------------------------------------------------
 // The reduced problem for n1 <= kRegMaxN: the same iteration with the FP32 part
 // of R in registers.  What bounds it is latency: a chain of products, sums and
@@ -1892,12 +1934,13 @@ template <bool CL>
 __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState *ms, IterState *st, const McSel *sel,
                                                               const double *cI, const double *bI, const double *HIIc,
                                                               const double *Hdiag, const float4 *rowf,
-                                                              const float *Rh, const float *Rl, int ldr, int tpr,
+                                                              float *Rh, float *Rl, int ldr, int tpr,
                                                               int crows, double *w, double *thr, double *etaout,
                                                               long long *cand) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ __align__(16) float s_r2[2][kRegSlots * 16];
-    __shared__ ff s_rff[kRegSlots * 2];
+    constexpr int kSlots = CL ? kRegSlots : kRegThreads / 32;   // warps of the cluster
+    __shared__ __align__(16) float s_r2[2][kSlots * 16];
+    __shared__ ff s_rff[kSlots * 2];
     __shared__ double s_red[32 * 4];
     __shared__ ff s_row0[6];                            // nu, R_00, (A x)_0 of the start, 1 / nu; theta and x.x of the start
     __shared__ ff s_x0;                                 // x_0 at the end (CL: from CTA 0)
@@ -1908,6 +1951,10 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
     __shared__ int s_nzr[32], s_flag, s_zero, s_late[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     if (ms->done || st->status) return;
+    if (!CL && ms->m_sel + 1 < crows && eig_short_fits(ms->m_sel + 1, crows, ldr)) {   // crows = m + 1: one CTA
+        eigen_short(P, ms, st, sel, cI, bI, HIIc, Hdiag, rowf, Rh, Rl, ldr, w, thr, etaout, cand);
+        return;
+    }
     unsigned rank = 0, C = 1;
     if (CL) {
         rank = cg::this_cluster().block_rank();
@@ -3120,7 +3167,9 @@ size_t mc_eigen_smem(int m) {
 }
 int mc_eigen_threads(int m) {
     const EigCfg g = eig_cfg(m + 1);
-    return g.reg ? 32 * ((g.tpr * ((g.crows + kRegRows - 1) / kRegRows) + 31) / 32) : g.tpr * 32 * ((g.crows + 31) / 32);
+    if (!g.reg) return g.tpr * 32 * ((g.crows + 31) / 32);
+    const int t = 32 * ((g.tpr * ((g.crows + kRegRows - 1) / kRegRows) + 31) / 32);
+    return g.C > 1 ? t : std::max(t, 32 * ((2 * g.crows + 31) / 32));   // (eigen_short: 2 threads a row)
 }
 int mc_eigen_cluster(int m) { return eig_cfg(m + 1).C; }
 int mc_ldr(int m) { return eig_ldr(m + 1); }
@@ -3250,8 +3299,7 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
         if (g.reg)
             cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen_reg<true> : k_mc_eigen_reg<false>, P, b.ms, b.st,
                                (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
-                               (const double *)b.Hdiag, (const float4 *)b.rowf, (const float *)b.Rh,
-                               (const float *)b.Rl, b.ldr, g.tpr, g.crows, b.w, b.thr, b.eta, b.cand);
+                               (const double *)b.Hdiag, (const float4 *)b.rowf, b.Rh, b.Rl, b.ldr, g.tpr, g.crows, b.w, b.thr, b.eta, b.cand);
         else
             cudaLaunchKernelEx(&cfg, g.C > 1 ? k_mc_eigen<true> : k_mc_eigen<false>, P, b.ms, b.st,
                                (const McSel *)b.sel, (const double *)b.cI, (const double *)b.bI, (const double *)b.HIIc,
