@@ -153,7 +153,9 @@ int maybe_raise_tau(cdfci_ctx *c, bool *changed) {
     return CDFCI_OK;
 }
 
-int run_iterations(cdfci_ctx *c, long long n) {
+// n iterations of the m = 1 loop; force (optional): start-vector entries, at most as many as the first
+// launch has iterations
+int run_iterations(cdfci_ctx *c, long long n, ForceList force = ForceList{}) {
     const long long chunk = c->prm.z_threshold_search ? std::min<long long>(c->chunk, 1024) : c->chunk;
     while (n > 0) {
         bool changed = false;
@@ -163,9 +165,10 @@ int run_iterations(cdfci_ctx *c, long long n) {
         if (c->gridmode)
             CK(launch_cd_loop_grid(c->P, c->d_st, c->d_rec, c->d_part,
                                    reinterpret_cast<unsigned long long *>(c->d_part + c->grid), c->d_bar, c->grid, k,
-                                   c->stream));
+                                   force, c->stream));
         else
-            CK(launch_cd_loop(c->P, c->d_st, c->d_rec, c->d_part, c->grid, k, c->stream));
+            CK(launch_cd_loop(c->P, c->d_st, c->d_rec, c->d_part, c->grid, k, force, c->stream));
+        force = ForceList{};
         n -= k;
     }
     return CDFCI_OK;
@@ -1458,10 +1461,14 @@ CDFCI_API int cdfci_set_initial(cdfci_handle c, const uint64_t *keys, const doub
     if (rc) return rc;
     if (!c->block) {
         CK(launch_init_state(c->d_st, c->d_rec, hk[0], hk[1], hc[0], c->stream));
-        rc = run_iterations(c, 1);
-        for (int64_t k = 1; !rc && k < n; ++k) {
-            CK(launch_force_next(c->d_rec, dk, dc, k, c->stream));
-            rc = run_iterations(c, 1);
+        // a launch takes as many entries as iterations (with z_threshold_search one, tau is looked at
+        // before each); the first one of every later launch is put into the record
+        const long long most = c->prm.z_threshold_search ? 1 : c->chunk;
+        for (int64_t k = 0; !rc && k < n;) {
+            const long long take = std::min<long long>(most, n - k);
+            if (k > 0) CK(launch_force_next(c->d_rec, dk, dc, k, c->stream));
+            rc = run_iterations(c, take, ForceList{dk + 2 * k, dc + k, take});
+            k += take;
         }
         if (rc) return rc;
     } else {

@@ -121,27 +121,32 @@ __device__ __forceinline__ double diag_pairs_warp(const Problem &P, const ColLis
                                                   const double *sJ, const double *sK, const unsigned short *pairs,
                                                   int npairs) {
     const int lane = threadIdx.x & 31, N = P.N, na = P.na, n = P.na + P.nb;
-    double y0 = 0.0, y1 = 0.0, y2 = 0.0, y3 = 0.0;
-    for (int k0 = lane; k0 < npairs; k0 += 128) {
-        double t[4];
+    double y[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b0 = 0; b0 < npairs; b0 += 128) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const int k = k0 + 32 * r;
-            t[r] = 0.0;
+            if (b0 + 32 * r >= npairs) break;          // uniform: a block of 32 pairs that no lane has
+            const int k = b0 + 32 * r + lane;
+            double t = 0.0;
             if (k < npairs) {
                 const unsigned pr = pairs[k];
                 const int u = pr & 0x7f, w = (pr >> 7) & 0x7f;
                 const int p = u < na ? L.occA[u] : L.occB[u - na];
                 const int q = w < na ? L.occA[w] : L.occB[w - na];
                 const double jv = sJ[p * N + q];
-                t[r] = (pr >> 14) ? jv - sK[p * N + q] : jv;
+                t = (pr >> 14) ? jv - sK[p * N + q] : jv;
             }
+            y[r] = b0 == 0 ? t : y[r] + t;
         }
-        y0 += t[0]; y1 += t[1]; y2 += t[2]; y3 += t[3];
     }
     double x = 0.0;
-    for (int u = lane; u < n; u += 32) x += sHd[u < na ? L.occA[u] : L.occB[u - na]];
-    x += (y0 + y1) + (y2 + y3);
+    for (int u = lane; u < n; u += 32) {
+        const double hv = sHd[u < na ? L.occA[u] : L.occB[u - na]];
+        x = u == lane ? hv : x + hv;
+    }
+    if (npairs > 64) y[0] = (y[0] + y[1]) + (y[2] + y[3]);
+    else if (npairs > 32) y[0] += y[1];
+    x += y[0];
     for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
     return __shfl_sync(0xffffffffu, x, 0);
 }
@@ -301,21 +306,25 @@ struct LoopState {
 
 // Warp-level combine: argmax of (gbits desc, key asc) with payload (slot, b, c),
 // sums of the counters and a lane-ordered sum of the nonzero gather values;
-// every lane returns the result.  The maximum of gbits comes from a
-// butterfly on gbits alone; only exact ties look at the keys.  The gather's
-// fixed shuffle-down tree (skipped when every lane holds 0) runs level by level
-// beside the butterfly, so their latencies overlap.
-__device__ __forceinline__ void warp_combine(Best &best, double &bb, double &cb, double &gather, int cnt[4], int &err) {
+// every lane returns the result.  The maximum of gbits comes from two 32-bit
+// warp reductions (high words, then the low words that go with the highest);
+// only exact ties look at the keys.  The gather's fixed shuffle-down tree is
+// skipped when every lane holds 0, and its levels above the `lanes` (uniform)
+// that hold anything are left out: they would add zeros.  A level is a shuffle
+// and an FP64 addition, whose issue takes the warp's scheduler 64 cycles.
+__device__ __forceinline__ void warp_combine(Best &best, double &bb, double &cb, double &gather, int cnt[4], int &err,
+                                             int lanes = 32) {
     const bool any_g = __any_sync(0xffffffffu, !is_zero(gather));
     for (int k = 0; k < 4; ++k) cnt[k] = __reduce_add_sync(0xffffffffu, (unsigned)cnt[k]);
     err = (int)__reduce_or_sync(0xffffffffu, (unsigned)err);
-    unsigned long long gmax = best.g;
+    const unsigned int ghi = (unsigned int)(best.g >> 32);
+    const unsigned int mhi = __reduce_max_sync(0xffffffffu, ghi);
+    const unsigned int mlo = __reduce_max_sync(0xffffffffu, ghi == mhi ? (unsigned int)best.g : 0u);
+    const unsigned long long gmax = ((unsigned long long)mhi << 32) | mlo;
+    if (any_g) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, gmax, off);
-        const double t = __shfl_down_sync(0xffffffffu, gather, off);
-        if (any_g) gather += t;
-        gmax = y > gmax ? y : gmax;
+        for (int off = 16; off > 0; off >>= 1)
+            if (off < lanes) gather += __shfl_down_sync(0xffffffffu, gather, off);
     }
     const unsigned int cand = __ballot_sync(0xffffffffu, best.g == gmax && best.slot >= 0);
     int win = cand ? __ffs(cand) - 1 : 0;
@@ -473,7 +482,8 @@ __device__ __forceinline__ void fold_partial(const CdPartial &x, bool first, Bes
 // written once every CTA has published its last one).
 template <bool kGrid, int kE>
 __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, CdRecord *rec, CdPartial *gpart,
-                                             unsigned long long *xchg, GridRound *rnd, long long n_iter) {
+                                             unsigned long long *xchg, GridRound *rnd, long long n_iter,
+                                             const ForceList &F) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     const int G = kGrid ? (int)gridDim.x : (int)cluster.num_blocks();
@@ -547,9 +557,26 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
     const int n_own = rank < nqs ? (nqs - 1 - rank) / G + 1 : 0;
     const int tb = min(min(n_own, lay.tb_max), Wp * kE);
     const int nterms = tb * 32 * (nocc + 1);
+    // The double-double books of an iteration, by two lanes of warp 2 beside the control warp's next
+    // choice (mu is read after the line search, behind the barrier that follows the choice), not in
+    // front of the iteration's last barrier: the chain of about 35 dependent FP64 operations takes
+    // some 2400 cycles (with that and the shorter combines, a N = 8 run of one CTA went from 7.79 to
+    // 7.39 us an iteration, of 57 CTAs from 13.1 to 12.6).  Lane 0: mu += 2 eta c_i + eta^2; lane 1: alpha += 2 eta b_i + eta^2 H_ii.
+    double bk_eta = 0.0, bk_y1 = 0.0, bk_y2 = 0.0;
+    bool bk_due = false;                               // uniform
+    auto books = [&]() {
+        if (warp == 2 && lane < 2) {
+            const dd x0 = lane == 0 ? ls.mu : ls.alpha;
+            const dd t = dd_add_fast(dd_two_prod(2.0 * bk_eta, bk_y1), dd_mul_d(dd_two_prod(bk_eta, bk_eta), bk_y2));
+            const dd r = dd_add_fast(x0, t);
+            if (lane == 0) ls.mu = r; else ls.alpha = r;
+        }
+    };
     int lastp = 1;
     for (long long it = 0; it < n_iter; ++it) {
         const int pin = lastp, pout = lastp ^ 1;
+        if (bk_due) books();
+        bk_due = false;
         // ---- choice of i (Eq. choose-i), by the control warp ----
         // every CTA's partial of the last column: lane l of the control warp folds CTAs l, l + 32, ...
         // (all lanes take part in the combine)
@@ -594,7 +621,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                         if (two) fold_partial(x1, false, bb, bj, cj, gsum, cnt, err);
                     }
                 }
-                warp_combine(bb, bj, cj, gsum, cnt, err);
+                if (G > 1) warp_combine(bb, bj, cj, gsum, cnt, err, G < 32 ? G : 32);   // one CTA: lane 0 has it all
             }
             if (tmo) {
                 if (lane == 0) {
@@ -817,16 +844,10 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             if (err) atomicOr(&s_err, 1);
         }
         __syncthreads();
-        if (warp == 1 && lane < 2) {
-            // beside the control warp's combine, on another scheduler and with the FP64 pipe of the
-            // element warps idle: lane 0: mu += 2 eta c_i + eta^2; lane 1: alpha += 2 eta b_i +
-            // eta^2 H_ii (double-double); read by the next iteration after the barrier
-            const dd x0 = lane == 0 ? ls.mu : ls.alpha;
-            const double y1 = lane == 0 ? sel.ci : sel.bi;
-            const double y2 = lane == 0 ? 1.0 : s_hii;
-            const dd t = dd_add_fast(dd_two_prod(2.0 * eta, y1), dd_mul_d(dd_two_prod(eta, eta), y2));
-            const dd r = dd_add_fast(x0, t);
-            if (lane == 0) ls.mu = r; else ls.alpha = r;
+        if (warp == 2 && lane < 2) {                   // what books() takes, before the choice overwrites it
+            bk_eta = eta;
+            bk_y1 = lane == 0 ? sel.ci : sel.bi;
+            bk_y2 = lane == 0 ? 1.0 : s_hii;
         }
         if (warp == 0) {
             const bool have = lane < kCdWarps;
@@ -836,7 +857,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             int c4[4] = {have ? r_cnt[0][lane] : 0, have ? r_cnt[1][lane] : 0, have ? r_cnt[2][lane] : 0,
                          have ? r_cnt[3][lane] : 0};
             int e2 = 0;
-            warp_combine(b, bj, cj, gs, c4, e2);
+            warp_combine(b, bj, cj, gs, c4, e2, kCdWarps);
             if (lane == 0) {
                 CdPartial pp;
                 pp.gbits = b.g; pp.ka = b.a; pp.kb = b.b; pp.slot = b.slot;
@@ -871,7 +892,12 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 }
                 const bool z0 = is_zero(ci), z1 = is_zero(ci_new);
                 ls.nnz_c += ((z0 && !z1) ? 1 : 0) - ((!z0 && z1) ? 1 : 0);
-                ls.forced = 0;
+                ls.forced = it + 1 < F.n ? 1 : 0;
+                if (it + 1 < F.n) {                    // a start vector's next entry
+                    ls.fa = __ldg(F.keys + 2 * (it + 1));
+                    ls.fb = __ldg(F.keys + 2 * (it + 1) + 1);
+                    ls.feta = __ldg(F.c + it + 1);
+                }
                 ls.have_prev = 1;
                 s_done = ls.done;
             }
@@ -885,8 +911,11 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             cluster.sync();                           // partials and table writes visible cluster-wide
         }
         lastp = pout;
+        bk_due = true;
         if (s_done || bad) break;                     // identical in every CTA
     }
+    if (bk_due) books();
+    __syncthreads();                                  // the books before the record
 
     // ---- state for the next launch / the finalisation ----
     if (kGrid && n_pub > 0 && warp == 0 && !s_tmo) {
@@ -926,16 +955,16 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
 // threads covers the column (the smaller loop body is faster), else kCdMaxE.
 template <int kE>
 __global__ void __launch_bounds__(kCdThreads, 1) k_cd_loop(Problem P, IterState *st, CdRecord *rec,
-                                                           CdPartial *gpart, long long n_iter) {
-    cd_loop_body<false, kE>(P, st, rec, gpart, nullptr, nullptr, n_iter);
+                                                           CdPartial *gpart, long long n_iter, ForceList F) {
+    cd_loop_body<false, kE>(P, st, rec, gpart, nullptr, nullptr, n_iter, F);
 }
 
 // the loop over every CTA of a cooperative launch (see cd_loop_body)
 template <int kE>
 __global__ void __launch_bounds__(kCdThreads, 1) k_cd_loop_grid(Problem P, IterState *st, CdRecord *rec,
                                                                 CdPartial *gpart, unsigned long long *xchg,
-                                                                GridRound *rnd, long long n_iter) {
-    cd_loop_body<true, kE>(P, st, rec, gpart, xchg, rnd, n_iter);
+                                                                GridRound *rnd, long long n_iter, ForceList F) {
+    cd_loop_body<true, kE>(P, st, rec, gpart, xchg, rnd, n_iter, F);
 }
 
 // Many independent problems in one launch: cluster k (blocks k*G .. k*G+G-1)
@@ -950,7 +979,7 @@ __global__ void __launch_bounds__(kCdThreads, 1) k_cd_loop_batch(const CdInstanc
     for (int t = threadIdx.x; t < (int)(sizeof(Problem) / 8); t += blockDim.x)
         reinterpret_cast<unsigned long long *>(&sP)[t] = reinterpret_cast<const unsigned long long *>(&inst[k].P)[t];
     __syncthreads();
-    cd_loop_body<false, kCdMaxE>(sP, inst[k].st, inst[k].rec, inst[k].part, nullptr, nullptr, n_iter);
+    cd_loop_body<false, kCdMaxE>(sP, inst[k].st, inst[k].rec, inst[k].part, nullptr, nullptr, n_iter, ForceList{});
 }
 
 // After a batch of iterations: write the pending recalculated b_i of the last
@@ -1325,7 +1354,7 @@ static bool cd_one_round(const Problem &P, int G) {
 }
 
 cudaError_t launch_cd_loop(const Problem &P, IterState *st, CdRecord *rec, CdPartial *part, int cluster,
-                           long long n_iter, cudaStream_t s) {
+                           long long n_iter, const ForceList &F, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster);
     cfg.blockDim = dim3(kCdThreads);
@@ -1338,8 +1367,8 @@ cudaError_t launch_cd_loop(const Problem &P, IterState *st, CdRecord *rec, CdPar
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cd_one_round(P, cluster)) return cudaLaunchKernelEx(&cfg, k_cd_loop<1>, P, st, rec, part, n_iter);
-    return cudaLaunchKernelEx(&cfg, k_cd_loop<kCdMaxE>, P, st, rec, part, n_iter);
+    if (cd_one_round(P, cluster)) return cudaLaunchKernelEx(&cfg, k_cd_loop<1>, P, st, rec, part, n_iter, F);
+    return cudaLaunchKernelEx(&cfg, k_cd_loop<kCdMaxE>, P, st, rec, part, n_iter, F);
 }
 
 cudaError_t launch_cd_loop_batch(const CdInstance *inst, int n_inst, int cluster, size_t smem, long long n_iter,
@@ -1374,7 +1403,8 @@ cudaError_t launch_cd_finalize_batch(const CdInstance *inst, int n_inst, int clu
 // holds G partials, xchg 2 G kXchgWords zero-initialised words, rnd a
 // zero-initialised GridRound (both kept between launches).
 cudaError_t launch_cd_loop_grid(const Problem &P, IterState *st, CdRecord *rec, CdPartial *gpart,
-                                unsigned long long *xchg, GridRound *rnd, int G, long long n_iter, cudaStream_t s) {
+                                unsigned long long *xchg, GridRound *rnd, int G, long long n_iter, const ForceList &F,
+                                cudaStream_t s) {
     if (G < 1) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(G);
@@ -1386,8 +1416,8 @@ cudaError_t launch_cd_loop_grid(const Problem &P, IterState *st, CdRecord *rec, 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cd_one_round(P, G)) return cudaLaunchKernelEx(&cfg, k_cd_loop_grid<1>, P, st, rec, gpart, xchg, rnd, n_iter);
-    return cudaLaunchKernelEx(&cfg, k_cd_loop_grid<kCdMaxE>, P, st, rec, gpart, xchg, rnd, n_iter);
+    if (cd_one_round(P, G)) return cudaLaunchKernelEx(&cfg, k_cd_loop_grid<1>, P, st, rec, gpart, xchg, rnd, n_iter, F);
+    return cudaLaunchKernelEx(&cfg, k_cd_loop_grid<kCdMaxE>, P, st, rec, gpart, xchg, rnd, n_iter, F);
 }
 
 // The largest CTA count of the grid-wide loop that can be co-resident (0 if none).

@@ -6,8 +6,16 @@
 
 namespace cdfci {
 
+// Start-vector entries that a launch of the m = 1 loop takes as forced steps: entry
+// k in its iteration k (entry 0 is already in the record); n <= n_iter.  The arrays
+// (device) are read during that launch only.
+struct ForceList {
+    const unsigned long long *keys = nullptr;
+    const double *c = nullptr;
+    long long n = 0;
+};
 cudaError_t launch_cd_loop(const Problem &P, IterState *st, CdRecord *rec, CdPartial *part, int cluster,
-                           long long n_iter, cudaStream_t s);
+                           long long n_iter, const ForceList &F, cudaStream_t s);
 size_t cd_dynamic_smem(const Problem &P);
 int cd_pick_cluster(int want, size_t smem);
 cudaError_t launch_cd_finalize(const Problem &P, IterState *st, CdRecord *rec, CdPartial *part, int cluster,
@@ -118,7 +126,8 @@ cudaError_t launch_mc_iteration(const Problem &P, const McBuffers &b, cudaStream
 
 // the m = 1 loop over more CTAs than a cluster holds (cooperative launch)
 cudaError_t launch_cd_loop_grid(const Problem &P, IterState *st, CdRecord *rec, CdPartial *gpart,
-                                unsigned long long *xchg, GridRound *rnd, int G, long long n_iter, cudaStream_t s);
+                                unsigned long long *xchg, GridRound *rnd, int G, long long n_iter, const ForceList &F,
+                                cudaStream_t s);
 int cd_max_grid(size_t smem);
 
 // batches of independent m = 1 problems: one launch, one cluster per instance
