@@ -633,8 +633,10 @@ __device__ __forceinline__ float cbrt_seed(float x) {
 // whose quartic is symmetric about -c_i): decided in single precision when
 // the distances differ by more than 1e-4 of their sum, else on the FP64
 // roots through the quartic's values and that identity.
-__device__ __forceinline__ double line_search(double v1, double v2, double v3) {
-    const float f1 = (float)v1, f2 = (float)v2, f3 = (float)v3;
+// f1 .. f3 are v1 .. v3 rounded to single precision; halley(x) = halley_cubic((double)x, v1, v2, v3).
+template <class Halley>
+__device__ __forceinline__ double line_search_from(float f1, float f2, float f3, double v1, double v2, double v3,
+                                                   const Halley &halley) {
     const float b = 3.0f * f3, c = 2.0f * f2, d = f1;
     const float sh = b * (1.0f / 12.0f);
     const float p = (12.0f * c - b * b) * (1.0f / 48.0f);
@@ -644,7 +646,7 @@ __device__ __forceinline__ double line_search(double v1, double v2, double v3) {
     if (!(del < 0.0f) || !(p < 0.0f)) {
         const float sd = sqrtf(fmaxf(del, 0.0f));
         const float x = cbrt_seed(-hq + sd) + cbrt_seed(-hq - sd) - sh;
-        return halley_cubic((double)newton_f32(x, f1, f2, f3), v1, v2, v3);
+        return halley(newton_f32(x, f1, f2, f3));
     }
     const float m = 2.0f * sqrtf(-tp);
     float arg = (3.0f * q / (2.0f * p)) * sqrtf(-3.0f / p);
@@ -654,15 +656,54 @@ __device__ __forceinline__ double line_search(double v1, double v2, double v3) {
     const float x2 = m * cosf(th - 2.09439510239319549f);
     const float x1 = m * cosf(th - 4.18879020478639098f);
     const float d1 = x2 - x1, d3 = x3 - x2;
-    if (d3 - d1 > 1e-4f * (d1 + d3)) return halley_cubic((double)newton_f32(x3 - sh, f1, f2, f3), v1, v2, v3);
-    if (d1 - d3 > 1e-4f * (d1 + d3)) return halley_cubic((double)newton_f32(x1 - sh, f1, f2, f3), v1, v2, v3);
-    const double r1 = halley_cubic((double)newton_f32(x1 - sh, f1, f2, f3), v1, v2, v3);
-    const double r3 = halley_cubic((double)newton_f32(x3 - sh, f1, f2, f3), v1, v2, v3);
+    if (d3 - d1 > 1e-4f * (d1 + d3)) return halley(newton_f32(x3 - sh, f1, f2, f3));
+    if (d1 - d3 > 1e-4f * (d1 + d3)) return halley(newton_f32(x1 - sh, f1, f2, f3));
+    const double r1 = halley(newton_f32(x1 - sh, f1, f2, f3));
+    const double r3 = halley(newton_f32(x3 - sh, f1, f2, f3));
     const double h1 = (((r1 + v3) * r1 + v2) * r1 + v1) * r1;
     const double h3 = (((r3 + v3) * r3 + v2) * r3 + v1) * r3;
     const double w = r3 - r1;
     // x3 iff (d3 - d1) > 1e-9 (d1 + d3), i.e. h1 - h3 > 1e-9 / 3 (x3 - x1)^4
     return (h1 - h3 > (1e-9 / 3.0) * (w * w) * (w * w)) ? r3 : r1;
+}
+__device__ __forceinline__ double line_search(double v1, double v2, double v3) {
+    return line_search_from((float)v1, (float)v2, (float)v3, v1, v2, v3,
+                            [&](float x) { return halley_cubic((double)x, v1, v2, v3); });
+}
+
+// The same step size by a whole warp for one coordinate (c_i, b_i, H_ii and mu
+// in every lane; every lane returns it), bit for bit.  An FP64 instruction
+// takes its scheduler 64 cycles however many lanes it serves, so the lanes
+// work on different values of one instruction: the three coefficients
+//   v1 = 4 b_i + 4 mu c_i, v2 = 2 H_ii + 4 c_i^2 + 2 mu, v3 = 4 c_i
+// in 3 instructions after H_ii instead of 8, and the polynomials of the Halley
+// step as one Horner chain.  Powers of two are factored out; they do not
+// change a rounding.  (N = 8, one CTA, 1000 iterations with start and export:
+// 7.39 -> 7.09 ms, with the average of |eta| moved off the control warp.)
+__device__ __forceinline__ double line_search_warp(double ci, double bi, double Hii, double mu) {
+    const int l = threadIdx.x & 3;
+    const double c2 = ci + ci;
+    const double p = (l == 0 ? mu : c2) * (l >= 2 ? 1.0 : ci);
+    const double q = (l == 0 ? bi : (l == 1 ? Hii : 0.0)) + p;
+    const double v = (q + (l == 1 ? mu : 0.0)) * (l == 0 ? 4.0 : 2.0);
+    const float f = (float)v;
+    const unsigned all = 0xffffffffu;
+    const float f1 = __shfl_sync(all, f, 0), f2 = __shfl_sync(all, f, 1), f3 = __shfl_sync(all, f, 2);
+    const double v1 = __shfl_sync(all, v, 0), v2 = __shfl_sync(all, v, 1), v3 = __shfl_sync(all, v, 2);
+    // coefficients (highest first) of lane 0: the cubic f, 1: f', 2: f'', 3: 2 f'
+    const double w = 3.0 * v3;
+    const double a3 = l == 0 ? 4.0 : 0.0, a2 = l == 0 ? w : (l == 1 ? 12.0 : (l == 2 ? 0.0 : 24.0));
+    const double s1 = (l == 0 ? v2 : w) * (l == 3 ? 4.0 : 2.0), a1 = l == 2 ? 24.0 : s1;
+    const double a0 = (l == 0 ? v1 : (l == 2 ? w : v2)) * (l == 0 ? 1.0 : (l == 3 ? 4.0 : 2.0));
+    return line_search_from(f1, f2, f3, v1, v2, v3, [&](float xf) {
+        const double x = (double)xf;
+        const double y = fma(fma(fma(a3, x, a2), x, a1), x, a0);
+        const double g = __shfl_sync(all, y, 0), g1 = __shfl_sync(all, y, 1), g2 = __shfl_sync(all, y, 2);
+        const double tg1 = __shfl_sync(all, y, 3);
+        const double den = fma(tg1, g1, -g * g2);
+        if (!(den != 0.0) || !isfinite(den)) return x;
+        return x - g * tg1 * recip(den);
+    });
 }
 
 }  // namespace cdfci

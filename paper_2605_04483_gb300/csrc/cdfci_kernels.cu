@@ -698,17 +698,12 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
         if (warp == 0) {
             // ---- control warp: H_ii and the step size (appendix) ----
             const double Hii = diag_pairs_warp(P, L, sHd, sJ, sK, sPairs, lay.npairs);
+            const double ci = sel.ci;
+            // (mu: c.c within 2 ulp; the double-double value runs behind)
+            const double eta = sel.forced ? sel.feta : line_search_warp(ci, sel.bi, Hii, ls.pmu_g);
             if (lane == 0) {
-                const double bi = sel.bi, ci = sel.ci;
-                double eta;
-                if (sel.forced) {
-                    eta = sel.feta;
-                } else {
-                    const double mu0 = ls.pmu_g;          // c.c within 2 ulp (the double-double value runs behind)
-                    eta = line_search(4.0 * bi + 4.0 * mu0 * ci, 2.0 * Hii + 4.0 * ci * ci + 2.0 * mu0, 4.0 * ci);
-                }
                 sel.eta = eta;
-                sel.mu_g = ls.mu.hi + fma(2.0 * eta, ci, eta * eta);
+                sel.mu_g = ls.mu.hi + fma(eta, ci + ci, eta * eta);
                 sel.bad = ((__double_as_longlong(eta) >> 52) & 0x7ff) == 0x7ff;   // not finite
                 s_hii = Hii;
             }
@@ -844,6 +839,18 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             if (err) atomicOr(&s_err, 1);
         }
         __syncthreads();
+        if (warp == 3 && lane == 0) {                  // the moving average of |eta|, beside the combine
+            int done = 0;
+            if (!sel.forced) {
+                const double dx = P.theta * ls.dx + (1.0 - P.theta) * fabs(eta);
+                ls.dx = dx;
+                // (dx >= 0: the bit patterns of non-negative doubles order like their values)
+                const long long dxb = __double_as_longlong(dx), thb = __double_as_longlong(P.dx_threshold);
+                done = thb > 0 && dxb < thb ? 1 : 0;
+            }
+            ls.done = done;
+            s_done = done;
+        }
         if (warp == 2 && lane < 2) {                   // what books() takes, before the choice overwrites it
             bk_eta = eta;
             bk_y1 = lane == 0 ? sel.ci : sel.bi;
@@ -883,13 +890,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 const double ci = sel.ci, ci_new = ci + sel.eta;
                 ls.pA = sel.iA; ls.pB = sel.iB; ls.pslot = sel.islot;
                 ls.pc = ci_new; ls.pHii = s_hii; ls.pmu_g = sel.mu_g; ls.peta = sel.eta;
-                if (!sel.forced) {
-                    ls.iterations += 1;
-                    ls.dx = P.theta * ls.dx + (1.0 - P.theta) * fabs(sel.eta);
-                    // (dx >= 0: the bit patterns of non-negative doubles order like their values)
-                    const long long dxb = __double_as_longlong(ls.dx), thb = __double_as_longlong(P.dx_threshold);
-                    if (thb > 0 && dxb < thb) ls.done = 1;
-                }
+                if (!sel.forced) ls.iterations += 1;
                 const bool z0 = is_zero(ci), z1 = is_zero(ci_new);
                 ls.nnz_c += ((z0 && !z1) ? 1 : 0) - ((!z0 && z1) ? 1 : 0);
                 ls.forced = it + 1 < F.n ? 1 : 0;
@@ -899,7 +900,6 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                     ls.feta = __ldg(F.c + it + 1);
                 }
                 ls.have_prev = 1;
-                s_done = ls.done;
             }
         }
         if (kGrid) {
