@@ -633,6 +633,18 @@ __device__ __forceinline__ float cbrt_seed(float x) {
 // whose quartic is symmetric about -c_i): decided in single precision when
 // the distances differ by more than 1e-4 of their sum, else on the FP64
 // roots through the quartic's values and that identity.
+// (the distances differ by 1e-4 of their sum or less; out of line, so that the loops that call this hold one
+// copy of the polishing)
+static __device__ __noinline__ double line_search_tie(float x1, float x3, float f1, float f2, float f3, double v1, double v2,
+                                               double v3) {
+    const double r1 = halley_cubic((double)newton_f32(x1, f1, f2, f3), v1, v2, v3);
+    const double r3 = halley_cubic((double)newton_f32(x3, f1, f2, f3), v1, v2, v3);
+    const double h1 = (((r1 + v3) * r1 + v2) * r1 + v1) * r1;
+    const double h3 = (((r3 + v3) * r3 + v2) * r3 + v1) * r3;
+    const double w = r3 - r1;
+    // x3 iff (d3 - d1) > 1e-9 (d1 + d3), i.e. h1 - h3 > 1e-9 / 3 (x3 - x1)^4
+    return (h1 - h3 > (1e-9 / 3.0) * (w * w) * (w * w)) ? r3 : r1;
+}
 // f1 .. f3 are v1 .. v3 rounded to single precision; halley(x) = halley_cubic((double)x, v1, v2, v3).
 template <class Halley>
 __device__ __forceinline__ double line_search_from(float f1, float f2, float f3, double v1, double v2, double v3,
@@ -643,28 +655,23 @@ __device__ __forceinline__ double line_search_from(float f1, float f2, float f3,
     const float q = (2.0f * b * b * b - 36.0f * b * c + 432.0f * d) * (1.0f / 1728.0f);
     const float hq = 0.5f * q, tp = p * (1.0f / 3.0f);
     const float del = hq * hq + tp * tp * tp;
+    float x;                                                  // the seed of the root taken
     if (!(del < 0.0f) || !(p < 0.0f)) {
         const float sd = sqrtf(fmaxf(del, 0.0f));
-        const float x = cbrt_seed(-hq + sd) + cbrt_seed(-hq - sd) - sh;
-        return halley(newton_f32(x, f1, f2, f3));
+        x = cbrt_seed(-hq + sd) + cbrt_seed(-hq - sd) - sh;
+    } else {
+        const float m = 2.0f * sqrtf(-tp);
+        float arg = (3.0f * q / (2.0f * p)) * sqrtf(-3.0f / p);
+        arg = fminf(1.0f, fmaxf(-1.0f, arg));
+        const float th = acosf(arg) * (1.0f / 3.0f);
+        const float x3 = m * cosf(th);                        // depressed roots x1 <= x2 <= x3
+        const float x2 = m * cosf(th - 2.09439510239319549f);
+        const float x1 = m * cosf(th - 4.18879020478639098f);
+        const float d1 = x2 - x1, d3 = x3 - x2;
+        if (!(fabsf(d3 - d1) > 1e-4f * (d1 + d3))) return line_search_tie(x1 - sh, x3 - sh, f1, f2, f3, v1, v2, v3);
+        x = (d3 > d1 ? x3 : x1) - sh;
     }
-    const float m = 2.0f * sqrtf(-tp);
-    float arg = (3.0f * q / (2.0f * p)) * sqrtf(-3.0f / p);
-    arg = fminf(1.0f, fmaxf(-1.0f, arg));
-    const float th = acosf(arg) * (1.0f / 3.0f);
-    const float x3 = m * cosf(th);                            // depressed roots x1 <= x2 <= x3
-    const float x2 = m * cosf(th - 2.09439510239319549f);
-    const float x1 = m * cosf(th - 4.18879020478639098f);
-    const float d1 = x2 - x1, d3 = x3 - x2;
-    if (d3 - d1 > 1e-4f * (d1 + d3)) return halley(newton_f32(x3 - sh, f1, f2, f3));
-    if (d1 - d3 > 1e-4f * (d1 + d3)) return halley(newton_f32(x1 - sh, f1, f2, f3));
-    const double r1 = halley(newton_f32(x1 - sh, f1, f2, f3));
-    const double r3 = halley(newton_f32(x3 - sh, f1, f2, f3));
-    const double h1 = (((r1 + v3) * r1 + v2) * r1 + v1) * r1;
-    const double h3 = (((r3 + v3) * r3 + v2) * r3 + v1) * r3;
-    const double w = r3 - r1;
-    // x3 iff (d3 - d1) > 1e-9 (d1 + d3), i.e. h1 - h3 > 1e-9 / 3 (x3 - x1)^4
-    return (h1 - h3 > (1e-9 / 3.0) * (w * w) * (w * w)) ? r3 : r1;
+    return halley(newton_f32(x, f1, f2, f3));
 }
 __device__ __forceinline__ double line_search(double v1, double v2, double v3) {
     return line_search_from((float)v1, (float)v2, (float)v3, v1, v2, v3,

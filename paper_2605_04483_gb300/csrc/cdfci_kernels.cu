@@ -51,8 +51,8 @@ __device__ __forceinline__ double warp_sum(double x) {
     return x;
 }
 
-constexpr int kCdThreads = 384;                 // threads per CTA of the cluster
-constexpr int kCdWarps = kCdThreads / 32;
+constexpr int kCdThreads = 384;                 // threads per CTA of the cluster: the control warp and 11 with elements
+constexpr int kCdWarps = kCdThreads / 32, kCdElemThreads = kCdThreads - 32;
 constexpr int kCdMaxE = 3;                      // elements whose slot loads a thread keeps in flight
 constexpr int kCdMaxCluster = 16;
 
@@ -231,21 +231,27 @@ __device__ __forceinline__ void issue_elem(const Problem &P, const ColLists &L, 
     }
     if (have_prev && x.ka == pA && x.kb == pB) { x.state = 3; return; }
     x.pos = (long long)(h & P.mask);
-    const Slot *s = P.table + x.pos;
-    ld_slot32(s, x.k0, x.cb0);
+    ld_slot32(P.table + x.pos, x.k0, x.cb0);
     x.state = 4;
 }
 
-// Finish the lookup of an issued element: compare the first slot, probe on if
-// needed.  Sets state 1 (found: c, bv), 2 (absent at pos) or 0 (value zero or
-// error, *err set).
+// Finish the lookup of an issued element: compare the loaded slot, then probe
+// on, kProbeAhead slots a load: the warp waits for its slowest lane, and a
+// dependent probe is an L2 round trip (700 cycles and more), of which every
+// warp paid for two or three even in a nearly empty table.  (One copy of the
+// comparison: the loop's code is as long as the instruction cache.)
+// Sets state 1 (found: c, b), 2 (absent at pos) or 0 (value zero or error,
+// *err set).
+constexpr int kProbeAhead = 2;
 __device__ __forceinline__ void resolve_elem(const Problem &P, IterState *st, Elem &x, int *err) {
     if (x.state != 4) return;
     if (is_zero(x.H)) { x.state = 0; return; }
     const bool both_nonzero = (P.na > 0) && (P.nb > 0);
     unsigned long long p = (unsigned long long)x.pos;
-    ulonglong2 k = x.k0;
-    double2 cb = x.cb0;
+    ulonglong2 k = x.k0, kn[kProbeAhead];
+    double2 cb = x.cb0, cn[kProbeAhead];
+    int left = 0;
+#pragma unroll 1
     for (int probe = 0; probe < P.max_probe; ++probe) {
         int spins = 0;
         while (both_nonzero && ((k.x == 0ull) != (k.y == 0ull))) {
@@ -255,7 +261,16 @@ __device__ __forceinline__ void resolve_elem(const Problem &P, IterState *st, El
         if (k.x == x.ka && (k.y & kKeyMaskB) == x.kb) { x.pos = (long long)p; x.cb0 = cb; x.state = 1; return; }
         if (k.x == 0ull && k.y == 0ull) { x.pos = (long long)p; x.state = 2; return; }
         p = (p + 1) & P.mask;
-        ld_slot32(P.table + p, k, cb);
+        if (left == 0) {
+#pragma unroll
+            for (int j = 0; j < kProbeAhead; ++j) ld_slot32(P.table + ((p + j) & P.mask), kn[j], cn[j]);
+            left = kProbeAhead;
+        }
+        --left;
+        k = kn[0];
+        cb = cn[0];
+#pragma unroll
+        for (int j = 0; j + 1 < kProbeAhead; ++j) { kn[j] = kn[j + 1]; cn[j] = cn[j + 1]; }
     }
     set_status(st, kErrTableFull);
     *err = 1;
@@ -302,6 +317,7 @@ struct LoopState {
     unsigned long long fa, fb;         // forced next coordinate and its step
     double feta;
     int forced, have_prev, done;
+    double qc, qb;                     // previous coordinate: c and b as its step used them
 };
 
 // Warp-level combine: argmax of (gbits desc, key asc) with payload (slot, b, c),
@@ -367,6 +383,11 @@ __device__ __forceinline__ void warp_combine(Best &best, double &bb, double &cb,
 // suffice.  The waits are bounded: on expiry the status becomes
 // CDFCI_ERR_TIMEOUT and the loop ends.
 constexpr int kXchgSpins = 1 << 21;
+// the barrier of the whole CTA, reached by the control warp and the element warps in different places
+__device__ __forceinline__ void cta_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 0;" ::: "memory");
+}
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
@@ -500,7 +521,6 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
     __shared__ Sel sel;
     __shared__ int s_done;
     __shared__ LoopState ls;                     // written by lane 0 of the control warp (warp 0) only
-    __shared__ double s_hii;
     __shared__ int s_err;
     __shared__ int s_fins;                       // 1: this CTA inserted the forced coordinate of this step
     __shared__ int s_tmo;                        // grid mode: a wait for the partials expired
@@ -532,6 +552,9 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
         ls.fa = R.fa; ls.fb = R.fb; ls.feta = R.feta;
         ls.forced = R.forced; ls.have_prev = R.have_prev; ls.done = 0;
         if (!kGrid) spart[1] = gpart[rank];
+        r_best[0] = Best{0ull, ~0ull, ~0ull, -1};    // the control warp holds no elements
+        r_bc[0][0] = r_bc[0][1] = r_bc[0][2] = 0.0;
+        for (int k = 0; k < 4; ++k) r_cnt[k][0] = 0;
         s_err = 0;
         s_done = 0;
         s_fins = 0;
@@ -557,25 +580,27 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
     const int n_own = rank < nqs ? (nqs - 1 - rank) / G + 1 : 0;
     const int tb = min(min(n_own, lay.tb_max), Wp * kE);
     const int nterms = tb * 32 * (nocc + 1);
-    // The double-double books of an iteration, by two lanes of warp 2 beside the control warp's next
-    // choice (mu is read after the line search, behind the barrier that follows the choice), not in
-    // front of the iteration's last barrier: the chain of about 35 dependent FP64 operations takes
-    // some 2400 cycles (with that and the shorter combines, a N = 8 run of one CTA went from 7.79 to
-    // 7.39 us an iteration, of 57 CTAs from 13.1 to 12.6).  Lane 0: mu += 2 eta c_i + eta^2; lane 1: alpha += 2 eta b_i + eta^2 H_ii.
-    double bk_eta = 0.0, bk_y1 = 0.0, bk_y2 = 0.0;
+    // The double-double books of an iteration, about 35 dependent FP64 operations (2400 cycles alone,
+    // more beside the element warps' own), must not sit in front of the iteration's last barrier.
+    // Several CTAs: by two lanes of warp 2 beside the fold and the control warp's next choice, which
+    // take as long (mu is read after the line search, behind the barrier that follows the choice).
+    // One CTA has no fold, and the choice alone is shorter: there the control warp does them while the
+    // others apply the column (N = 8: 6.90 ms a run with the first, 6.31 with this).  Lane 0:
+    // mu += 2 eta c_i + eta^2; lane 1: alpha += 2 eta b_i + eta^2 H_ii.
+    constexpr int kBooks = 2;
     bool bk_due = false;                               // uniform
     auto books = [&]() {
-        if (warp == 2 && lane < 2) {
-            const dd x0 = lane == 0 ? ls.mu : ls.alpha;
-            const dd t = dd_add_fast(dd_two_prod(2.0 * bk_eta, bk_y1), dd_mul_d(dd_two_prod(bk_eta, bk_eta), bk_y2));
-            const dd r = dd_add_fast(x0, t);
+        if (lane < 2) {
+            const double e = ls.peta, y1 = lane == 0 ? ls.qc : ls.qb, y2 = lane == 0 ? 1.0 : ls.pHii;
+            const dd t = dd_add_fast(dd_two_prod(2.0 * e, y1), dd_mul_d(dd_two_prod(e, e), y2));
+            const dd r = dd_add_fast(lane == 0 ? ls.mu : ls.alpha, t);
             if (lane == 0) ls.mu = r; else ls.alpha = r;
         }
     };
     int lastp = 1;
     for (long long it = 0; it < n_iter; ++it) {
         const int pin = lastp, pout = lastp ^ 1;
-        if (bk_due) books();
+        if (bk_due && warp == kBooks) books();
         bk_due = false;
         // ---- choice of i (Eq. choose-i), by the control warp ----
         // every CTA's partial of the last column: lane l of the control warp folds CTAs l, l + 32, ...
@@ -609,6 +634,8 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             if (ls.have_prev) {
                 if (kGrid && it > 0) {
                     // folded above
+                } else if (!kGrid && G == 1) {             // one CTA: its own partial is all
+                    fold_partial(spart[pin], true, bb, bj, cj, gsum, cnt, err);
                 } else {
                     for (int r = lane; r < G; r += 64) {       // two loads in flight per lane
                         const bool two = r + 32 < G;
@@ -621,7 +648,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                         if (two) fold_partial(x1, false, bb, bj, cj, gsum, cnt, err);
                     }
                 }
-                if (G > 1) warp_combine(bb, bj, cj, gsum, cnt, err, G < 32 ? G : 32);   // one CTA: lane 0 has it all
+                if (G > 1) warp_combine(bb, bj, cj, gsum, cnt, err, G < 32 ? G : 32);
             }
             if (tmo) {
                 if (lane == 0) {
@@ -693,8 +720,6 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             if ((iB >> t) & 1ull) L.occB[rb] = (unsigned char)t; else L.virB[t - rb] = (unsigned char)t;
         }
         __syncwarp();
-        Elem el[kE];
-        unsigned long long hAc = 0ull, hBc = 0ull;
         if (warp == 0) {
             // ---- control warp: H_ii and the step size (appendix) ----
             const double Hii = diag_pairs_warp(P, L, sHd, sJ, sK, sPairs, lay.npairs);
@@ -705,15 +730,39 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 sel.eta = eta;
                 sel.mu_g = ls.mu.hi + fma(eta, ci + ci, eta * eta);
                 sel.bad = ((__double_as_longlong(eta) >> 52) & 0x7ff) == 0x7ff;   // not finite
-                s_hii = Hii;
             }
-#pragma unroll
-            for (int k = 0; k < kE; ++k) el[k].state = 0;
+            // ---- the state after this iteration, while the others apply ----
+            cta_sync();
+            if (lane == 0) {
+                const double ci_new = ci + eta;
+                ls.pA = iA; ls.pB = iB; ls.pslot = sel.islot;
+                ls.pc = ci_new; ls.pHii = Hii; ls.pmu_g = sel.mu_g; ls.peta = eta;
+                ls.qc = ci; ls.qb = sel.bi;
+                if (!sel.forced) {
+                    ls.iterations += 1;
+                    ls.dx = P.theta * ls.dx + (1.0 - P.theta) * fabs(eta);
+                    // (dx >= 0: the bit patterns of non-negative doubles order like their values)
+                    const long long dxb = __double_as_longlong(ls.dx), thb = __double_as_longlong(P.dx_threshold);
+                    if (thb > 0 && dxb < thb) ls.done = 1;
+                }
+                const bool z0 = is_zero(ci), z1 = is_zero(ci_new);
+                ls.nnz_c += ((z0 && !z1) ? 1 : 0) - ((!z0 && z1) ? 1 : 0);
+                ls.forced = it + 1 < F.n ? 1 : 0;
+                if (it + 1 < F.n) {                    // a start vector's next entry
+                    ls.fa = __ldg(F.keys + 2 * (it + 1));
+                    ls.fb = __ldg(F.keys + 2 * (it + 1) + 1);
+                    ls.feta = __ldg(F.c + it + 1);
+                }
+                ls.have_prev = 1;
+                s_done = ls.done;
+            }
+            __syncwarp();
+            if (!kGrid && G == 1) books();
         } else {
             // ---- element warps: term loads of this CTA's singles (from the lists alone), the
             // column's single-excitation tables, decode, first probes, values ----
             const int u = tid - 32;
-            constexpr int kU = kCdThreads - 32;
+            constexpr int kU = kCdElemThreads;
             constexpr int kR = 2;
             double tv[kR] = {0.0, 0.0};
             if (tb > 0) {                              // uniform in the CTA; nterms >= 1 then
@@ -721,141 +770,128 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 for (int r = 0; r < kR; ++r)
                     tv[r] = __ldg(single_term_ptr(P, L, rank, G, nocc, nsing, min(u + r * kU, nterms - 1)));
             }
-            build_singles(P, L, iA, iB, tabA, tabB, tid - 32, kCdThreads - 32);
-            asm volatile("bar.sync 1, %0;" ::"r"(kCdThreads - 32) : "memory");
-            hAc = hash_alpha(iA);
-            hBc = hash_beta(iB);
-#pragma unroll
-            for (int k = 0; k < kE; ++k)
-                issue_elem(P, L, tabA, tabB, iA, iB, hAc, hBc, e0 + k * stride, nh, have_prev, pA, pB, el[k]);
-            // this thread's singles that the term table covers (first round: block (warp - 1) + W' k)
-            bool ts[kE];
-#pragma unroll
-            for (int k = 0; k < kE; ++k) ts[k] = el[k].state != 0 && el[k].ix.kind <= 1 && (warp - 1) + Wp * k < tb;
-#pragma unroll
-            for (int k = 0; k < kE; ++k)
-                if (el[k].state != 0 && !ts[k]) el[k].H = element_value(P, L, el[k].ix);
-            if (tb > 0) {                              // uniform in the CTA
-#pragma unroll
-                for (int r = 0; r < kR; ++r)
-                    if (u + r * kU < nterms) sTerm[u + r * kU] = tv[r];
-                for (int base = u + kR * kU; base < nterms; base += kR * kU) {
-#pragma unroll
-                    for (int r = 0; r < kR; ++r)
-                        tv[r] = __ldg(single_term_ptr(P, L, rank, G, nocc, nsing, min(base + r * kU, nterms - 1)));
-#pragma unroll
-                    for (int r = 0; r < kR; ++r)
-                        if (base + r * kU < nterms) sTerm[base + r * kU] = tv[r];
-                }
-                asm volatile("bar.sync 1, %0;" ::"r"(kCdThreads - 32) : "memory");
+            build_singles(P, L, iA, iB, tabA, tabB, tid - 32, kCdElemThreads);
+            named_bar_sync(1, kCdElemThreads);
+            const unsigned long long hAc = hash_alpha(iA), hBc = hash_beta(iB);
+            Best best{0ull, ~0ull, ~0ull, -1};
+            double bbest = 0.0, cbest = 0.0, gather = 0.0;
+            int cnt[4] = {0, 0, 0, 0};                 // elements, applied, dropped, inserted
+            int err = 0;
+            const unsigned long long tau_bits = abs_bits(P.tau);
+            double eta = 0.0, mu = 0.0, pb = 0.0, pc = 0.0;
+            long long pslot = -1;
+            // rounds of kE elements a thread (kE = 1: one round covers the column).  One copy of the code for
+            // every round, the step size awaited in the first: the loop's code does not fit the
+            // instruction cache.
+            bool first = true;
+            for (long long eb = e0;;) {
+                Elem el[kE];
 #pragma unroll
                 for (int k = 0; k < kE; ++k)
-                    if (ts[k]) {
-                        const int ls = ((warp - 1) + Wp * k) * 32 + lane;
-                        el[k].H = single_sum(sTerm + ls * (nocc + 1), nocc, el[k].ix.sgn);
+                    issue_elem(P, L, tabA, tabB, iA, iB, hAc, hBc, eb + k * stride, nh, have_prev, pA, pB, el[k]);
+                // this thread's singles that the term table covers (the first round: block (warp - 1) + W' k)
+                bool ts[kE];
+#pragma unroll
+                for (int k = 0; k < kE; ++k) ts[k] = first && el[k].state != 0 && el[k].ix.kind <= 1 && (warp - 1) + Wp * k < tb;
+#pragma unroll
+                for (int k = 0; k < kE; ++k)
+                    if (el[k].state != 0 && !ts[k]) el[k].H = element_value(P, L, el[k].ix);
+                if (first && tb > 0) {                     // uniform in the CTA
+#pragma unroll
+                    for (int r = 0; r < kR; ++r)
+                        if (u + r * kU < nterms) sTerm[u + r * kU] = tv[r];
+                    for (int base = u + kR * kU; base < nterms; base += kR * kU) {
+#pragma unroll
+                        for (int r = 0; r < kR; ++r)
+                            tv[r] = __ldg(single_term_ptr(P, L, rank, G, nocc, nsing, min(base + r * kU, nterms - 1)));
+#pragma unroll
+                        for (int r = 0; r < kR; ++r)
+                            if (base + r * kU < nterms) sTerm[base + r * kU] = tv[r];
                     }
+                    named_bar_sync(1, kCdElemThreads);
+#pragma unroll
+                    for (int k = 0; k < kE; ++k)
+                        if (ts[k]) {
+                            const int ls = ((warp - 1) + Wp * k) * 32 + lane;
+                            el[k].H = single_sum(sTerm + ls * (nocc + 1), nocc, el[k].ix.sgn);
+                        }
+                }
+                if (first) {
+                    cta_sync();
+                    eta = sel.eta;
+                    mu = sel.mu_g;
+                    pslot = sel.pslot;
+                    pb = sel.pb;
+                    pc = sel.pc;
+                    first = false;
+                    if (sel.bad) break;
+                }
+                // ---- apply: b_j += eta H_ji with compression, gather, candidates ----
+#pragma unroll
+                for (int k = 0; k < kE; ++k) resolve_elem(P, st, el[k], &err);
+#pragma unroll
+                for (int k = 0; k < kE; ++k) {
+                    Elem &x = el[k];
+                    if (x.state == 0) continue;
+                    const double H = x.H;
+                    const double v = eta * H;
+                    const bool big = abs_bits(v) >= tau_bits;
+                    double cj, bn;
+                    long long sj;
+                    if (x.state == 3) {                       // the previous coordinate: c and b known
+                        cj = pc;
+                        sj = pslot;
+                        if (is_zero(H)) { P.table[sj].bv = pb; continue; }
+                        ++cnt[0];
+                        if (!(!is_zero(cj) || big)) { P.table[sj].bv = pb; ++cnt[2]; continue; }
+                        bn = pb + v;
+                    } else if (x.state == 1) {
+                        cj = x.cb0.x;
+                        sj = x.pos;
+                        ++cnt[0];
+                        if (!(!is_zero(cj) || big)) { ++cnt[2]; continue; }
+                        bn = x.cb0.y + v;
+                    } else {                                  // absent
+                        ++cnt[0];
+                        if (!big) { ++cnt[2]; continue; }
+                        sj = claim_slot(P, st, x.ka, x.kb, x.pos, &err);
+                        if (sj < 0) continue;
+                        cj = 0.0;
+                        bn = v;
+                        ++cnt[3];
+                    }
+                    ++cnt[1];
+                    P.table[sj].bv = bn;
+                    unsigned long long gb;
+                    if (!is_zero(cj)) {
+                        gather = fma(H, cj, gather);
+                        gb = abs_bits(fma(mu, cj, bn));
+                    } else {
+                        gb = abs_bits(bn);
+                    }
+                    if (better(gb, x.ka, x.kb, best.g, best.a, best.b)) {
+                        best = Best{gb, x.ka, x.kb, sj};
+                        bbest = bn;
+                        cbest = cj;
+                    }
+                }
+                eb += kE * stride;
+                if (kE == 1 || eb >= nh) break;
+            }
+            // ---- the warp's partial ----
+            warp_combine(best, bbest, cbest, gather, cnt, err);
+            if (lane == 0) {
+                r_best[warp] = best;
+                r_bc[warp][0] = bbest;
+                r_bc[warp][1] = cbest;
+                r_bc[warp][2] = gather;
+                for (int k = 0; k < 4; ++k) r_cnt[k][warp] = cnt[k];
+                if (err) atomicOr(&s_err, 1);
             }
         }
-        __syncthreads();
-        const double eta = sel.eta;
-        const double mu = sel.mu_g;
-        const unsigned long long tau_bits = abs_bits(P.tau);
-        const long long pslot = sel.pslot;
-        const double pb = sel.pb, pc = sel.pc;
-        const bool bad = sel.bad != 0;
-
-        // ---- apply: b_j += eta H_ji with compression, gather, candidates ----
-        Best best{0ull, ~0ull, ~0ull, -1};
-        double bbest = 0.0, cbest = 0.0, gather = 0.0;
-        int cnt[4] = {0, 0, 0, 0};                     // elements, applied, dropped, inserted
-        int err = 0;
-        for (long long eb = e0; !bad && eb < nh;) {
-#pragma unroll
-            for (int k = 0; k < kE; ++k) resolve_elem(P, st, el[k], &err);
-#pragma unroll
-            for (int k = 0; k < kE; ++k) {
-                Elem &x = el[k];
-                if (x.state == 0) continue;
-                const double H = x.H;
-                const double v = eta * H;
-                const bool big = abs_bits(v) >= tau_bits;
-                double cj, bn;
-                long long sj;
-                if (x.state == 3) {                       // the previous coordinate: c and b known
-                    cj = pc;
-                    sj = pslot;
-                    if (is_zero(H)) { P.table[sj].bv = pb; continue; }
-                    ++cnt[0];
-                    if (!(!is_zero(cj) || big)) { P.table[sj].bv = pb; ++cnt[2]; continue; }
-                    bn = pb + v;
-                } else if (x.state == 1) {
-                    cj = x.cb0.x;
-                    sj = x.pos;
-                    ++cnt[0];
-                    if (!(!is_zero(cj) || big)) { ++cnt[2]; continue; }
-                    bn = x.cb0.y + v;
-                } else {                                  // absent
-                    ++cnt[0];
-                    if (!big) { ++cnt[2]; continue; }
-                    sj = claim_slot(P, st, x.ka, x.kb, x.pos, &err);
-                    if (sj < 0) continue;
-                    cj = 0.0;
-                    bn = v;
-                    ++cnt[3];
-                }
-                ++cnt[1];
-                P.table[sj].bv = bn;
-                unsigned long long gb;
-                if (!is_zero(cj)) {
-                    gather = fma(H, cj, gather);
-                    gb = abs_bits(fma(mu, cj, bn));
-                } else {
-                    gb = abs_bits(bn);
-                }
-                if (better(gb, x.ka, x.kb, best.g, best.a, best.b)) {
-                    best = Best{gb, x.ka, x.kb, sj};
-                    bbest = bn;
-                    cbest = cj;
-                }
-            }
-            eb += kE * stride;
-            if (eb >= nh) break;
-#pragma unroll
-            for (int k = 0; k < kE; ++k)
-                issue_elem(P, L, tabA, tabB, iA, iB, hAc, hBc, eb + k * stride, nh, have_prev, pA, pB, el[k]);
-#pragma unroll
-            for (int k = 0; k < kE; ++k)
-                if (el[k].state != 0) el[k].H = element_value(P, L, el[k].ix);
-        }
-
         // ---- CTA partial into this CTA's shared memory ----
-        if (warp != 0) warp_combine(best, bbest, cbest, gather, cnt, err);   // warp 0 holds no elements
-        if (lane == 0) {
-            r_best[warp] = best;
-            r_bc[warp][0] = bbest;
-            r_bc[warp][1] = cbest;
-            r_bc[warp][2] = gather;
-            for (int k = 0; k < 4; ++k) r_cnt[k][warp] = cnt[k];
-            if (err) atomicOr(&s_err, 1);
-        }
         __syncthreads();
-        if (warp == 3 && lane == 0) {                  // the moving average of |eta|, beside the combine
-            int done = 0;
-            if (!sel.forced) {
-                const double dx = P.theta * ls.dx + (1.0 - P.theta) * fabs(eta);
-                ls.dx = dx;
-                // (dx >= 0: the bit patterns of non-negative doubles order like their values)
-                const long long dxb = __double_as_longlong(dx), thb = __double_as_longlong(P.dx_threshold);
-                done = thb > 0 && dxb < thb ? 1 : 0;
-            }
-            ls.done = done;
-            s_done = done;
-        }
-        if (warp == 2 && lane < 2) {                   // what books() takes, before the choice overwrites it
-            bk_eta = eta;
-            bk_y1 = lane == 0 ? sel.ci : sel.bi;
-            bk_y2 = lane == 0 ? 1.0 : s_hii;
-        }
+        const bool bad = sel.bad != 0;
         if (warp == 0) {
             const bool have = lane < kCdWarps;
             Best b = have ? r_best[lane] : Best{0ull, ~0ull, ~0ull, -1};
@@ -874,9 +910,8 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 pp.err = s_err | (bad ? 1 : 0);
                 if (kGrid) spart[0] = pp; else spart[pout] = pp;
                 // the coordinate's own slot: c_i += eta, b_i as used (rank 0 writes)
-                const double ci = sel.ci, ci_new = ci + sel.eta;
                 if (rank == 0 && !bad) {
-                    P.table[sel.islot].c = ci_new;
+                    P.table[sel.islot].c = ls.pc;
                     P.table[sel.islot].bv = sel.bi;
                 }
                 if (bad && rank == 0) set_status(st, kErrNonfinite);
@@ -885,21 +920,6 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 __syncwarp();
                 const unsigned int q = q0 + (unsigned int)it + 1u;
                 xchg_publish(xchg + ((size_t)(q & 1u) * G + rank) * kXchgWords, spart[0], q, lane);
-            }
-            if (lane == 0) {
-                const double ci = sel.ci, ci_new = ci + sel.eta;
-                ls.pA = sel.iA; ls.pB = sel.iB; ls.pslot = sel.islot;
-                ls.pc = ci_new; ls.pHii = s_hii; ls.pmu_g = sel.mu_g; ls.peta = sel.eta;
-                if (!sel.forced) ls.iterations += 1;
-                const bool z0 = is_zero(ci), z1 = is_zero(ci_new);
-                ls.nnz_c += ((z0 && !z1) ? 1 : 0) - ((!z0 && z1) ? 1 : 0);
-                ls.forced = it + 1 < F.n ? 1 : 0;
-                if (it + 1 < F.n) {                    // a start vector's next entry
-                    ls.fa = __ldg(F.keys + 2 * (it + 1));
-                    ls.fb = __ldg(F.keys + 2 * (it + 1) + 1);
-                    ls.feta = __ldg(F.c + it + 1);
-                }
-                ls.have_prev = 1;
             }
         }
         if (kGrid) {
@@ -911,10 +931,10 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             cluster.sync();                           // partials and table writes visible cluster-wide
         }
         lastp = pout;
-        bk_due = true;
+        bk_due = kGrid || G > 1;
         if (s_done || bad) break;                     // identical in every CTA
     }
-    if (bk_due) books();
+    if (bk_due && warp == kBooks) books();
     __syncthreads();                                  // the books before the record
 
     // ---- state for the next launch / the finalisation ----
