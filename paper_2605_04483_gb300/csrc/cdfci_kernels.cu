@@ -1147,9 +1147,23 @@ __global__ void __launch_bounds__(256) k_export(Problem P, const IterState *st, 
                                                 double *b, long long cap, unsigned long long *counter) {
     const double s = st->scale.hi + st->scale.lo;
     export_rows(P, cap, counter, [&](long long, const Slot &sl, long long pos) {
-        reinterpret_cast<ulonglong2 *>(keys)[pos] = make_ulonglong2(sl.a, sl.b & kKeyMaskB);
+        if (keys) reinterpret_cast<ulonglong2 *>(keys)[pos] = make_ulonglong2(sl.a, sl.b & kKeyMaskB);
         if (c) c[pos] = sl.c * s;
         if (b) b[pos] = sl.bv * s;
+    });
+}
+
+// xCDFCI: every stored determinant with its rows (k1 values of C and of B).
+// (2^22 slots, 0.27 M rows of 4 states: 140 us with an atomic a row.)
+__global__ void __launch_bounds__(256) k_x_export(Problem P, const double *rows, int k1, unsigned long long *keys,
+                                                  double *C, double *B, long long cap, unsigned long long *counter) {
+    export_rows(P, cap, counter, [&](long long i, const Slot &sl, long long pos) {
+        if (keys) reinterpret_cast<ulonglong2 *>(keys)[pos] = make_ulonglong2(sl.a, sl.b & kKeyMaskB);
+        const double *r = rows + i * 2 * k1;
+        for (int a = 0; a < k1; ++a) {
+            if (C) C[pos * k1 + a] = r[a];
+            if (B) B[pos * k1 + a] = r[k1 + a];
+        }
     });
 }
 
@@ -1515,6 +1529,14 @@ cudaError_t launch_export(const Problem &P, const IterState *st, unsigned long l
     long long grid = (P.capacity + kExportTile - 1) / kExportTile;
     if (grid > 152 * 6) grid = 152 * 6;
     k_export<<<(int)grid, 256, 0, s>>>(P, st, keys, c, b, cap, counter);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_x_export(const Problem &P, const XBuffers &b, int k1, unsigned long long *keys, double *C,
+                            double *B, long long cap, unsigned long long *counter, cudaStream_t s) {
+    long long grid = (P.capacity + kExportTile - 1) / kExportTile;
+    if (grid > 152 * 6) grid = 152 * 6;
+    k_x_export<<<(int)grid, 256, 0, s>>>(P, b.rows, k1, keys, C, B, cap, counter);
     return cudaGetLastError();
 }
 

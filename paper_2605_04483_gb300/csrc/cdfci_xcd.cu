@@ -710,35 +710,9 @@ __global__ void k_x_diag_list(Problem P, const unsigned long long *keys, long lo
     }
 }
 
-// Every stored determinant with its rows (k1 values of C and of B).
-__global__ void k_x_export(Problem P, const double *rows, int k1, unsigned long long *keys, double *C, double *B,
-                           long long cap, unsigned long long *counter) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P.capacity;
-         i += (long long)gridDim.x * blockDim.x) {
-        const Slot sl = P.table[i];
-        if (sl.a == 0ull && sl.b == 0ull) continue;
-        const unsigned long long pos = atomicAdd(counter, 1ull);
-        if ((long long)pos >= cap) continue;
-        keys[2 * pos] = sl.a;
-        keys[2 * pos + 1] = sl.b & kKeyMaskB;
-        for (int a = 0; a < k1; ++a) {
-            C[pos * k1 + a] = rows[i * 2 * k1 + a];
-            B[pos * k1 + a] = rows[i * 2 * k1 + k1 + a];
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // host
 // ---------------------------------------------------------------------------
-cudaError_t launch_x_export(const Problem &P, const XBuffers &b, int k1, unsigned long long *keys, double *C,
-                            double *B, long long cap, unsigned long long *counter, cudaStream_t s) {
-    long long grid = (P.capacity + 255) / 256;
-    if (grid > 152 * 16) grid = 152 * 16;
-    k_x_export<<<(int)grid, 256, 0, s>>>(P, b.rows, k1, keys, C, B, cap, counter);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_x_diag_list(const Problem &P, const unsigned long long *keys, long long n, double *out,
                                cudaStream_t s) {
     const long long blocks = std::min<long long>((n + 7) / 8, 1024);
