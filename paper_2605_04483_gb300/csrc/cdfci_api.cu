@@ -1045,16 +1045,22 @@ CDFCI_API int cdfci_optorb(const double *h, const double *g, int M, int N, int n
     CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct StreamGuard { cudaStream_t s; ~StreamGuard() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{s};
     DevTemp tmp;
-    double *dh = tmp.alloc<double>(M2), *dg = tmp.alloc<double>(M4), *dU = tmp.alloc<double>(MN);
-    double *t1 = tmp.alloc<double>(M2 * M * N), *t2 = tmp.alloc<double>(M2 * N2), *g3 = tmp.alloc<double>(M * N3);
-    double *g4 = tmp.alloc<double>(N4), *hU = tmp.alloc<double>(MN), *h2 = tmp.alloc<double>(N2);
-    double *r1 = tmp.alloc<double>(N2), *r2 = tmp.alloc<double>(N4), *G = tmp.alloc<double>(MN);
-    double *Uo = tmp.alloc<double>(MN), *Go = tmp.alloc<double>(MN), *X = tmp.alloc<double>(MN);
-    double *Xn = tmp.alloc<double>(MN), *Gm = tmp.alloc<double>(N2), *Ub = tmp.alloc<double>(MN);
-    double *sc = tmp.alloc<double>(8);
-    if (!dh || !dg || !dU || !t1 || !t2 || !g3 || !g4 || !hU || !h2 || !r1 || !r2 || !G || !Uo || !Go || !X || !Xn ||
-        !Gm || !Ub || !sc)
-        return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+    // every array in one allocation
+    const long long sizes[] = {M2, M4, MN, M2 * M * N, M2 * N2, M * N3, N4, MN, N2, N2, N4, MN, MN, MN, MN, kOoParts + 4};
+    long long total = 0;
+    for (long long n : sizes) total += (n + 31) / 32 * 32;
+    double *mem = tmp.alloc<double>((size_t)total);
+    if (!mem) return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+    double *a[sizeof(sizes) / sizeof(sizes[0])];
+    long long at = 0;
+    for (size_t k = 0; k < sizeof(sizes) / sizeof(sizes[0]); ++k) {
+        a[k] = mem + at;
+        at += (sizes[k] + 31) / 32 * 32;
+    }
+    double *dh = a[0], *dg = a[1], *dU = a[2], *t1 = a[3], *t2 = a[4], *g3 = a[5], *g4 = a[6], *hU = a[7], *h2 = a[8];
+    double *r1 = a[9], *r2 = a[10], *G = a[11], *Uo = a[12], *Go = a[13], *Ub = a[14], *sc = a[15];
+    const OoState os{sc, sc + 1, sc + 4, reinterpret_cast<unsigned int *>(sc + 2), reinterpret_cast<int *>(sc + 3)};
+    CK(cudaMemsetAsync(sc, 0, 4 * sizeof(double), s));
     CK(cudaMemcpyAsync(dh, h, M2 * sizeof(double), cudaMemcpyDefault, s));
     CK(cudaMemcpyAsync(dg, g, M4 * sizeof(double), cudaMemcpyDefault, s));
     CK(cudaMemcpyAsync(dU, hU0.data(), MN * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -1068,36 +1074,6 @@ CDFCI_API int cdfci_optorb(const double *h, const double *g, int M, int N, int n
         if (e == cudaSuccess) e = oo_contract(dh, Uc, hU, M, M, N, 1, s);
         if (e == cudaSuccess) e = oo_contract(hU, Uc, h2, 1, M, N, N, s);
         return e;
-    };
-    auto read = [&](int k, double *out) -> int {
-        CK(cudaMemcpyAsync(out, sc, k * sizeof(double), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        return CDFCI_OK;
-    };
-    auto objective = [&](double *P) -> int {                       // P4 from h', g' and the RDMs
-        CK(oo_dot(h2, r1, N2, sc, s));
-        CK(oo_dot(g4, r2, N4, sc + 1, s));
-        double v[2];
-        int r = read(2, v);
-        *P = v[0] + 0.5 * v[1];
-        return r;
-    };
-    auto polar = [&]() -> int {                                    // X <- orth(X) (Newton-Schulz on X / ||X||_F)
-        CK(oo_dot(X, X, MN, sc, s));
-        CK(oo_scale(X, sc, MN, s));
-        std::vector<double> gm((size_t)N2);
-        for (int k = 0; k < 200; ++k) {
-            CK(oo_gram(X, Gm, M, N, s));
-            CK(cudaMemcpyAsync(gm.data(), Gm, N2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            double err = 0.0;
-            for (int a = 0; a < N; ++a)
-                for (int b = 0; b < N; ++b) err = std::max(err, std::fabs(gm[(size_t)a * N + b] - (a == b ? 1.0 : 0.0)));
-            if (err < 4e-16 * N) return CDFCI_OK;
-            CK(oo_ns(X, Gm, Xn, M, N, s));
-            std::swap(X, Xn);
-        }
-        return fail(CDFCI_ERR_INTERNAL, "the orthogonal projection did not converge");
     };
     for (int it = 0; it < p->outer; ++it) {
         CK(transform(dU));
@@ -1113,40 +1089,18 @@ CDFCI_API int cdfci_optorb(const double *h, const double *g, int M, int N, int n
         if (rc) return rc;
         energies[it] = st.energy;
         // the orbital subproblem with these RDMs
-        double P = 0.0, best = 0.0;
-        if ((rc = objective(&P))) return rc;
-        best = P;
-        CK(cudaMemcpyAsync(Ub, dU, bMN, cudaMemcpyDeviceToDevice, s));
-        CK(oo_grad(hU, r1, g3, r2, G, M, N, s));
-        CK(oo_dot(G, G, MN, sc, s));
-        double gg = 0.0;
-        if ((rc = read(1, &gg))) return rc;
-        double t = 0.1 / std::max(1.0, std::sqrt(gg));
+        CK(oo_objective(h2, r1, g4, r2, os, dU, Ub, M, N, 1, s));
+        if (p->bb_steps > 0) CK(oo_grad(hU, r1, g3, r2, G, M, N, s));
         for (int k = 0; k < p->bb_steps; ++k) {
-            if (k > 0) {
-                CK(oo_axpy(dU, Uo, 1.0, X, MN, s));                  // S = U - U_old
-                CK(oo_axpy(G, Go, 1.0, Xn, MN, s));                  // Y = G - G_old
-                CK(oo_dot(X, X, MN, sc, s));
-                CK(oo_dot(X, Xn, MN, sc + 1, s));
-                CK(oo_dot(Xn, Xn, MN, sc + 2, s));
-                double d[3];
-                if ((rc = read(3, d))) return rc;
-                if (std::fabs(d[1]) > 0.0 && d[2] > 0.0) t = (k % 2 == 1) ? d[0] / std::fabs(d[1]) : std::fabs(d[1]) / d[2];
-                t = std::min(std::max(t, 1e-10), 1e10);
-            }
-            CK(cudaMemcpyAsync(Uo, dU, bMN, cudaMemcpyDeviceToDevice, s));
-            CK(cudaMemcpyAsync(Go, G, bMN, cudaMemcpyDeviceToDevice, s));
-            CK(oo_axpy(dU, G, t, X, MN, s));                         // X = U - t grad
-            if ((rc = polar())) return rc;
-            CK(cudaMemcpyAsync(dU, X, bMN, cudaMemcpyDeviceToDevice, s));
+            CK(oo_move(dU, G, Uo, Go, os, k, M, N, s));
             CK(transform(dU));
-            CK(oo_grad(hU, r1, g3, r2, G, M, N, s));
-            if ((rc = objective(&P))) return rc;
-            if (P < best) {
-                best = P;
-                CK(cudaMemcpyAsync(Ub, dU, bMN, cudaMemcpyDeviceToDevice, s));
-            }
+            if (k + 1 < p->bb_steps) CK(oo_grad(hU, r1, g3, r2, G, M, N, s));
+            CK(oo_objective(h2, r1, g4, r2, os, dU, Ub, M, N, 0, s));
         }
+        int failed = 0;
+        CK(cudaMemcpyAsync(&failed, os.failed, sizeof(failed), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (failed) return fail(CDFCI_ERR_INTERNAL, "the orthogonal projection did not converge");
         CK(cudaMemcpyAsync(dU, Ub, bMN, cudaMemcpyDeviceToDevice, s));
     }
     CK(cudaMemcpyAsync(U, dU, bMN, cudaMemcpyDefault, s));

@@ -59,11 +59,16 @@ cudaError_t oo_contract(const double *in, const double *U, double *out, long lon
                         cudaStream_t s);
 cudaError_t oo_grad(const double *hU, const double *g1, const double *g3, const double *g2, double *G, int M, int N,
                     cudaStream_t s);
-cudaError_t oo_dot(const double *x, const double *y, long long n, double *out, cudaStream_t s);
-cudaError_t oo_axpy(const double *x, const double *z, double t, double *y, long long n, cudaStream_t s);
-cudaError_t oo_scale(double *x, const double *sq, long long n, cudaStream_t s);
-cudaError_t oo_gram(const double *X, double *Gm, int M, int N, cudaStream_t s);
-cudaError_t oo_ns(const double *X, const double *Gm, double *Xn, int M, int N, cudaStream_t s);
+constexpr int kOoParts = 152;          // most blocks of the objective's sum
+struct OoState {                       // the descent's scalars, on the device
+    double *t, *best, *part;           // step, lowest objective, the blocks' parts (kOoParts)
+    unsigned int *counter;             // the objective's finished blocks (zero between launches)
+    int *failed;                       // 1: an orthogonal projection did not converge
+};
+cudaError_t oo_objective(const double *h2, const double *r1, const double *g4, const double *r2, const OoState &st,
+                         const double *U, double *Ub, int M, int N, int first, cudaStream_t s);
+cudaError_t oo_move(double *U, const double *G, double *Uo, double *Go, const OoState &st, int k, int M, int N,
+                    cudaStream_t s);
 
 // checkpoint / restore
 cudaError_t launch_ckpt_export(const Problem &P, unsigned long long *keys, double *c, double *b, unsigned char *flags,
