@@ -678,6 +678,28 @@ __device__ __forceinline__ double line_search(double v1, double v2, double v3) {
                             [&](float x) { return halley_cubic((double)x, v1, v2, v3); });
 }
 
+// line_search by a whole warp (the same arguments in every lane; every lane
+// returns the result): f, f' and f'' of the Halley step as one Horner chain over
+// the lanes (see line_search_warp).
+__device__ __forceinline__ double line_search_lanes(float f1, float f2, float f3, double v1, double v2, double v3) {
+    const int l = threadIdx.x & 3;
+    const unsigned all = 0xffffffffu;
+    // coefficients (highest first) of lane 0: the cubic f, 1: f', 2: f'', 3: 2 f'
+    const double w = 3.0 * v3;
+    const double a3 = l == 0 ? 4.0 : 0.0, a2 = l == 0 ? w : (l == 1 ? 12.0 : (l == 2 ? 0.0 : 24.0));
+    const double s1 = (l == 0 ? v2 : w) * (l == 3 ? 4.0 : 2.0), a1 = l == 2 ? 24.0 : s1;
+    const double a0 = (l == 0 ? v1 : (l == 2 ? w : v2)) * (l == 0 ? 1.0 : (l == 3 ? 4.0 : 2.0));
+    return line_search_from(f1, f2, f3, v1, v2, v3, [&](float xf) {
+        const double x = (double)xf;
+        const double y = fma(fma(fma(a3, x, a2), x, a1), x, a0);
+        const double g = __shfl_sync(all, y, 0), g1 = __shfl_sync(all, y, 1), g2 = __shfl_sync(all, y, 2);
+        const double tg1 = __shfl_sync(all, y, 3);
+        const double den = fma(tg1, g1, -g * g2);
+        if (!(den != 0.0) || !isfinite(den)) return x;
+        return x - g * tg1 * recip(den);
+    });
+}
+
 // The same step size by a whole warp for one coordinate (c_i, b_i, H_ii and mu
 // in every lane; every lane returns it), bit for bit.  An FP64 instruction
 // takes its scheduler 64 cycles however many lanes it serves, so the lanes
@@ -697,20 +719,7 @@ __device__ __forceinline__ double line_search_warp(double ci, double bi, double 
     const unsigned all = 0xffffffffu;
     const float f1 = __shfl_sync(all, f, 0), f2 = __shfl_sync(all, f, 1), f3 = __shfl_sync(all, f, 2);
     const double v1 = __shfl_sync(all, v, 0), v2 = __shfl_sync(all, v, 1), v3 = __shfl_sync(all, v, 2);
-    // coefficients (highest first) of lane 0: the cubic f, 1: f', 2: f'', 3: 2 f'
-    const double w = 3.0 * v3;
-    const double a3 = l == 0 ? 4.0 : 0.0, a2 = l == 0 ? w : (l == 1 ? 12.0 : (l == 2 ? 0.0 : 24.0));
-    const double s1 = (l == 0 ? v2 : w) * (l == 3 ? 4.0 : 2.0), a1 = l == 2 ? 24.0 : s1;
-    const double a0 = (l == 0 ? v1 : (l == 2 ? w : v2)) * (l == 0 ? 1.0 : (l == 3 ? 4.0 : 2.0));
-    return line_search_from(f1, f2, f3, v1, v2, v3, [&](float xf) {
-        const double x = (double)xf;
-        const double y = fma(fma(fma(a3, x, a2), x, a1), x, a0);
-        const double g = __shfl_sync(all, y, 0), g1 = __shfl_sync(all, y, 1), g2 = __shfl_sync(all, y, 2);
-        const double tg1 = __shfl_sync(all, y, 3);
-        const double den = fma(tg1, g1, -g * g2);
-        if (!(den != 0.0) || !isfinite(den)) return x;
-        return x - g * tg1 * recip(den);
-    });
+    return line_search_lanes(f1, f2, f3, v1, v2, v3);
 }
 
 }  // namespace cdfci

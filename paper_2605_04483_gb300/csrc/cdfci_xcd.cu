@@ -17,7 +17,9 @@
 // What bounds an iteration is the latency of its dependent memory requests and
 // FP64 chains (a column of the N = 24 problem is one element a thread).  As four
 // launches (selection, preparation with S and M, column, recalculation) it took
-// 55.4 us with K + 1 = 4 (N = 24, 6 + 5 electrons), now 34.1 us.
+// 55.4 us with K + 1 = 4 (N = 24, 6 + 5 electrons), as two 34.1 us; now 29.6 us, with a warp
+// for each scheduler's FP64 pipe, H_ii beside the gradient in the step, independent sums over the
+// lanes and the loads that start a kernel ahead of its flags.
 // The energies (the pencil (M, S)) are computed on request by k_x_energies.
 // Each row j occurs once in a column, so B_j is updated by plain loads and
 // stores, and every reduction has a fixed order: the iteration is
@@ -48,9 +50,13 @@ __device__ __forceinline__ bool x_better(const XBest &x, const XBest &y) {
 }
 
 
-// ||G_j||_inf, G_j = 4 B_j + 4 C_j S, from the row's C and B halves
-__device__ __forceinline__ double x_gnorm(const double (&c)[kXMax], const double (&bb)[kXMax], const double *S, int k1) {
-    double m = 0.0;
+// max_a |B_a + (C S)_a| as a bit pattern (||G_j||_inf / 4, G_j = 4 B_j + 4 C_j S; the
+// factor changes no rounding and no order), from the row's C and B halves; a NaN
+// counts as zero.  Every FP64 instruction takes its scheduler 64 cycles, so the
+// maximum is taken over the bits.
+__device__ __forceinline__ unsigned long long x_gnorm(const double (&c)[kXMax], const double (&bb)[kXMax],
+                                                      const double *S, int k1) {
+    unsigned long long m = 0ull;
 #pragma unroll
     for (int a = 0; a < kXMax; ++a) {
         if (a >= k1) break;
@@ -60,14 +66,48 @@ __device__ __forceinline__ double x_gnorm(const double (&c)[kXMax], const double
             if (b >= k1) break;
             s = fma(c[b], S[b * k1 + a], s);
         }
-        m = fmax(m, fabs(4.0 * bb[a] + 4.0 * s));
+        const unsigned long long x = x_abs_bits(bb[a] + s);
+        if (x <= 0x7ff0000000000000ull && x > m) m = x;
     }
     return m;
 }
 
+// Sums of the k1 values over the warp, the values halved with the lanes: 6 FP64
+// additions for up to 4 values and 9 for 8, instead of 5 a value.  Lane l returns
+// the sum of value x_sum_of(l, k1); its copies are the lanes of equal result.
+__device__ __forceinline__ int x_sum_of(int lane, int k1) {
+    return k1 > 4 ? (lane >> 2) : (lane >> 3);
+}
+__device__ __forceinline__ double x_warp_sums(double (&v)[kXMax], int k1) {
+    const int lane = threadIdx.x & 31;
+    const unsigned all = 0xffffffffu;
+    double x[4];
+    int o = 16;
+    if (k1 > 4) {                                                    // uniform
+        const bool up = lane & 16;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = (up ? v[q + 4] : v[q]) + __shfl_xor_sync(all, up ? v[q] : v[q + 4], 16);
+        o = 8;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = v[q];
+    }
+    bool up = lane & o;
+    const double y0 = (up ? x[2] : x[0]) + __shfl_xor_sync(all, up ? x[0] : x[2], o);
+    const double y1 = (up ? x[3] : x[1]) + __shfl_xor_sync(all, up ? x[1] : x[3], o);
+    o >>= 1;
+    up = lane & o;
+    double z = (up ? y1 : y0) + __shfl_xor_sync(all, up ? y0 : y1, o);
+    for (o >>= 1; o > 0; o >>= 1) z += __shfl_xor_sync(all, z, o);
+    return z;
+}
+
 }  // namespace
 
-constexpr int kXThreads = 256;
+// Four warps a block, one for each scheduler of an SM: a column of the N = 24
+// problem (14.5 k elements) is then a warp a scheduler, where eight warps on half
+// the SMs shared their FP64 pipes.
+constexpr int kXThreads = 128;
 
 // Row j of C and of B (k1 values each) into cv and bv, all loads in flight
 // together: 16-byte loads when k1 is even (each half is then whole pairs, and
@@ -154,147 +194,195 @@ __device__ __forceinline__ double x_diag(const Problem &P, const ColLists &L) {
     return __shfl_sync(0xffffffffu, x, 0);
 }
 
-// The step of the chosen row (warp 0 of a block): H_ii, the quartic and eta, the
-// scatter weights, C_i += eta g; c and b of the row as they were are left for the
-// update of S and M.  forced >= 0: the start step of row {fA, fB} with g =
-// e_forced and eta = 1.
+// The step of the chosen row (warps 0 and 1 of a block): H_ii, the quartic and
+// eta, the scatter weights, C_i += eta g; c and b of the row as they were are left
+// for the update of S and M.  forced >= 0: the start step of row {fA, fB} with g =
+// e_forced and eta = 1.  Warp 1 computes H_ii beside the gradient and its products
+// and keeps the books beside the update of C; independent sums are spread over
+// the lanes (an FP64 instruction costs its issue, not its lanes).
 struct XStepShared {
     ColLists L;
     double c[kXMax], g[kXMax], b[kXMax], t[kXMax];
-    double eta, gn;
+    double eta, gn, Hii;
     int stop;
 };
+__device__ __forceinline__ void x_pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 __device__ void x_step(const Problem &P, XState *xs, IterState *st, double *rows, const double *sS, XStepShared &W,
                        long long s, unsigned long long A, unsigned long long B, int forced) {
-    const int k1 = xs->k1, lane = threadIdx.x & 31;
-    if (lane < k1) {                                                  // loads in flight beside the lists
-        W.c[lane] = __ldcg(rows + s * 2 * k1 + lane);
-        W.b[lane] = __ldcg(rows + s * 2 * k1 + k1 + lane);
+    const int k1 = xs->k1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned all = 0xffffffffu;
+    double c0 = 0.0, b0 = 0.0, g0 = 0.0;
+    if (warp == 1) {
+        for (int t = lane; t < P.N; t += 32) {
+            const int ra = __popcll(A & low_mask(t)), rb = __popcll(B & low_mask(t));
+            if ((A >> t) & 1ull) W.L.occA[ra] = (unsigned char)t; else W.L.virA[t - ra] = (unsigned char)t;
+            if ((B >> t) & 1ull) W.L.occB[rb] = (unsigned char)t; else W.L.virB[t - rb] = (unsigned char)t;
+        }
+        __syncwarp();
+        const double Hii = x_diag(P, W.L);
+        if (lane == 0) W.Hii = Hii;
+        x_pair_sync();
+        x_pair_sync();                                                // the step is known
+        if (W.stop) return;
+        if (lane == 0) {
+            xs->slot = s; xs->A = A; xs->B = B;
+            xs->eta = W.eta;
+            xs->Hii = Hii;
+            xs->go = 1;
+            if (forced < 0) {
+                const double dx = P.theta * xs->dx + (1.0 - P.theta) * fabs(W.eta) * W.gn;   // W.gn = ||g||
+                xs->dx = dx;
+                xs->iterations += 1;
+                if (P.dx_threshold > 0.0 && dx < P.dx_threshold) xs->done = 1;
+            }
+        }
+        return;
     }
-    for (int t = lane; t < P.N; t += 32) {
-        const int ra = __popcll(A & low_mask(t)), rb = __popcll(B & low_mask(t));
-        if ((A >> t) & 1ull) W.L.occA[ra] = (unsigned char)t; else W.L.virA[t - ra] = (unsigned char)t;
-        if ((B >> t) & 1ull) W.L.occB[rb] = (unsigned char)t; else W.L.virB[t - rb] = (unsigned char)t;
+    if (lane < k1) {
+        c0 = __ldcg(rows + s * 2 * k1 + lane);
+        b0 = __ldcg(rows + s * 2 * k1 + k1 + lane);
+        W.c[lane] = c0;
+        W.b[lane] = b0;
     }
     if (lane == 0) W.stop = 0;
     __syncwarp();
     if (lane < k1) {                                                  // G_a, lane a
         double m = 0.0;
         for (int b = 0; b < k1; ++b) m = fma(W.c[b], sS[b * k1 + lane], m);
-        W.g[lane] = forced >= 0 ? (lane == forced ? 1.0 : 0.0) : 4.0 * W.b[lane] + 4.0 * m;
+        g0 = forced >= 0 ? (lane == forced ? 1.0 : 0.0) : 4.0 * b0 + 4.0 * m;
+        W.g[lane] = g0;
     }
     __syncwarp();
-    const double Hii = x_diag(P, W.L);
     if (lane < k1 && forced < 0) {                                    // (S g)_a, lane a: the term of g S g^T
         double t = 0.0;
         for (int b = 0; b < k1; ++b) t = fma(sS[lane * k1 + b], W.g[b], t);
         W.t[lane] = t;
     }
     __syncwarp();
-    if (lane == 0) {
-        double eta = 1.0;
-        if (forced < 0) {
-            // h(eta) = f(C + eta e_i g) - f(C) = w4 eta^4 + w3 eta^3 + w2 eta^2 + w1 eta with w4 = ||g||^4,
-            // w3 = 4 ||g||^2 c.g, w2 = 2 H_ii ||g||^2 + 2 (c.g)^2 + 2 ||c||^2 ||g||^2 + 2 g S g^T,
-            // w1 = ||g||^2 (the directional derivative)
-            double gg = 0.0, cg = 0.0, cc = 0.0, gSg = 0.0;
-            for (int a = 0; a < k1; ++a) {
-                gg = fma(W.g[a], W.g[a], gg);
-                cg = fma(W.c[a], W.g[a], cg);
-                cc = fma(W.c[a], W.c[a], cc);
-                gSg = fma(W.g[a], W.t[a], gSg);
-            }
-            // In t = eta ||g|| the quartic is monic with O(1) coefficients (w / w4 would grow like
-            // 1 / ||g||^2 near convergence and overflow the single-precision root stage):
-            // t^4 + 4 (c.u) t^3 + (2 H_ii + 2 (c.u)^2 + 2 ||c||^2 + 2 u S u^T) t^2 + ||g|| t, u = g / ||g||.
-            const double ign = rsqrt(gg), gn = gg * ign;
-            W.gn = gn;
-            if (!(gn > 0.0)) { xs->done = 1; W.stop = 1; }
-            else {
-                const double cu = cg * ign;
-                const double v3 = 4.0 * cu;
-                const double v2 = 2.0 * Hii + 2.0 * cu * cu + 2.0 * cc + 2.0 * (gSg * ign) * ign;
-                eta = line_search(gn, v2, v3) * ign;
-                if (!isfinite(eta)) { set_status(st, kErrNonfinite); W.stop = 1; }
+    // h(eta) = f(C + eta e_i g) - f(C) = w4 eta^4 + w3 eta^3 + w2 eta^2 + w1 eta with w4 = ||g||^4,
+    // w3 = 4 ||g||^2 c.g, w2 = 2 H_ii ||g||^2 + 2 (c.g)^2 + 2 ||c||^2 ||g||^2 + 2 g S g^T,
+    // w1 = ||g||^2 (the directional derivative).  Lane 0 sums g.g, 1 c.g, 2 c.c, 3 g.(S g).
+    const double *x = (lane & 3) == 0 || (lane & 3) == 3 ? W.g : W.c;
+    const double *y = (lane & 3) == 3 ? W.t : ((lane & 3) == 2 ? W.c : W.g);
+    double d = 0.0;
+    if (forced < 0)
+        for (int a = 0; a < k1; ++a) d = fma(x[a], y[a], d);
+    const double gg = __shfl_sync(all, d, 0), cg = __shfl_sync(all, d, 1), cc = __shfl_sync(all, d, 2);
+    const double gSg = __shfl_sync(all, d, 3);
+    // In t = eta ||g|| the quartic is monic with O(1) coefficients (w / w4 would grow like
+    // 1 / ||g||^2 near convergence and overflow the single-precision root stage):
+    // t^4 + 4 (c.u) t^3 + (2 H_ii + 2 (c.u)^2 + 2 ||c||^2 + 2 u S u^T) t^2 + ||g|| t, u = g / ||g||.
+    double ign = 1.0, gn = 1.0, v3 = 0.0, part = 0.0, us = 0.0;
+    if (forced < 0) {
+        ign = rsqrt(gg);
+        gn = gg * ign;
+        const double cu = cg * ign;
+        v3 = 4.0 * cu;
+        part = 2.0 * cu * cu;
+        us = 2.0 * (gSg * ign) * ign;
+    }
+    x_pair_sync();
+    const double Hii = W.Hii;
+    double eta = 1.0;
+    bool stop = false;
+    if (forced < 0) {
+        if (!(gn > 0.0)) {
+            stop = true;
+            if (lane == 0) xs->done = 1;
+        } else {
+            const double v2 = 2.0 * Hii + part + 2.0 * cc + us;
+            eta = line_search_lanes((float)gn, (float)v2, (float)v3, gn, v2, v3) * ign;
+            if (!isfinite(eta)) {
+                stop = true;
+                if (lane == 0) set_status(st, kErrNonfinite);
             }
         }
-        W.eta = eta;
     }
-    __syncwarp();
-    if (W.stop) return;
-    const double eta = W.eta;
+    if (lane == 0) {
+        W.eta = eta;
+        W.gn = gn;
+        W.stop = stop ? 1 : 0;
+    }
+    x_pair_sync();
+    if (stop) return;                                                 // uniform
     // C_i += eta g (lane a), the scatter weights eta g and their largest magnitude
     const bool on = lane < k1;
     double cn = 0.0, wa = 0.0;
     if (on) {
-        const double c0 = W.c[lane], g0 = W.g[lane];
         cn = fma(eta, g0, c0);
         rows[s * 2 * k1 + lane] = cn;
         wa = eta * g0;
         xs->wv[lane] = wa;
         xs->g[lane] = g0;
         xs->c_old[lane] = c0;
-        xs->b_old[lane] = W.b[lane];
+        xs->b_old[lane] = b0;
     }
-    const unsigned was = __ballot_sync(0xffffffffu, on && W.c[lane & (kXMax - 1)] != 0.0);
-    const unsigned now = __ballot_sync(0xffffffffu, on && cn != 0.0);
-    double wmax = fabs(wa);
+    const unsigned was = __ballot_sync(all, on && !is_zero(c0));
+    const unsigned now = __ballot_sync(all, on && !is_zero(cn));
+    unsigned long long wb = x_abs_bits(wa);                           // (finite: eta is, and g with it)
 #pragma unroll
-    for (int off = kXMax / 2; off > 0; off >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, off));
+    for (int off = kXMax / 2; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(all, wb, off);
+        wb = o > wb ? o : wb;
+    }
     if (lane == 0) {
-        xs->slot = s; xs->A = A; xs->B = B;
+        const double wmax = __longlong_as_double((long long)wb);
         xs->nnz_c += (now ? 1 : 0) - (was ? 1 : 0);
         xs->thr = wmax > 0.0 ? (P.tau > 0.0 ? P.tau / wmax : 0.0) : 1.0e308;
-        xs->eta = eta;
-        xs->Hii = Hii;
-        xs->go = 1;
-        if (forced < 0) {
-            xs->dx = P.theta * xs->dx + (1.0 - P.theta) * fabs(eta) * W.gn;   // W.gn = ||g||
-            xs->iterations += 1;
-            if (P.dx_threshold > 0.0 && xs->dx < P.dx_threshold) xs->done = 1;
-        }
     }
 }
 
 __global__ void __launch_bounds__(kXThreads) k_x_choose(Problem P, XState *xs, IterState *st, const long long *cand,
-                                                        double *rows, XBest *bbest, unsigned int *counter, int forced,
-                                                        unsigned long long fA, unsigned long long fB) {
+                                                        long long cap_cand, double *rows, XBest *bbest,
+                                                        unsigned int *counter, int forced, unsigned long long fA,
+                                                        unsigned long long fB) {
     __shared__ double sS[kXMax * kXMax];
-    __shared__ XBest wb[kXThreads / 32];
+    __shared__ XBest wb[kXThreads / 32], s_best;
     __shared__ XStepShared W;
     __shared__ bool s_last;
-    __shared__ long long s_slot;
-    const int k1 = xs->k1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (xs->done || st->status) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // every load that needs no other first: the flags, S, the count, this thread's first candidate
+    const int t0 = blockIdx.x * blockDim.x + tid;
+    const dd Sx = tid < kXMax * kXMax ? xs->S[tid] : dd{0.0, 0.0};
+    const int k1 = xs->k1, n = xs->n_cand, done = xs->done, status = st->status;
+    long long s = t0 < cap_cand ? cand[t0] : 0;
+    if (done || status) {
         if (blockIdx.x == 0 && tid == 0) xs->go = 0;                 // no step this iteration
         return;
     }
-    for (int t = tid; t < k1 * k1; t += blockDim.x) sS[t] = xs->S[t].hi + xs->S[t].lo;
-    __syncthreads();
     if (forced >= 0) {                                               // one block
-        if (warp != 0) return;
-        if (lane == 0) {
+        if (tid < k1 * k1) sS[tid] = Sx.hi + Sx.lo;
+        if (tid == 0) {
             xs->go = 0;
             xs->eta = 0.0;
             bool ins = false;
-            const long long s = table_find(P, st, fA, fB, true, &ins);
-            if (s >= 0 && ins) { xs->n_slots += 1; xs->inserted += 1; }
-            s_slot = s;
+            const long long at = table_find(P, st, fA, fB, true, &ins);
+            if (at >= 0 && ins) { xs->n_slots += 1; xs->inserted += 1; }
+            s_best.slot = at;
         }
-        __syncwarp();
-        if (s_slot >= 0) x_step(P, xs, st, rows, sS, W, s_slot, fA, fB, forced);
+        __syncthreads();
+        if (s_best.slot >= 0 && warp <= 1) x_step(P, xs, st, rows, sS, W, s_best.slot, fA, fB, forced);
         return;
     }
-    const int n = xs->n_cand;
     XBest best{0ull, ~0ull, ~0ull, -1};
-    for (int t = blockIdx.x * blockDim.x + tid; t < n; t += gridDim.x * blockDim.x) {
-        const long long s = cand[t];
-        double rc[kXMax], rb[kXMax];
+    double rc[kXMax], rb[kXMax];
+    ulonglong2 key = make_ulonglong2(0ull, 0ull);
+    if (t0 < n) {
         x_load_row(rows, s, k1, rc, rb);
-        const ulonglong2 key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + s));
-        P.table[s].b = key.y & kKeyMaskB;                          // no longer a candidate
-        const XBest x{x_abs_bits(x_gnorm(rc, rb, sS, k1)), key.x, key.y & kKeyMaskB, s};
+        key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + s));
+    }
+    if (tid < k1 * k1) sS[tid] = Sx.hi + Sx.lo;
+    __syncthreads();
+    for (int t = t0; t < n;) {
+        P.table[s].b = key.y & kKeyMaskB;                            // no longer a candidate
+        const XBest x{x_gnorm(rc, rb, sS, k1), key.x, key.y & kKeyMaskB, s};
         if (x_better(x, best)) best = x;
+        t += gridDim.x * blockDim.x;
+        if (t < n) {
+            s = cand[t];
+            x_load_row(rows, s, k1, rc, rb);
+            key = __ldcg(reinterpret_cast<const ulonglong2 *>(P.table + s));
+        }
     }
     auto warp_best = [&](XBest b) {
         for (int off = 16; off > 0; off >>= 1) {
@@ -319,26 +407,30 @@ __global__ void __launch_bounds__(kXThreads) k_x_choose(Problem P, XState *xs, I
         s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!s_last || warp != 0) return;
+    if (!s_last || warp > 1) return;
     __threadfence();
-    // the last block's warp 0 reduces the blocks' winners (lane l takes blocks l, l + 32, ...) and takes the step
-    XBest b{0ull, ~0ull, ~0ull, -1};
-    for (int k = lane; k < (int)gridDim.x; k += 32) {
-        const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(bbest + k);
-        const ulonglong2 x = __ldcg(q), y = __ldcg(q + 1);
-        const XBest z{x.x, x.y, y.x, (long long)y.y};
-        if (x_better(z, b)) b = z;
+    // the last block's warp 0 reduces the blocks' winners (lane l takes blocks l, l + 32, ...), and
+    // warps 0 and 1 take the step
+    if (warp == 0) {
+        XBest b{0ull, ~0ull, ~0ull, -1};
+        for (int k = lane; k < (int)gridDim.x; k += 32) {
+            const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(bbest + k);
+            const ulonglong2 x = __ldcg(q), y = __ldcg(q + 1);
+            const XBest z{x.x, x.y, y.x, (long long)y.y};
+            if (x_better(z, b)) b = z;
+        }
+        b = warp_best(b);
+        if (lane == 0) {
+            *counter = 0u;
+            xs->n_cand = 0;
+            xs->go = 0;
+            xs->eta = 0.0;
+            if (b.slot < 0) xs->done = 1;                            // nothing left to choose
+            s_best = b;
+        }
     }
-    b = warp_best(b);
-    if (lane == 0) {
-        *counter = 0u;
-        xs->n_cand = 0;
-        xs->go = 0;
-        xs->eta = 0.0;
-        if (b.slot < 0) xs->done = 1;                                // nothing left to choose
-    }
-    __syncwarp();
-    if (b.slot >= 0) x_step(P, xs, st, rows, sS, W, b.slot, b.a, b.b, -1);
+    x_pair_sync();
+    if (s_best.slot >= 0) x_step(P, xs, st, rows, sS, W, s_best.slot, s_best.a, s_best.b, -1);
 }
 
 // The slot of key {a, b} by linear probing from pos (no insert), whose first key
@@ -425,7 +517,6 @@ __global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, I
     __shared__ double sw[kXMax];
     __shared__ double sg[kXThreads / 32][kXMax];
     __shared__ unsigned int s_cnt[4][kXThreads / 32];
-    __shared__ double red[kXMax][kXThreads];
     __shared__ bool s_last;
     if (!xs->go) return;                                             // no step this iteration
     const int nb = (int)gridDim.x - 1;                               // blocks of the column; one more for S and M
@@ -473,7 +564,7 @@ __global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, I
 #pragma unroll
                 for (int a = 0; a < kXMax; ++a) {
                     if (at < 0) rc[a] = rb[a] = 0.0;                 // a row that is not there yet is zero
-                    cnz = cnz || (a < k1 && rc[a] != 0.0);
+                    cnz = cnz || (a < k1 && !is_zero(rc[a]));
                 }
                 if (at != -2 && !cnz && !(fabs(H) >= thr)) {
                     ++c2;
@@ -530,13 +621,11 @@ __global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, I
             }
         }
     }
-    // gather: warp tree, then warps in order (fixed order)
-#pragma unroll
-    for (int a = 0; a < kXMax; ++a) {
-        if (a >= k1) break;
-        double v = gat[a];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) sg[warp][a] = v;
+    // gather: warp sums, then warps in order (fixed order)
+    {
+        const double v = x_warp_sums(gat, k1);
+        const int a = x_sum_of(lane, k1);
+        if (a < k1 && (lane & (k1 > 4 ? 3 : 7)) == 0) sg[warp][a] = v;
     }
     // counters: warp sums (no shared-memory atomics), then the warps in order
     c0 = __reduce_add_sync(0xffffffffu, c0); c1 = __reduce_add_sync(0xffffffffu, c1);
@@ -564,7 +653,8 @@ __global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, I
     if (st->status) return;
     const long long s = xs->slot;
     const double Hii = xs->Hii;
-    // every state at once: per state, the thread's blocks in order, then the same pairwise tree
+    const double cs = tid < k1 ? __ldcg(rows + s * 2 * k1 + tid) : 0.0;
+    // per state: the thread's blocks in order, the warp's sums, the warps in order
     double v[kXMax];
 #pragma unroll
     for (int a = 0; a < kXMax; ++a) v[a] = 0.0;
@@ -573,17 +663,16 @@ __global__ void __launch_bounds__(kXThreads) k_x_column(Problem P, XState *xs, I
         for (int a = 0; a < kXMax; ++a)
             if (a < k1) v[a] += __ldcg(gathp + (size_t)k * k1 + a);
     }
-#pragma unroll
-    for (int a = 0; a < kXMax; ++a)
-        if (a < k1) red[a][tid] = v[a];
+    {
+        const double t = x_warp_sums(v, k1);
+        const int a = x_sum_of(lane, k1);
+        if (a < k1 && (lane & (k1 > 4 ? 3 : 7)) == 0) sg[warp][a] = t;
+    }
     __syncthreads();
-    // (256 partial sums per state: warp a adds state a's, 8 per lane in order, then a tree)
-    if (warp < k1) {
-        double t = 0.0;
-#pragma unroll
-        for (int q = 0; q < kXThreads / 32; ++q) t += red[warp][32 * q + lane];
-        for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-        if (lane == 0) rows[s * 2 * k1 + k1 + warp] = fma(Hii, __ldcg(rows + s * 2 * k1 + warp), t);
+    if (tid < k1) {
+        double t = sg[0][tid];
+        for (int w = 1; w < kXThreads / 32; ++w) t += sg[w][tid];
+        rows[s * 2 * k1 + k1 + tid] = fma(Hii, cs, t);
     }
     if (tid == 0) {
         const unsigned long long kb = P.table[s].b;
@@ -720,13 +809,13 @@ cudaError_t launch_x_diag_list(const Problem &P, const unsigned long long *keys,
     return cudaGetLastError();
 }
 
-// blocks of a column: an element per thread, at most two blocks per SM; of the choice: a candidate
-// per thread, at most one block per SM
+// blocks of a column: an element per thread, at most four blocks per SM; of the choice: a candidate
+// per thread, at most two blocks per SM
 int x_scatter_blocks(const Problem &P) {
     const long long nh = P.doubles_vanish ? P.seg[2] : P.seg[5];
-    return (int)std::max<long long>(1, std::min<long long>(152 * 2, (nh - 1 + kXThreads - 1) / kXThreads));
+    return (int)std::max<long long>(1, std::min<long long>(152 * 4, (nh - 1 + kXThreads - 1) / kXThreads));
 }
-int x_select_blocks(const Problem &P) { return std::min(152, x_scatter_blocks(P)); }
+int x_select_blocks(const Problem &P) { return std::min(152 * 2, x_scatter_blocks(P)); }
 
 size_t x_block_bytes() { return sizeof(XBest); }
 
@@ -737,12 +826,12 @@ static cudaError_t launch_x_column(const Problem &P, const XBuffers &b, cudaStre
 
 cudaError_t launch_x_start(const Problem &P, const XBuffers &b, unsigned long long A, unsigned long long B, int k,
                            cudaStream_t s) {
-    k_x_choose<<<1, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.rows, static_cast<XBest *>(b.bbest), b.counter, k, A, B);
+    k_x_choose<<<1, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.cap_cand, b.rows, static_cast<XBest *>(b.bbest), b.counter, k, A, B);
     return launch_x_column(P, b, s);
 }
 
 cudaError_t launch_x_iteration(const Problem &P, const XBuffers &b, cudaStream_t s) {
-    k_x_choose<<<b.nselect, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.rows, static_cast<XBest *>(b.bbest), b.counter,
+    k_x_choose<<<b.nselect, kXThreads, 0, s>>>(P, b.xs, b.st, b.cand, b.cap_cand, b.rows, static_cast<XBest *>(b.bbest), b.counter,
                                                -1, 0ull, 0ull);
     return launch_x_column(P, b, s);
 }
