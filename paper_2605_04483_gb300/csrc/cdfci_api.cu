@@ -919,11 +919,13 @@ struct PairBuffers {
     void *mem = nullptr;
     PairList Q{};
     double *extra = nullptr;
+    static constexpr long long kMost = 1ll << 31;      // positions are 32 bits, the table has twice as many records
+    bool at_most() const { return Q.cap >= kMost; }
     ~PairBuffers() { cudaFree(mem); }
     int make(const Problem &P, long long est, size_t n_extra) {
         cudaFree(mem);
         mem = nullptr;
-        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, 1ll << 29)));
+        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, kMost)));
         pair_sizes(P, est, &Q);
         size_t at = 0;
         auto part = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
@@ -958,6 +960,8 @@ int exact_rq(cdfci_ctx *c, const Problem &P, double *E) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "energy: %s", cudaGetErrorString(e));
+        if (n > pb.Q.cap && pb.at_most())
+            return fail(CDFCI_ERR_NOMEM, "more than 2^31 determinants with c != 0");
     } while (n > pb.Q.cap);
     return fill_stats(c, nullptr);
 }
@@ -1632,6 +1636,8 @@ int rdm_device(cdfci_ctx *c, double *g1, double *g2) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "rdm: %s", cudaGetErrorString(e));
+        if (n > pb.Q.cap && pb.at_most())
+            return fail(CDFCI_ERR_NOMEM, "more than 2^31 determinants with c != 0");
     } while (n > pb.Q.cap);
     if (!(norm > 0.0)) return fail(CDFCI_ERR_ARG, "rdm: the stored vector is zero");
     return CDFCI_OK;
