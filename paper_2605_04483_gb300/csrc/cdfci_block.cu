@@ -2287,12 +2287,18 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
                     float mu, yx = 1.0f, yw, yp;
                     if (!ritz_near(s, have_p, mu, yw, yp)) ritz_full(s, have_p, mu, yx, yw, yp);
                     // the next p = yw w + yp p: its length, and its part along the new x = yx x + p
-                    const float pn2 = yw * (yw * s.ww + 2.0f * yp * s.wp) + yp * yp * s.pp;
-                    const float xp0 = yx * (yw * s.xw + yp * s.xp);
+                    float pn2 = yw * (yw * s.ww + 2.0f * yp * s.wp) + yp * yp * s.pp;
+                    float xp0 = yx * (yw * s.xw + yp * s.xp);
+                    float xn = yx * yx * s.xx + 2.0f * xp0 + pn2;             // |new x|^2
+                    // where x is exact up to rounding (a symmetric block can be solved in one iteration) w is
+                    // rounding too and the pencil without meaning: a pair whose parts cancel is no step
+                    if (!(yx * yx * s.xx < 1e4f * xn)) {
+                        mu = 0.0f; yx = 1.0f; yw = 0.0f; yp = 0.0f;
+                        pn2 = 0.0f; xp0 = 0.0f; xn = s.xx;
+                    }
                     if (lane == 0) {
                         s_y[0] = mu; s_y[1] = yx; s_y[2] = yw; s_y[3] = yp;
                         s_y[4] = pn2 > 0.0f ? rsqrtf(pn2) : 0.0f;
-                        const float xn = yx * yx * s.xx + 2.0f * xp0 + pn2;   // |new x|^2
                         s_y[5] = __fdividef(xp0 + pn2, xn);
                         s_y[6] = xn;
                     }
