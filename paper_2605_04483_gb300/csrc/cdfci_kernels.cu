@@ -235,6 +235,22 @@ __device__ __forceinline__ void issue_elem(const Problem &P, const ColLists &L, 
     x.state = 4;
 }
 
+// Whether issue_elem compares an element of the column of {iA, iB} with {pA, pB}
+// (another determinant): the singles, and unless every double vanishes the
+// doubles, of opposite spins only where they conserve momentum.
+// (Out of line and of plain arguments: a rare branch of the loop, which keeps its registers and its code.)
+static __device__ __noinline__ bool column_meets(int doubles_vanish, const unsigned char *ksub, const unsigned char *kadd,
+                                                 int N, unsigned long long iA, unsigned long long iB,
+                                                 unsigned long long pA, unsigned long long pB) {
+    const int dA = __popcll(iA ^ pA), d = dA + __popcll(iB ^ pB);
+    if (d > 4 || (d > 2 && doubles_vanish)) return false;
+    if (dA != 2 || d == 2 || !ksub) return true;
+    auto transfer = [&](unsigned long long X, unsigned long long Y) {       // of the single excitation X -> Y
+        return (int)__ldg(ksub + (__ffsll((long long)(X & ~Y)) - 1) * N + (__ffsll((long long)(Y & ~X)) - 1));
+    };
+    return __ldg(kadd + transfer(iA, pA) * N + transfer(iB, pB)) == 0;       // (k_conserved)
+}
+
 // Finish the lookup of an issued element: compare the loaded slot, then probe
 // on, kProbeAhead slots a load: the warp waits for its slowest lane, and a
 // dependent probe is an L2 round trip (700 cycles and more), of which every
@@ -677,10 +693,10 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 if (ls.forced) {
                     // a start vector's entry: insert it if absent; its c and b as stored now.  The
                     // previous coordinate's recalculated b is written by the element thread that meets
-                    // it in this column; an entry more than a double excitation away has no such
-                    // element, so CTA 0 writes it here.
+                    // it in this column; where no element of the column is that coordinate, CTA 0
+                    // writes it here.
                     if (ls.have_prev && rank == 0 &&
-                        __popcll(ls.pA ^ ls.fa) + __popcll(ls.pB ^ ls.fb) > 4)
+                        !column_meets(P.doubles_vanish, P.ksub, P.kadd, P.N, ls.fa, ls.fb, ls.pA, ls.pB))
                         P.table[ls.pslot].bv = pb;
                     // every CTA looks the entry up; the one whose insert wins counts it in its partial
                     bool ins = false;
