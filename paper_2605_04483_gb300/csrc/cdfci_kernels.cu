@@ -539,6 +539,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
     __shared__ LoopState ls;                     // written by lane 0 of the control warp (warp 0) only
     __shared__ int s_err;
     __shared__ int s_fins;                       // 1: this CTA inserted the forced coordinate of this step
+    __shared__ int s_owed;                       // CTA 0: 1: the c of a forced step is not in the table yet
     __shared__ int s_tmo;                        // grid mode: a wait for the partials expired
     __shared__ CdPartial s_x1[kGrid ? 2 : 1][32];   // grid mode: the partials polled by warps 0 and 1
     extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -574,6 +575,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
         s_err = 0;
         s_done = 0;
         s_fins = 0;
+        s_owed = 0;
         s_tmo = 0;
     }
     if (kGrid) __syncthreads(); else cluster.sync();
@@ -723,6 +725,15 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
         }
         }
         __syncthreads();
+        // Every CTA reads c and b of a forced coordinate's slot by itself, and nothing orders those reads
+        // before the end of the same iteration: CTA 0 writes that slot's c here, an iteration later (every
+        // CTA has since passed a cluster barrier or published its partial), or behind the loop.  Nobody
+        // reads it in between: in this iteration the slot is the previous coordinate's, whose c every CTA
+        // has.  (Its b stays as it was read until the recalculated one is written.)
+        if (tid == 32 && s_owed && !s_tmo) {
+            P.table[sel.pslot].c = sel.pc;
+            s_owed = 0;
+        }
         if (sel.stop) break;                          // identical in every CTA of the cluster
         const unsigned long long iA = sel.iA, iB = sel.iB;
         const bool have_prev = sel.have_prev != 0;
@@ -925,10 +936,14 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 s_fins = 0;
                 pp.err = s_err | (bad ? 1 : 0);
                 if (kGrid) spart[0] = pp; else spart[pout] = pp;
-                // the coordinate's own slot: c_i += eta, b_i as used (rank 0 writes)
+                // the coordinate's own slot: c_i += eta, b_i as used (rank 0 writes; a forced one later)
                 if (rank == 0 && !bad) {
-                    P.table[sel.islot].c = ls.pc;
-                    P.table[sel.islot].bv = sel.bi;
+                    if (G > 1 && sel.forced) {
+                        s_owed = 1;
+                    } else {
+                        P.table[sel.islot].c = ls.pc;
+                        P.table[sel.islot].bv = sel.bi;
+                    }
                 }
                 if (bad && rank == 0) set_status(st, kErrNonfinite);
             }
@@ -967,12 +982,16 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             if (fin) {
                 gpart[rank] = spart[0];
                 if (rank == 0) rnd->round = __ldcg(&rnd->round) + n_pub;   // written by rank 0 alone
+                if (s_owed) P.table[ls.pslot].c = ls.pc;
             } else {
                 set_status(st, kErrTimeout);
             }
         }
     }
-    if (!kGrid && tid == 0) gpart[rank] = spart[lastp];
+    if (!kGrid && tid == 0) {
+        gpart[rank] = spart[lastp];
+        if (s_owed) P.table[ls.pslot].c = ls.pc;     // (every CTA has passed the last iteration's barrier)
+    }
     if (tid == 0 && rank == 0) {      // lane 0 of the control warp holds the state
         CdRecord o;
         o.a = ls.pA; o.b = ls.pB; o.slot = ls.pslot;
