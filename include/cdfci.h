@@ -172,7 +172,9 @@ int cdfci_step(cdfci_handle h, int64_t n_iter, cdfci_stats *stats);
 /*
  * Energy of the current vector: mode 0 = alpha / mu (double-double ratio,
  * Alg. 1 last line); mode 1 = exact Rayleigh quotient sum_i c_i (Hc)_i / c.c
- * recomputed from the stored c with fresh columns (independent of b).
+ * recomputed from the stored c with fresh elements (independent of b; memory:
+ * see cdfci_rdm).  c = 0, the method's minimum where nothing of negative energy
+ * can be reached from the start, has no energy: NaN (0 / 0).
  */
 int cdfci_energy(cdfci_handle h, int mode, double *E);
 
@@ -419,8 +421,13 @@ int cdfci_last_step(cdfci_handle h, uint64_t *keys, double *eta, int64_t cap, in
  *   rdm2[((p*N+q)*N+r)*N+s]   = Gamma_pqrs = sum_st <a+_ps a+_rt a_st a_qs>
  * in chemists' order, so that E = sum h_pq gamma_pq + 1/2 sum (pq|rs) Gamma_pqrs.
  * rdm1 (N*N doubles) and rdm2 (N^4 doubles, or NULL) are host or device memory.
- * Cost: one pass over the stored determinants, each enumerating all its
- * single and double excitations with a table lookup per excitation.
+ * Cost: one pass over the determinants with c != 0, each enumerating the half
+ * of its single and double excitations that raise its key, with a lookup where
+ * a bit filter does not rule it out.  Memory during the call (cdfci_gradient,
+ * cdfci_energy mode 1 and cdfci_energy_with likewise): 64 to 150 bytes per
+ * determinant with c != 0 for a list of them with its filter; where the device
+ * has no room for it, or they are more than 2^31, the call works in the solver's
+ * table without it, with a lookup per excitation (several times slower).
  */
 int cdfci_rdm(cdfci_handle h, double *rdm1, double *rdm2);
 

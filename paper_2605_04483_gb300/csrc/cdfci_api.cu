@@ -911,39 +911,62 @@ CDFCI_API int cdfci_energy_with(cdfci_handle c, const double *h, const double *g
 }  // extern "C"
 
 namespace {
-// Room for the list of the determinants with c != 0, its filters, and `extra` doubles beside them
-// (one allocation, freed by the destructor).  The first guess at their number is the snapshot's
-// count, which a restored checkpoint may have stated wrongly: the callers look at the device's
-// count afterwards and, if it is larger, come back with that.
+// Room for the list of the determinants with c != 0, its filters, and `extra`
+// doubles beside them (one allocation, freed by the destructor).  The list is the
+// fast way and takes 64 to 150 bytes a determinant; where the device has no room
+// for it (a handle whose table fills the memory), or there are more than 2^31
+// determinants, the sums do without it (Q.rec = NULL) and need `extra` alone.
+// The first guess at the number is the snapshot's count, which a restored
+// checkpoint may have stated wrongly: without room for it the determinants are
+// counted; one that was too small shows in the device's count (again()).
 struct PairBuffers {
     void *mem = nullptr;
     PairList Q{};
     double *extra = nullptr;
     static constexpr long long kMost = 1ll << 31;      // positions are 32 bits, the table has twice as many records
-    bool at_most() const { return Q.cap >= kMost; }
     ~PairBuffers() { cudaFree(mem); }
-    int make(const Problem &P, long long est, size_t n_extra) {
+    int make(cdfci_ctx *c, const Problem &P, long long est, size_t n_extra) {
+        if (est <= kMost && room(P, est, n_extra)) return CDFCI_OK;
+        unsigned long long n = 0;
+        CK(launch_count_nonzero(P, c->d_counter, c->stream));
+        CK(cudaMemcpyAsync(&n, c->d_counter, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        if (n < (unsigned long long)est && n <= (unsigned long long)kMost && room(P, (long long)n, n_extra)) return CDFCI_OK;
+        return room(P, 0, n_extra) ? CDFCI_OK : fail(CDFCI_ERR_NOMEM, "device allocation failed");
+    }
+    // After a listing that counted n: whether there are more than it had room for.
+    bool again(unsigned long long n) const { return Q.rec && n > Q.cap; }
+
+private:
+    // Memory for a list of est determinants (0: no list) and the extra doubles; false when it cannot be had.
+    bool room(const Problem &P, long long est, size_t n_extra) {
         cudaFree(mem);
         mem = nullptr;
-        est = std::max<long long>(1, std::min<long long>(est, std::min<long long>(P.capacity, kMost)));
+        const bool listed = est > 0;
+        est = std::max<long long>(1, std::min<long long>(listed ? est : kMost, P.capacity));
         pair_sizes(P, est, &Q);
+        if (!listed) Q.nb1 = 0;
         size_t at = 0;
         auto part = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
-        const size_t orec = part(((size_t)Q.imask + 1) * sizeof(PairRec)), op = part((size_t)est * sizeof(unsigned));
-        const size_t o1 = part(Q.nb1 / 8), o2 = part(((size_t)Q.mask2 + 1) / 8), on = part(sizeof(unsigned));
+        size_t orec = 0, op = 0, o1 = 0, o2 = 0, on = 0;
+        if (listed) {
+            orec = part(((size_t)Q.imask + 1) * sizeof(PairRec)); op = part((size_t)est * sizeof(unsigned));
+            o1 = part(Q.nb1 / 8); o2 = part(((size_t)Q.mask2 + 1) / 8); on = part(sizeof(*Q.n));
+        }
         const size_t ox = part(n_extra * sizeof(double));
         if (cudaMalloc(&mem, at) != cudaSuccess) {
+            cudaGetLastError();
             mem = nullptr;
-            return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+            return false;
         }
         unsigned char *m = static_cast<unsigned char *>(mem);
-        Q.rec = reinterpret_cast<PairRec *>(m + orec);
+        Q.rec = listed ? reinterpret_cast<PairRec *>(m + orec) : nullptr;
         Q.pos = reinterpret_cast<unsigned *>(m + op);
         Q.f1 = reinterpret_cast<unsigned *>(m + o1);
         Q.f2 = reinterpret_cast<unsigned *>(m + o2);
-        Q.n = reinterpret_cast<unsigned *>(m + on);
+        Q.n = reinterpret_cast<unsigned long long *>(m + on);
         extra = reinterpret_cast<double *>(m + ox);
-        return CDFCI_OK;
+        return true;
     }
 };
 
@@ -951,18 +974,16 @@ struct PairBuffers {
 int exact_rq(cdfci_ctx *c, const Problem &P, double *E) {
     PairBuffers pb;
     const size_t np = 2 * rq_partials(P);
-    unsigned n = (unsigned)std::max<long long>(c->h_st->nnz_c, 1);
+    unsigned long long n = (unsigned long long)std::max<long long>(c->h_st->nnz_c, 1);
     do {
-        const int rc = pb.make(P, n, np + 1);
+        const int rc = pb.make(c, P, (long long)n, np + 1);
         if (rc) return rc;
         cudaError_t e = launch_rq(P, c->d_st, pb.Q, pb.extra, pb.extra + np, c->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(E, pb.extra + np, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && pb.Q.rec) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "energy: %s", cudaGetErrorString(e));
-        if (n > pb.Q.cap && pb.at_most())
-            return fail(CDFCI_ERR_NOMEM, "more than 2^31 determinants with c != 0");
-    } while (n > pb.Q.cap);
+    } while (pb.again(n));
     return fill_stats(c, nullptr);
 }
 }  // namespace
@@ -1625,20 +1646,18 @@ namespace {
 int rdm_device(cdfci_ctx *c, double *g1, double *g2) {
     const size_t n2 = (size_t)c->P.N * c->P.N, n4 = n2 * n2;
     PairBuffers pb;
-    unsigned n = (unsigned)std::max<long long>(c->h_st->nnz_c, 1);
+    unsigned long long n = (unsigned long long)std::max<long long>(c->h_st->nnz_c, 1);
     double norm = 0.0;
     do {
-        const int rc = pb.make(c->P, n, n2 + n4 + 1);
+        const int rc = pb.make(c, c->P, (long long)n, n2 + n4 + 1);
         if (rc) return rc;
         double *raw1 = pb.extra, *raw2 = raw1 + n2, *nrm = raw2 + n4;
         cudaError_t e = launch_rdm(c->P, c->d_st, pb.Q, raw1, raw2, nrm, g1, g2, c->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&norm, nrm, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && pb.Q.rec) e = cudaMemcpyAsync(&n, pb.Q.n, sizeof(n), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "rdm: %s", cudaGetErrorString(e));
-        if (n > pb.Q.cap && pb.at_most())
-            return fail(CDFCI_ERR_NOMEM, "more than 2^31 determinants with c != 0");
-    } while (n > pb.Q.cap);
+    } while (pb.again(n));
     if (!(norm > 0.0)) return fail(CDFCI_ERR_ARG, "rdm: the stored vector is zero");
     return CDFCI_OK;
 }

@@ -144,7 +144,8 @@ cudaError_t launch_cd_finalize_batch(const CdInstance *inst, int n_inst, int clu
 // The determinants with c != 0: a table of records (at most half full), the
 // positions of the occupied ones (in no particular order) and bit filters;
 // `est` is their expected number, `cap` the most that are taken (n > cap after
-// the listing: list again with room for n).
+// the listing: list again with room for n).  rec = NULL: no list, the sums walk
+// the solver's table and look every excitation up there (`est` at least 1).
 struct __align__(32) PairRec {
     unsigned long long a, b;
     double c;
@@ -153,12 +154,14 @@ struct __align__(32) PairRec {
 struct PairList {
     PairRec *rec;                      // imask + 1 records
     unsigned *pos;
-    unsigned *n, cap, est;
+    unsigned long long *n;
+    unsigned cap, est;
     unsigned imask;
     unsigned *f1, nb1;                 // filter 1: nb1 bits (0: not used)
     unsigned *f2, mask2;               // filter 2: mask2 + 1 bits (where filter 1 is not used)
 };
 void pair_sizes(const Problem &P, long long est, PairList *Q);   // everything but the pointers
+cudaError_t launch_count_nonzero(const Problem &P, unsigned long long *n, cudaStream_t s);
 size_t rq_partials(const Problem &P);   // pairs of doubles that launch_rq needs
 cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, double *g1_raw, double *g2_raw,
                        double *norm, double *g1, double *g2, cudaStream_t s);

@@ -87,11 +87,11 @@ __global__ void __launch_bounds__(256) k_pair_list(Problem P, IterState *st, Pai
         const bool on = (a | b) != 0ull && !is_zero(c);
         const unsigned m = __ballot_sync(0xffffffffu, on);
         if (!m) continue;
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(L.n, (unsigned)__popc(m));
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(L.n, (unsigned long long)__popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (!on) continue;
-        const unsigned pos = base + __popc(m & ((1u << lane) - 1u));
+        const unsigned long long pos = base + (unsigned)__popc(m & ((1u << lane) - 1u));
         if (pos >= L.cap) continue;                     // the caller sees n > cap and lists again
         unsigned long long z = 0ull;
         for (unsigned long long x = a; x; x &= x - 1) z ^= s_z[__ffsll((long long)x) - 1];
@@ -116,6 +116,45 @@ __global__ void __launch_bounds__(256) k_pair_list(Problem P, IterState *st, Pai
             L.pos[pos] = at;
         }
         if (probe > L.imask) set_status(st, kErrInternal);
+    }
+}
+
+// The number of determinants with c != 0.
+__global__ void __launch_bounds__(256) k_count_nonzero(Problem P, unsigned long long *n) {
+    unsigned long long mine = 0ull;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P.capacity; i += (long long)gridDim.x * blockDim.x) {
+        unsigned long long a, b;
+        double c;
+        ld_slot_cg(P.table + i, a, b, c);
+        mine += ((a | b) != 0ull && !is_zero(c)) ? 1 : 0;
+    }
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(n, mine);
+}
+
+// visit(A, B, c) for every determinant with c != 0 of this warp's share: of the list, or where there is none
+// of the solver's table (32 slots a load).  The whole warp calls it together.
+template <bool kListed, class Visit>
+__device__ __forceinline__ void for_each_nonzero(const Problem &P, const PairList &Q, const Visit &visit) {
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const unsigned w0 = blockIdx.x * nwarps + (threadIdx.x >> 5), step = gridDim.x * nwarps;
+    if (kListed) {
+        const unsigned n = (unsigned)(*Q.n < Q.cap ? *Q.n : Q.cap);
+        for (unsigned at = w0; at < n; at += step) {
+            const PairRec J = Q.rec[Q.pos[at]];
+            visit(J.a, J.b, J.c);
+        }
+        return;
+    }
+    for (long long s0 = 32ll * w0; s0 < P.capacity; s0 += 32ll * step) {
+        unsigned long long a = 0ull, b = 0ull;
+        double c = 0.0;
+        if (s0 + lane < P.capacity) ld_slot_cg(P.table + s0 + lane, a, b, c);
+        b &= kKeyMaskB;
+        for (unsigned m = __ballot_sync(0xffffffffu, (a | b) != 0ull && !is_zero(c)); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            visit(__shfl_sync(0xffffffffu, a, src), __shfl_sync(0xffffffffu, b, src), __shfl_sync(0xffffffffu, c, src));
+        }
     }
 }
 
@@ -208,10 +247,14 @@ __host__ __device__ __forceinline__ size_t pair_warp_bytes(int nsA, int nsB) {
 // per lane times kPairU alpha singles; same-spin doubles: one virtual pair per
 // lane times kPairU occupied pairs; singles: one per lane); the ones whose bit
 // is set join the warp's queue as (kind, x, y), and the queue is looked up 32 at
-// a time, every lane its own element.  kF1: filter 1 (shared memory) is tested
-// in the loop and filter 2 (L2) in the lookup; else filter 2 in the loop.
-template <class Sink, bool kF1>
-__global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink sink, int singles_only) {
+// a time, every lane its own element.
+// How an element is found: by filter 1 (shared memory) in the loop, then the
+// list's table; by filter 2 (L2) in the loop, then that table; or, where there is
+// no room for a list, without a filter in the solver's table.
+enum { kFindF1, kFindF2, kFindSlots };
+template <class Sink, int kFind>
+__global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, IterState *st, PairList Q, Sink sink, int singles_only) {
+    constexpr bool kF1 = kFind == kFindF1;
     extern __shared__ __align__(16) unsigned char s_raw[];
     unsigned *s_f = reinterpret_cast<unsigned *>(s_raw);
     const unsigned nw1 = kF1 ? Q.nb1 / 32 : 0;
@@ -225,20 +268,17 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink s
     for (unsigned t = threadIdx.x; t < nw1; t += blockDim.x) s_f[t] = Q.f1[t];
     if (threadIdx.x < 128) s_z[threadIdx.x] = orb_word(threadIdx.x);
     __syncthreads();
-    const unsigned n = min(*Q.n, Q.cap);
     const int N = P.N;
     auto half = [](unsigned long long z) { return kF1 ? (unsigned)z : (unsigned)(z >> 32); };
     auto zA = [&](int p) { return half(s_z[p]); };
     auto zB = [&](int p) { return half(s_z[64 + p]); };
     auto maybe = [&](unsigned h) {                      // the filter bit of an element
+        if (kFind == kFindSlots) return true;
         const unsigned k = kF1 ? __umulhi(h, Q.nb1) : (h & Q.mask2);
         const unsigned w = kF1 ? s_f[k >> 5] : __ldg(Q.f2 + (k >> 5));
         return ((w >> (k & 31)) & 1u) != 0u;
     };
-    for (unsigned at = blockIdx.x * nwarps + warp; at < n; at += gridDim.x * nwarps) {
-        const PairRec J = Q.rec[Q.pos[at]];
-        const unsigned long long A = J.a, B = J.b;
-        const double cJ = J.c;
+    for_each_nonzero<kFind != kFindSlots>(P, Q, [&](unsigned long long A, unsigned long long B, double cJ) {
         unsigned long long zJ = 0ull;
         for (int t = lane; t < N; t += 32) {
             const int ra = __popcll(A & low_mask(t)), rb = __popcll(B & low_mask(t));
@@ -383,15 +423,21 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink s
                             if (x.kind == 1) { x.i = j; x.a = b; } else { x.j = j; x.b = b; }
                         }
                     }
-                    unsigned pos = (unsigned)(z >> 32) & Q.imask;
                     double cI = 0.0;
-                    for (unsigned probe = 0; probe <= Q.imask; ++probe) {
-                        unsigned long long ka, kb;
-                        double c;
-                        ld_rec(Q.rec + pos, ka, kb, c);
-                        if (ka == oa && kb == ob) { cI = c; break; }
-                        if ((ka | kb) == 0ull) break;
-                        pos = (pos + 1) & Q.imask;
+                    if (kFind == kFindSlots) {
+                        bool ins = false;
+                        const long long at = table_find(P, st, oa, ob, false, &ins);
+                        if (at >= 0) cI = __ldcg(&P.table[at].c);
+                    } else {
+                        unsigned pos = (unsigned)(z >> 32) & Q.imask;
+                        for (unsigned probe = 0; probe <= Q.imask; ++probe) {
+                            unsigned long long ka, kb;
+                            double c;
+                            ld_rec(Q.rec + pos, ka, kb, c);
+                            if (ka == oa && kb == ob) { cI = c; break; }
+                            if ((ka | kb) == 0ull) break;
+                            pos = (pos + 1) & Q.imask;
+                        }
                     }
                     if (!is_zero(cI)) sink.hit(P, L, x, cJ, cI);
                 }
@@ -400,7 +446,7 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink s
             if (type == 4) break;
         }
         __syncwarp();
-    }
+    });
     sink.finish((int)(blockIdx.x * nwarps + warp), lane);
 }
 
@@ -412,6 +458,7 @@ __global__ void __launch_bounds__(1024, 1) k_pairs(Problem P, PairList Q, Sink s
 // pairs that are occupied (testing every pair of spin-orbitals in registers took
 // 540 us for 300 k determinants of 10 electrons in 32 spin-orbitals).
 __host__ __device__ __forceinline__ size_t diag_warp_bytes(int N) { return ((size_t)N * (2 * N + 1) + 16) * sizeof(double); }
+template <bool kListed>
 __global__ void __launch_bounds__(256) k_rdm_diag(Problem P, PairList Q, double *g1, double *g2, double *norm) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int N = P.N, NS = 2 * N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -428,14 +475,12 @@ __global__ void __launch_bounds__(256) k_rdm_diag(Problem P, PairList Q, double 
     for (int t = lane; t < npairs; t += 32) s[t] = 0.0;
     __syncthreads();
     double nrm = 0.0;
-    const unsigned n = min(*Q.n, Q.cap);
-    for (unsigned at = blockIdx.x * nwarps + warp; at < n; at += gridDim.x * nwarps) {
-        const PairRec key = Q.rec[Q.pos[at]];
-        const double c2 = key.c * key.c;
+    for_each_nonzero<kListed>(P, Q, [&](unsigned long long A, unsigned long long B, double cJ) {
+        const double c2 = cJ * cJ;
         nrm += c2;
         for (int t = lane; t < N; t += 32) {
-            if ((key.a >> t) & 1ull) occ[__popcll(key.a & low_mask(t))] = (unsigned char)t;
-            if ((key.b >> t) & 1ull) occ[P.na + __popcll(key.b & low_mask(t))] = (unsigned char)(N + t);
+            if ((A >> t) & 1ull) occ[__popcll(A & low_mask(t))] = (unsigned char)t;
+            if ((B >> t) & 1ull) occ[P.na + __popcll(B & low_mask(t))] = (unsigned char)(N + t);
         }
         __syncwarp();
         for (int t = lane; t < nep; t += 32) {
@@ -443,7 +488,7 @@ __global__ void __launch_bounds__(256) k_rdm_diag(Problem P, PairList Q, double 
             s[q * (q + 1) / 2 + p] += c2;
         }
         __syncwarp();
-    }
+    });
     if (lane == 0 && nrm != 0.0) atomicAdd(norm, nrm);
     // the block's sums, each pair once
     __syncthreads();
@@ -595,8 +640,16 @@ void pair_sizes(const Problem &P, long long est, PairList *Q) {
     Q->cap = Q->est = (unsigned)est;
 }
 
+cudaError_t launch_count_nonzero(const Problem &P, unsigned long long *n, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(n, 0, sizeof(*n), s);
+    if (e != cudaSuccess) return e;
+    k_count_nonzero<<<(unsigned)std::min<long long>((P.capacity + 255) / 256, 152 * 8), 256, 0, s>>>(P, n);
+    return cudaGetLastError();
+}
+
 static cudaError_t launch_pair_list(const Problem &P, IterState *st, const PairList &Q, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(Q.n, 0, sizeof(unsigned), s);
+    if (!Q.rec) return cudaSuccess;                     // no list
+    cudaError_t e = cudaMemsetAsync(Q.n, 0, sizeof(*Q.n), s);
     if (e == cudaSuccess && Q.nb1) e = cudaMemsetAsync(Q.f1, 0, Q.nb1 / 8, s);
     if (e == cudaSuccess && !Q.nb1) e = cudaMemsetAsync(Q.f2, 0, ((size_t)Q.mask2 + 1) / 8, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(Q.rec, 0, ((size_t)Q.imask + 1) * sizeof(PairRec), s);
@@ -608,13 +661,13 @@ static cudaError_t launch_pair_list(const Problem &P, IterState *st, const PairL
 }
 
 template <class Sink>
-static cudaError_t launch_pairs(const Problem &P, const PairList &Q, const Sink &sink, int singles_only,
+static cudaError_t launch_pairs(const Problem &P, IterState *st, const PairList &Q, const Sink &sink, int singles_only,
                                 cudaStream_t s) {
     const PairShape g = pair_shape(P, Q);
-    auto kernel = Q.nb1 ? k_pairs<Sink, true> : k_pairs<Sink, false>;
+    auto kernel = !Q.rec ? k_pairs<Sink, kFindSlots> : (Q.nb1 ? k_pairs<Sink, kFindF1> : k_pairs<Sink, kFindF2>);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
     if (e != cudaSuccess) return e;
-    kernel<<<g.blocks, 32 * g.warps, g.smem, s>>>(P, Q, sink, singles_only);
+    kernel<<<g.blocks, 32 * g.warps, g.smem, s>>>(P, st, Q, sink, singles_only);
     return cudaGetLastError();
 }
 
@@ -626,15 +679,16 @@ cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, doubl
     if (e == cudaSuccess) e = cudaMemsetAsync(g2_raw, 0, n4 * sizeof(double), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(norm, 0, sizeof(double), s);
     if (e == cudaSuccess) e = launch_pair_list(P, st, Q, s);
-    if (e == cudaSuccess) e = launch_pairs(P, Q, RdmSink{g1_raw, g2_raw}, 0, s);
+    if (e == cudaSuccess) e = launch_pairs(P, st, Q, RdmSink{g1_raw, g2_raw}, 0, s);
     if (e != cudaSuccess) return e;
     int dw = 8;                                         // warps a block: their arrays within 100 KB (200 KB for one)
     while (dw > 1 && dw * diag_warp_bytes(N) > 100 * 1024) --dw;
     const size_t dsm = dw * diag_warp_bytes(N) + (size_t)(P.na + P.nb) * (P.na + P.nb + 1);
-    e = cudaFuncSetAttribute(k_rdm_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    auto diag = Q.rec ? k_rdm_diag<true> : k_rdm_diag<false>;
+    e = cudaFuncSetAttribute(diag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     const long long dblocks = std::max<long long>(1, std::min<long long>(152 * 2, ((long long)Q.est + 8 * dw - 1) / (8 * dw)));
-    k_rdm_diag<<<(unsigned)dblocks, 32 * dw, dsm, s>>>(P, Q, g1_raw, g2_raw, norm);
+    diag<<<(unsigned)dblocks, 32 * dw, dsm, s>>>(P, Q, g1_raw, g2_raw, norm);
     k_rdm_finalize<<<152 * 4, 256, 0, s>>>(N, g1_raw, g2_raw, norm, g1, g2);
     return cudaGetLastError();
 }
@@ -643,7 +697,7 @@ size_t rq_partials(const Problem &P) { return 152 * (size_t)pair_warps(P); }
 
 cudaError_t launch_rq(const Problem &P, IterState *st, const PairList &Q, double *partial, double *out, cudaStream_t s) {
     cudaError_t e = launch_pair_list(P, st, Q, s);
-    if (e == cudaSuccess) e = launch_pairs(P, Q, QuotientSink{partial, 0.0, 0.0}, P.doubles_vanish, s);
+    if (e == cudaSuccess) e = launch_pairs(P, st, Q, QuotientSink{partial, 0.0, 0.0}, P.doubles_vanish, s);
     if (e != cudaSuccess) return e;
     const PairShape g = pair_shape(P, Q);
     k_rq_final<<<1, 1024, 0, s>>>(partial, g.blocks * g.warps, out);
