@@ -287,8 +287,12 @@ __device__ void x_step(const Problem &P, XState *xs, IterState *st, double *rows
     bool stop = false;
     if (forced < 0) {
         if (!(gn > 0.0)) {
+            // a zero gradient ends the run; gn is NaN where g.g is, or has overflowed (inf times 1 / inf)
             stop = true;
-            if (lane == 0) xs->done = 1;
+            if (lane == 0) {
+                if (gg == 0.0) xs->done = 1;
+                else set_status(st, kErrNonfinite);
+            }
         } else {
             const double v2 = 2.0 * Hii + part + 2.0 * cc + us;
             eta = line_search_lanes((float)gn, (float)v2, (float)v3, gn, v2, v3) * ign;
