@@ -113,6 +113,7 @@ struct McBuffers {
     float *Rh, *Rl;                // reduced matrix R as float-float pairs, leading dimension ldr
     int ldr;
     int m, cand_grid, scatter_grid;
+    int batch_cand_grid, batch_scatter_grid;   // beside the other problems of a batch
     long long cap_cand;            // entries of cand / gkey / ties
 };
 size_t mc_eigen_smem(int m);
