@@ -254,11 +254,14 @@ static __device__ __noinline__ bool column_meets(int doubles_vanish, const unsig
 // Finish the lookup of an issued element: compare the loaded slot, then probe
 // on, kProbeAhead slots a load: the warp waits for its slowest lane, and a
 // dependent probe is an L2 round trip (700 cycles and more), of which every
-// warp paid for two or three even in a nearly empty table.  (One copy of the
-// comparison: the loop's code is as long as the instruction cache.)
+// warp paid for two or three even in a nearly empty table.  Two slots a load
+// where a thread has one element; one where it has kCdMaxE, whose registers have
+// no room for more (with two: N = 32, 8 + 8 electrons 18.1 -> 19.0 us an
+// iteration, a batch of 96 problems 6.63e9 -> 6.05e9 elements/s).  (One copy of
+// the comparison: the loop's code is as long as the instruction cache.)
 // Sets state 1 (found: c, b), 2 (absent at pos) or 0 (value zero or error,
 // *err set).
-constexpr int kProbeAhead = 2;
+template <int kProbeAhead>
 __device__ __forceinline__ void resolve_elem(const Problem &P, IterState *st, Elem &x, int *err) {
     if (x.state != 4) return;
     if (is_zero(x.H)) { x.state = 0; return; }
@@ -807,12 +810,14 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
             const unsigned long long tau_bits = abs_bits(P.tau);
             double eta = 0.0, mu = 0.0, pb = 0.0, pc = 0.0;
             long long pslot = -1;
-            // rounds of kE elements a thread (kE = 1: one round covers the column).  One copy of the code for
-            // every round, the step size awaited in the first: the loop's code does not fit the
-            // instruction cache.
-            bool first = true;
-            for (long long eb = e0;;) {
-                Elem el[kE];
+            // Rounds of kE elements a thread (kE = 1: one round covers the column), the step size awaited in
+            // the first.  One copy of the code for every round where it is best, as the loop's code does not
+            // fit the instruction cache; two for the grid's rounds of kCdMaxE, whose elements are generated
+            // with fewer live registers then (one copy spills 300 bytes; N = 26, 7 + 7 electrons, 64 CTAs:
+            // 13.1 -> 12.0 us an iteration, but 8 CTAs in a cluster 22.1 -> 23.6).
+            constexpr bool kTwoCopies = kGrid && kE > 1;
+            Elem el[kE];
+            auto generate = [&](long long eb, bool first) {
 #pragma unroll
                 for (int k = 0; k < kE; ++k)
                     issue_elem(P, L, tabA, tabB, iA, iB, hAc, hBc, eb + k * stride, nh, have_prev, pA, pB, el[k]);
@@ -843,19 +848,30 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                             el[k].H = single_sum(sTerm + ls * (nocc + 1), nocc, el[k].ix.sgn);
                         }
                 }
+            };
+            auto await_step = [&]() {
+                cta_sync();
+                eta = sel.eta;
+                mu = sel.mu_g;
+                pslot = sel.pslot;
+                pb = sel.pb;
+                pc = sel.pc;
+            };
+            if (kTwoCopies) {
+                generate(e0, true);
+                await_step();
+            }
+            bool first = true;
+            for (long long eb = e0;;) {
+                if (!kTwoCopies) generate(eb, first);
                 if (first) {
-                    cta_sync();
-                    eta = sel.eta;
-                    mu = sel.mu_g;
-                    pslot = sel.pslot;
-                    pb = sel.pb;
-                    pc = sel.pc;
+                    if (!kTwoCopies) await_step();
                     first = false;
                     if (sel.bad) break;
                 }
                 // ---- apply: b_j += eta H_ji with compression, gather, candidates ----
 #pragma unroll
-                for (int k = 0; k < kE; ++k) resolve_elem(P, st, el[k], &err);
+                for (int k = 0; k < kE; ++k) resolve_elem<kE == 1 ? 2 : 1>(P, st, el[k], &err);
 #pragma unroll
                 for (int k = 0; k < kE; ++k) {
                     Elem &x = el[k];
@@ -904,6 +920,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
                 }
                 eb += kE * stride;
                 if (kE == 1 || eb >= nh) break;
+                if (kTwoCopies) generate(eb, false);
             }
             // ---- the warp's partial ----
             warp_combine(best, bbest, cbest, gather, cnt, err);
