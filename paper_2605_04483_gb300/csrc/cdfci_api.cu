@@ -930,8 +930,13 @@ struct PairBuffers {
     PairList Q{};
     double *extra = nullptr;
     static constexpr long long kMost = 1ll << 31;      // positions are 32 bits, the table has twice as many records
+    // A few determinants with short columns in a small table: a list is a launch more than it saves.  (RDMs of
+    // 78 determinants with columns of 316 elements 99 us with a list, 85 without; 3 with columns of 1,425:
+    // 103, 97; 2 with columns of 3,690: 113, 123, as every lookup goes to the table.)
+    static constexpr long long kFew = 128, kFewElements = 1024, kFewSlots = 1 << 16;
     ~PairBuffers() { cudaFree(mem); }
     int make(cdfci_ctx *c, const Problem &P, long long est, size_t n_extra) {
+        if (est <= kFew && P.nh <= kFewElements && P.capacity <= kFewSlots && room(P, 0, n_extra)) return CDFCI_OK;
         if (est <= kMost && room(P, est, n_extra)) return CDFCI_OK;
         unsigned long long n = 0;
         CK(launch_count_nonzero(P, c->d_counter, c->stream));
@@ -956,7 +961,8 @@ private:
         auto part = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
         size_t orec = 0, op = 0, o1 = 0, o2 = 0, on = 0;
         if (listed) {
-            orec = part(((size_t)Q.imask + 1) * sizeof(PairRec)); op = part((size_t)est * sizeof(unsigned));
+            op = part((size_t)est * sizeof(unsigned));
+            orec = part(((size_t)Q.imask + 1) * sizeof(PairRec));
             o1 = part(Q.nb1 / 8); o2 = part(((size_t)Q.mask2 + 1) / 8); on = part(sizeof(*Q.n));
         }
         const size_t ox = part(n_extra * sizeof(double));
@@ -971,6 +977,8 @@ private:
         Q.f1 = reinterpret_cast<unsigned *>(m + o1);
         Q.f2 = reinterpret_cast<unsigned *>(m + o2);
         Q.n = reinterpret_cast<unsigned long long *>(m + on);
+        Q.zero = m + orec;
+        Q.zero_end = m + ox;
         extra = reinterpret_cast<double *>(m + ox);
         return true;
     }
@@ -1675,17 +1683,18 @@ CDFCI_API int cdfci_rdm(cdfci_handle c, double *rdm1, double *rdm2) {
     int rc = fill_stats(c, nullptr);
     if (rc) return rc;
     const size_t n2 = (size_t)c->P.N * c->P.N, n4 = n2 * n2;
-    double *g1 = nullptr, *g2 = nullptr;
-    if (cudaMalloc(&g1, n2 * sizeof(double)) != cudaSuccess || cudaMalloc(&g2, n4 * sizeof(double)) != cudaSuccess) {
-        cudaFree(g1); cudaFree(g2);
+    double *g1 = nullptr;
+    if (cudaMalloc(&g1, (n2 + n4) * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
         return fail(CDFCI_ERR_NOMEM, "device allocation failed");
     }
+    double *g2 = g1 + n2;
     rc = rdm_device(c, g1, g2);
     cudaError_t e = cudaSuccess;
     if (!rc) e = cudaMemcpyAsync(rdm1, g1, n2 * sizeof(double), cudaMemcpyDefault, c->stream);
     if (!rc && e == cudaSuccess && rdm2) e = cudaMemcpyAsync(rdm2, g2, n4 * sizeof(double), cudaMemcpyDefault, c->stream);
     if (!rc && e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(g1); cudaFree(g2);
+    cudaFree(g1);
     if (rc) return rc;
     if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "rdm copy: %s", cudaGetErrorString(e));
     return CDFCI_OK;
@@ -1698,20 +1707,21 @@ CDFCI_API int cdfci_gradient(cdfci_handle c, double *dE_dh, double *dE_dg, doubl
     if (rc) return rc;
     const int N = c->P.N;
     const size_t n2 = (size_t)N * N, n4 = n2 * n2;
-    double *g1 = nullptr, *g2 = nullptr, *F = nullptr, *oh = nullptr, *og = nullptr, *ok = nullptr;
-    bool okm = cudaMalloc(&g1, n2 * sizeof(double)) == cudaSuccess && cudaMalloc(&g2, n4 * sizeof(double)) == cudaSuccess &&
-               cudaMalloc(&F, n2 * sizeof(double)) == cudaSuccess && cudaMalloc(&oh, n2 * sizeof(double)) == cudaSuccess &&
-               cudaMalloc(&og, n4 * sizeof(double)) == cudaSuccess && cudaMalloc(&ok, n2 * sizeof(double)) == cudaSuccess;
+    double *g1 = nullptr;
+    if (cudaMalloc(&g1, (4 * n2 + 2 * n4) * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(CDFCI_ERR_NOMEM, "device allocation failed");
+    }
+    double *F = g1 + n2, *oh = F + n2, *ok = oh + n2, *g2 = ok + n2, *og = g2 + n4;
     cudaError_t e = cudaSuccess;
-    if (!okm) rc = fail(CDFCI_ERR_NOMEM, "device allocation failed");
-    if (!rc) rc = rdm_device(c, g1, g2);
+    rc = rdm_device(c, g1, g2);
     if (!rc) e = launch_gradient(N, c->d_h, c->d_g, g1, g2, F, dE_dh ? oh : nullptr, dE_dg ? og : nullptr,
                                  dE_dkappa ? ok : nullptr, c->stream);
     if (!rc && e == cudaSuccess && dE_dh) e = cudaMemcpyAsync(dE_dh, oh, n2 * sizeof(double), cudaMemcpyDefault, c->stream);
     if (!rc && e == cudaSuccess && dE_dg) e = cudaMemcpyAsync(dE_dg, og, n4 * sizeof(double), cudaMemcpyDefault, c->stream);
     if (!rc && e == cudaSuccess && dE_dkappa) e = cudaMemcpyAsync(dE_dkappa, ok, n2 * sizeof(double), cudaMemcpyDefault, c->stream);
     if (!rc && e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(g1); cudaFree(g2); cudaFree(F); cudaFree(oh); cudaFree(og); cudaFree(ok);
+    cudaFree(g1);
     if (rc) return rc;
     if (e != cudaSuccess) return fail(CDFCI_ERR_CUDA, "gradient: %s", cudaGetErrorString(e));
     return CDFCI_OK;

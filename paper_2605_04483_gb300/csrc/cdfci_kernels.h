@@ -160,10 +160,13 @@ struct PairList {
     unsigned imask;
     unsigned *f1, nb1;                 // filter 1: nb1 bits (0: not used)
     unsigned *f2, mask2;               // filter 2: mask2 + 1 bits (where filter 1 is not used)
+    unsigned char *zero;               // rec, the filter and n lie in [zero, zero_end), cleared together
+    unsigned char *zero_end;           // (without a list zero = zero_end)
 };
 void pair_sizes(const Problem &P, long long est, PairList *Q);   // everything but the pointers
 cudaError_t launch_count_nonzero(const Problem &P, unsigned long long *n, cudaStream_t s);
 size_t rq_partials(const Problem &P);   // pairs of doubles that launch_rq needs
+// (the sums' scratch: g1_raw, g2_raw and norm one after the other from Q.zero_end on)
 cudaError_t launch_rdm(const Problem &P, IterState *st, const PairList &Q, double *g1_raw, double *g2_raw,
                        double *norm, double *g1, double *g2, cudaStream_t s);
 // c^T H c / c^T c with H from P's integrals
