@@ -232,10 +232,12 @@ int cdfci_energies(cdfci_handle h, double *E, int32_t cap, int32_t *n_out);
  * like cdfci_step) launch by launch instead of as a graph, with a CUDA event
  * recorded before every launch on the handle's stream, and writes into ms the
  * milliseconds spent from each launch to the next, summed over the
- * iterations, in launch order: 0 choice keys + level-0 histogram, 1 level-1
- * histogram and the levels below it, 2 collect, 3 exact ties and the sort of
- * the chosen set, 4 c_I / b_I / H_II, 5 reduced problem, 6 scatter of the m
- * columns, 7 b_I recalculated.  *n_kernels = 8 (host pointer); ms holds up to
+ * iterations, in launch order: 0 choice keys + their histogram around the last
+ * threshold, 1 radix passes where that does not resolve the choice, 2 the
+ * chosen set collected (exact ties included) and put in order, 3 nothing (two
+ * events in a row, about zero: part of 2 since they are one launch), 4 c_I / b_I /
+ * H_II, 5 reduced problem, 6 scatter of the m columns with the update of mu and
+ * alpha, 7 b_I recalculated.  *n_kernels = 8 (host pointer); ms holds up to
  * cap values (host pointer).  CDFCI_ERR_CAPACITY if cap < 8,
  * CDFCI_ERR_UNIMPLEMENTED for other handles.
  */

@@ -17,16 +17,18 @@
 //      issue the 32-byte slot loads and evaluate the elements (the singles'
 //      O(n) sums spread over the CTA through a shared-memory term table);
 //   3. meanwhile the control warp computes H_ii (from shared-memory copies of
-//      diag(h), J and K) and one lane the step size eta (appendix);
+//      diag(h), J and K) and the step size eta (appendix), the whole warp both;
 //   4. every element thread applies b_j += eta H_ji with the compression rule
 //      (c_j != 0 or |eta H_ji| >= tau), inserting absent keys with a 16-byte
 //      CAS, and accumulates the gather sum_j H_ji c_j and its best candidate;
-//   5. the control warp combines the CTA's partial and writes it while two
-//      lanes of warp 1 update mu and alpha (double-double); cluster or grid
-//      barrier.
+//   5. the control warp combines the CTA's partial and writes it; cluster
+//      barrier, or the partial's publication.  mu and alpha (double-double) are
+//      updated by two lanes of warp 2 beside the next choice, with one CTA by two
+//      of the control warp beside step 4.
 // In an m = 1 column every j occurs once, so each b_j has a single writer:
 // plain loads and stores, no atomics.  The previous coordinate's slot is
-// written by the thread whose excitation equals it, with the recalculated b.
+// written by the thread whose excitation equals it, with the recalculated b (by
+// CTA 0 where a start vector's next entry has no such excitation).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -510,8 +512,8 @@ __device__ __forceinline__ void fold_partial(const CdPartial &x, bool first, Bes
 // gather, counters) into its own shared memory, and after the cluster barrier
 // warp 0 of every CTA reads all partials through distributed shared memory and
 // reduces them in a fixed order, so every CTA makes the same choice.  The
-// serial steps (H_ii, eta, the double-double scalars) run on single lanes;
-// their results reach the other warps through shared memory.  Every exit
+// results of the serial steps (H_ii, eta, the double-double scalars) reach the
+// other warps through shared memory.  Every exit
 // decision uses data all CTAs read identically, so all CTAs reach every
 // cluster barrier.
 //
@@ -539,7 +541,7 @@ __device__ __forceinline__ void cd_loop_body(const Problem &P, IterState *st, Cd
     __shared__ int r_cnt[4][kCdWarps];
     __shared__ Sel sel;
     __shared__ int s_done;
-    __shared__ LoopState ls;                     // written by lane 0 of the control warp (warp 0) only
+    __shared__ LoopState ls;                     // written by lane 0 of the control warp (warp 0); mu, alpha: see books
     __shared__ int s_err;
     __shared__ int s_fins;                       // 1: this CTA inserted the forced coordinate of this step
     __shared__ int s_owed;                       // CTA 0: 1: the c of a forced step is not in the table yet
