@@ -159,6 +159,12 @@ __device__ __forceinline__ void ff_mac(float &sh, float &sl, float ah, float al,
     sl = __fadd_rn(sl, __fadd_rn(s.lo, e));
 }
 
+// Another CTA's shared memory may be written only once that CTA runs: every thread
+// of a cluster arrives when it starts and waits before the first such write.  (No
+// data is handed over: relaxed, without the fence of a whole barrier.)
+__device__ __forceinline__ void cluster_started_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_started_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
 // Block or cluster sums of K values held by the row leads (the other threads
 // hold zero): every warp reduces in a fixed tree, lane 0 of every warp writes
 // its K partials into slot (rank * warps + warp) of the scratch of every CTA
@@ -1321,6 +1327,7 @@ __device__ __forceinline__ void eigen_rows(const Problem &P, McState *ms, IterSt
     if (CL) {
         rank = cg::this_cluster().block_rank();
         C = cg::this_cluster().num_blocks();
+        cluster_started_arrive();
     }
     const int m = ms->m_sel, n1 = m + 1;
     // this CTA's rows of R (absolute indices [a0, a1)); one CTA: all
@@ -1444,6 +1451,7 @@ __device__ __forceinline__ void eigen_rows(const Problem &P, McState *ms, IterSt
     const bool late = in_smem && nown > 0 && !mbar_wait0(&s_bar, 1 << 22);
     bool any_late = __syncthreads_or(late);             // scalars, and this block's copy of R, complete
     if (CL) {
+        cluster_started_wait();
         if (tid == 0) {
             cg::cluster_group cl = cg::this_cluster();
             for (unsigned r = 0; r < C; ++r) cl.map_shared_rank(s_late, r)[rank] = any_late ? 1 : 0;
@@ -1959,6 +1967,7 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
     if (CL) {
         rank = cg::this_cluster().block_rank();
         C = cg::this_cluster().num_blocks();
+        cluster_started_arrive();
     }
     const int ns = (int)C * nw, slot = (int)rank * nw + warp;
     auto sync_all = [&]() { if (CL) cg::this_cluster().sync(); else __syncthreads(); };
@@ -2087,6 +2096,7 @@ __global__ void __launch_bounds__(kRegThreads) k_mc_eigen_reg(Problem P, McState
     const bool late = nown > 0 && !mbar_wait0(&s_bar, 1 << 22);
     bool any_late = __syncthreads_or(late);
     if (CL) {
+        cluster_started_wait();
         if (tid == 0) everywhere(s_late, [&](int *p) { p[rank] = any_late ? 1 : 0; });
         cg::this_cluster().sync();
         any_late = false;
